@@ -70,12 +70,6 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
            ((uint64_t)1 << 46);
 }
 
-// The same for an operand of K columns (stride byte offset K * 16).
-__device__ __forceinline__ uint64_t sdesc_k(uint32_t saddr, uint32_t k) {
-    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)((k * 16u) >> 4) << 32) |
-           ((uint64_t)1 << 46);
-}
-
 // Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both K-major,
 // N >> 3 at bit 17, M >> 4 at bit 24.
 __host__ __device__ constexpr uint32_t idesc(uint32_t m, uint32_t n) {
@@ -464,8 +458,8 @@ __global__ void __launch_bounds__(TC_ROWS) k_surrogate_tc(BatchArgs a) {
 
 
 // =======================================================================================
-// Training on the tensor cores.  A CTA of 128 threads takes minibatches of 128 rows of one
-// network; thread t owns row t of every activation and lane t of tensor memory.
+// Training on the tensor cores.  A CTA of 512 threads takes minibatches of 128 rows of one
+// network, one CTA per network.
 //   forward:   Z1 = G W1, H1 = relu(Z1 + b1); Z2 = H1 W2, H2 = relu(Z2 + b2); Y = H2 W3 + b3
 //   backward:  dY = s (Y - T); dZ2 = (dY W3^T) . [H2 > 0]; dZ1 = (dZ2 W2^T) . [H1 > 0]
 //   gradients: dW1 = G^T dZ1 and dW2 = H1^T dZ2 as one M = 128, N = 128 product
@@ -474,38 +468,52 @@ __global__ void __launch_bounds__(TC_ROWS) k_surrogate_tc(BatchArgs a) {
 // Every product takes BF16 operands from shared memory and accumulates in FP32 in tensor
 // memory; the batch-dimension products read transposed copies the epilogues write.  Then
 // FP32 Adam on the master weights.
+//
+// What bounds it: the steps of a network are a serial chain of six products with an epilogue
+// between any two, so a step is latency, not throughput, and a network has one SM.  The split
+// follows from that: warp w owns tensor-memory lanes 32 (w mod 4) .. + 31 (the rows a warp may
+// read) and 16 of the 64 columns (w / 4), so every epilogue, the features and Adam run in 16
+// warps instead of 4, a thread holding 16 columns of a row.  The same thread owns the 16
+// weights whose gradient the last product leaves in its tensor-memory lane: their FP32 masters
+// and Adam moments stay in its registers for all steps of a launch, and the gradient goes from
+// tensor memory to the update without a stage in shared memory.  The transposed operands' core
+// matrices are TR_LBO = 144 bytes apart instead of 128, so that the 32 lanes of a store to one
+// row fall into different banks (128: four-way conflicts).
+// Measured: 64 networks, 256 steps of 128 rows in 2.15 ms (8.4 us per step); 15.3 ms (60 us per
+// step) with 4 warps, unpadded transposed operands, and masters, moments and gradient in memory.
 // =======================================================================================
 constexpr uint32_t TR_COLS = 256;               // tensor-memory columns of the training kernel
+constexpr uint32_t TR_T = 512;                  // threads: 16 warps, four per 32 rows
+constexpr uint32_t TR_LBO = 144;                // padded distance of core matrices along K
+constexpr uint32_t TR_SBO_T = 16 * TR_LBO;      // 8-row groups of a [rows][128] operand
+constexpr uint32_t TR_SBO_W = 8 * TR_LBO;       // 8-row groups of a [rows][64] operand
+constexpr uint32_t TR_REST = 323;               // parameters outside W1 and W2
 
 struct St {                                     // byte offsets into dynamic shared memory
     static constexpr uint32_t a0 = 0;           // [128][64] features, then H2 (A of layers 1, 3)
     static constexpr uint32_t a1 = 16384;       // [128][64] H1 (A of layer 2)
     static constexpr uint32_t dz2 = 32768;      // [128][64] dZ2 (A of dH1 = dZ2 W2^T)
     static constexpr uint32_t dy = 49152;       // [128][16] dY, columns >= 3 zero (A of dH2)
-    static constexpr uint32_t gT = 53248;       // [64][128] G^T   \ gT, h1T: one 128-row operand
-    static constexpr uint32_t h1T = 69632;      // [64][128] H1^T  / h1T, h2T: another
-    static constexpr uint32_t h2T = 86016;      // [64][128] H2^T
-    static constexpr uint32_t dz1T = 102400;    // [64][128] dZ1^T \ one 128-row operand
-    static constexpr uint32_t dz2T = 118784;    // [64][128] dZ2^T /
-    static constexpr uint32_t dyT = 135168;     // [16][128] dY^T, rows >= 3 zero
-    static constexpr uint32_t w1t = 139264;     // [64][64] W1^T (B of layer 1)
-    static constexpr uint32_t w2t = 147456;     // [64][64] W2^T (B of layer 2)
-    static constexpr uint32_t w3t = 155648;     // [16][64] W3^T, rows >= 3 zero (B of layer 3)
-    static constexpr uint32_t w2n = 157696;     // [64][64] W2 (B of dH1)
-    static constexpr uint32_t w3n = 165888;     // [64][16] W3, columns >= 3 zero (B of dH2)
-    static constexpr uint32_t bias = 167936;    // b1[64], b2[64], b3[4] FP32
-    static constexpr uint32_t mbar = 168464;    // 8-byte mbarrier
-    static constexpr uint32_t tmem = 168472;    // tensor-memory base written by tcgen05.alloc
-    // one step's gradient, FP32: rows of W1 and of W2 at a stride of GROW floats (a padded
-    // stride spreads the rows written by the 32 lanes of a warp over the banks), then W3, b1,
-    // b2, b3 in parameter order
-    static constexpr uint32_t GROW = 68;
-    static constexpr uint32_t gw1 = 168960;
-    static constexpr uint32_t gw2 = gw1 + 64 * GROW * 4;
-    static constexpr uint32_t grest = gw2 + 64 * GROW * 4;   // W3 (192), b1 (64), b2 (64), b3 (3)
-    static constexpr uint32_t end = grest + 324 * 4;
+    static constexpr uint32_t gT = 53248;               // [64][128] G^T   \ gT, h1T: one 128-row operand
+    static constexpr uint32_t h1T = gT + 8 * TR_SBO_T;  // [64][128] H1^T  / h1T, h2T: another
+    static constexpr uint32_t h2T = h1T + 8 * TR_SBO_T;   // [64][128] H2^T
+    static constexpr uint32_t dz1T = h2T + 8 * TR_SBO_T;  // [64][128] dZ1^T \ one 128-row operand
+    static constexpr uint32_t dz2T = dz1T + 8 * TR_SBO_T; // [64][128] dZ2^T /
+    static constexpr uint32_t dyT = dz2T + 8 * TR_SBO_T;  // [16][128] dY^T, rows >= 3 zero
+    static constexpr uint32_t w1t = dyT + 2 * TR_SBO_T;   // [64][64] W1^T (B of layer 1)
+    static constexpr uint32_t w2t = w1t + 8 * TR_SBO_W;   // [64][64] W2^T (B of layer 2)
+    static constexpr uint32_t w3t = w2t + 8 * TR_SBO_W;   // [16][64] W3^T, rows >= 3 zero (B of layer 3)
+    static constexpr uint32_t w2n = w3t + 2048;           // [64][64] W2 (B of dH1)
+    static constexpr uint32_t w3n = w2n + 8192;           // [64][16] W3, columns >= 3 zero (B of dH2)
+    static constexpr uint32_t bias = w3n + 2048;          // b1[64], b2[64], b3[4] FP32
+    static constexpr uint32_t grest = bias + 132 * 4;     // one step's gradient of W3 (192), b1, b2, b3
+    static constexpr uint32_t sched = grest + 324 * 4;    // learning rate and the two bias corrections
+    static constexpr uint32_t mbar = sched + 16;          // 8-byte mbarrier
+    static constexpr uint32_t tmem = mbar + 8;            // tensor-memory base written by tcgen05.alloc
+    static constexpr uint32_t end = tmem + 8;
 };
 static_assert(St::end <= 227 * 1024, "shared memory of the training kernel");
+static_assert(St::mbar % 8 == 0 && St::w2n % 16 == 0 && St::w1t % 16 == 0, "alignment of the operands and the mbarrier");
 
 struct TcTrainArgs {
     float* theta;            // n_mats x MLP_PARAMS FP32 masters
@@ -525,97 +533,127 @@ struct TcTrainArgs {
     int mode;                // 0: Adam steps, 1: accumulate the gradient only
 };
 
+// Byte offset of element (r, c) of an operand with padded core matrices.
+__device__ __forceinline__ uint32_t cm_off_p(uint32_t r, uint32_t c, uint32_t sbo) {
+    return (r >> 3) * sbo + (c >> 3) * TR_LBO + (r & 7u) * 16u + (c & 7u) * 2u;
+}
+
+// Shared-memory matrix descriptor of any leading and stride byte offset (no swizzle).
+__device__ __forceinline__ uint64_t sdesc_ls(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
+           ((uint64_t)1 << 46);
+}
+
+// An operand of a product: its address and layout.
+struct TrOp {
+    uint32_t addr, lbo, sbo;
+};
+
 __device__ __forceinline__ void put_bf16(unsigned char* sm, uint32_t off, float x) {
     *reinterpret_cast<__nv_bfloat16*>(sm + off) = __float2bfloat16_rn(x);
 }
 
-// The network's parameters as BF16 operands (both orientations where the backward pass
-// needs them) and FP32 biases.
-__device__ void tr_load_weights(unsigned char* sm, const float* __restrict__ th) {
-    for (uint32_t i = threadIdx.x; i < 64u * 64u; i += blockDim.x) {
-        const uint32_t in = i >> 6, out = i & 63u;
-        put_bf16(sm, St::w1t + cm_off(out, in), th[P_W1 + i]);
-        const float w2 = th[P_W2 + i];
-        put_bf16(sm, St::w2t + cm_off(out, in), w2);
-        put_bf16(sm, St::w2n + cm_off(in, out), w2);
-    }
-    for (uint32_t i = threadIdx.x; i < 16u * 64u; i += blockDim.x) {
-        const uint32_t out = i >> 6, in = i & 63u;
-        const float w = out < 3 ? th[P_W3 + in * 3 + out] : 0.0f;
-        put_bf16(sm, St::w3t + cm_off_k(out, in, 64), w);
-        put_bf16(sm, St::w3n + cm_off_k(in, out, 16), w);
-    }
-    float* bias = reinterpret_cast<float*>(sm + St::bias);
-    for (uint32_t i = threadIdx.x; i < 132u; i += blockDim.x)
-        bias[i] = i < 64 ? th[P_B1 + i] : (i < 128 ? th[P_B2 + i - 64] : (i < 131 ? th[P_B3 + i - 128] : 0.0f));
+// `k16` K = 16 steps of one product (one thread).
+__device__ __forceinline__ void tr_issue(uint32_t d, TrOp a, TrOp b, uint32_t id, uint32_t k16) {
+    for (uint32_t s = 0; s < k16; ++s)
+        mma_bf16(d, sdesc_ls(a.addr + 2u * a.lbo * s, a.lbo, a.sbo), sdesc_ls(b.addr + 2u * b.lbo * s, b.lbo, b.sbo), id,
+                 s > 0);
 }
 
 // Makes the operand rows written by every thread visible to the tensor cores, issues
-// `k16` K = 16 steps of one product from thread 0 and waits for it.  False if the wait
-// ran out (every thread gets the same answer).
-__device__ __forceinline__ bool tr_mma(uint32_t mbar, uint32_t* phase, uint32_t d, uint32_t a, uint32_t ka,
-                                       uint32_t b, uint32_t kb, uint32_t id, uint32_t k16) {
+// `k16` K = 16 steps of one product from thread 0 and waits for it.  False if this thread's
+// wait ran out; the steps' end brings the threads' answers together.
+__device__ __forceinline__ bool tr_mma(uint32_t mbar, uint32_t* phase, uint32_t d, TrOp a, TrOp b, uint32_t id,
+                                       uint32_t k16) {
     fence_async_smem();
     fence_before();
     __syncthreads();
     if (threadIdx.x == 0) {
         fence_after();
-        for (uint32_t s = 0; s < k16; ++s) mma_bf16(d, sdesc_k(a + 256u * s, ka), sdesc_k(b + 256u * s, kb), id, s > 0);
+        tr_issue(d, a, b, id, k16);
         mma_commit(mbar);
     }
     const bool done = mbar_wait(mbar, *phase);
     *phase ^= 1u;
-    const bool ok = !__syncthreads_or(!done);
     fence_after();
-    return ok;
+    return done;
 }
 
-// relu(acc + bias) of 64 accumulator columns: row t of a [128][64] operand, column t of a
-// [64][128] transposed one, and the relu'(h) > 0 mask of the BF16 values.
-__device__ __forceinline__ uint64_t tr_hidden(unsigned char* sm, uint32_t dst, uint32_t dstT, uint32_t taddr,
-                                              const float* bias, uint32_t t) {
-    uint64_t mask = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        float v[16];
-        tmem_ld16(taddr + 16u * q, v);
-        uint32_t p[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            p[k] = pack2(fmaxf(v[2 * k] + bias[16 * q + 2 * k], 0.0f), fmaxf(v[2 * k + 1] + bias[16 * q + 2 * k + 1], 0.0f));
-            const uint32_t c = 16 * q + 2 * k;
-            *reinterpret_cast<uint16_t*>(sm + dstT + cm_off_k(c, t, 128)) = (uint16_t)(p[k] & 0xFFFFu);
-            *reinterpret_cast<uint16_t*>(sm + dstT + cm_off_k(c + 1, t, 128)) = (uint16_t)(p[k] >> 16);
-            mask |= (uint64_t)((p[k] & 0x7FFFu) != 0 && !(p[k] & 0x8000u)) << c;
-            mask |= (uint64_t)(((p[k] >> 16) & 0x7FFFu) != 0 && !(p[k] & 0x80000000u)) << (c + 1);
-        }
-        *reinterpret_cast<uint4*>(sm + dst + cm_off(t, 16 * q)) = make_uint4(p[0], p[1], p[2], p[3]);
-        *reinterpret_cast<uint4*>(sm + dst + cm_off(t, 16 * q + 8)) = make_uint4(p[4], p[5], p[6], p[7]);
+// Sixteen BF16 columns c0 .. c0 + 15 of row t (packed in pairs) into row t of a [128][64]
+// operand (dst != ~0u) and column t of a [64][128] transposed one.
+__device__ __forceinline__ void tr_store16(unsigned char* sm, uint32_t dst, uint32_t dstT, const uint32_t (&p)[8],
+                                           uint32_t t, uint32_t c0) {
+    if (dst != ~0u) {
+        *reinterpret_cast<uint4*>(sm + dst + cm_off(t, c0)) = make_uint4(p[0], p[1], p[2], p[3]);
+        *reinterpret_cast<uint4*>(sm + dst + cm_off(t, c0 + 8)) = make_uint4(p[4], p[5], p[6], p[7]);
     }
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) {
+        *reinterpret_cast<uint16_t*>(sm + dstT + cm_off_p(c0 + 2 * k, t, TR_SBO_T)) = (uint16_t)(p[k] & 0xFFFFu);
+        *reinterpret_cast<uint16_t*>(sm + dstT + cm_off_p(c0 + 2 * k + 1, t, TR_SBO_T)) = (uint16_t)(p[k] >> 16);
+    }
+}
+
+// The eight frequencies 8 half + 1 .. 8 half + 8 of coordinate x for row t: sin into columns
+// col .. col + 7 and cos into col + 16 .. col + 23 of G, and the same of G^T.  The values are
+// tc_features' (its packed operations round each lane as these scalar ones).
+__device__ __forceinline__ void tr_features(unsigned char* sm, uint32_t t, float x, uint32_t half, uint32_t col) {
+    float S1, C1;
+    sincospif(x, &S1, &C1);
+    float sk = S1, ck = C1;
+    if (half) sincospif(9.0f * x, &sk, &ck);
+    uint32_t ws[4], wc[4];
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+        const float sn = fmaf(sk, C1, __fmul_rn(ck, S1));
+        const float cn = fmaf(ck, C1, __fmul_rn(sk, -S1));
+        ws[j / 2] = pack2(sk, sn);
+        wc[j / 2] = pack2(ck, cn);
+        if (j < 6) {
+            sk = fmaf(sn, C1, __fmul_rn(cn, S1));
+            ck = fmaf(cn, C1, __fmul_rn(sn, -S1));
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t c0 = col + 16u * h;
+        const uint32_t w[4] = {h ? wc[0] : ws[0], h ? wc[1] : ws[1], h ? wc[2] : ws[2], h ? wc[3] : ws[3]};
+        *reinterpret_cast<uint4*>(sm + St::a0 + cm_off(t, c0)) = make_uint4(w[0], w[1], w[2], w[3]);
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) {
+            *reinterpret_cast<uint16_t*>(sm + St::gT + cm_off_p(c0 + 2 * k, t, TR_SBO_T)) = (uint16_t)(w[k] & 0xFFFFu);
+            *reinterpret_cast<uint16_t*>(sm + St::gT + cm_off_p(c0 + 2 * k + 1, t, TR_SBO_T)) = (uint16_t)(w[k] >> 16);
+        }
+    }
+}
+
+// relu(acc + bias) of this thread's 16 accumulator columns of row t into both copies; returns
+// the relu'(h) > 0 mask of the BF16 values.
+__device__ __forceinline__ uint32_t tr_hidden(unsigned char* sm, uint32_t dst, uint32_t dstT, uint32_t taddr,
+                                              const float* bias, uint32_t t, uint32_t c0) {
+    float v[16];
+    tmem_ld16(taddr + c0, v);
+    uint32_t p[8], mask = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        p[k] = pack2(fmaxf(v[2 * k] + bias[c0 + 2 * k], 0.0f), fmaxf(v[2 * k + 1] + bias[c0 + 2 * k + 1], 0.0f));
+        mask |= (uint32_t)((p[k] & 0x7FFFu) != 0 && !(p[k] & 0x8000u)) << (2 * k);
+        mask |= (uint32_t)(((p[k] >> 16) & 0x7FFFu) != 0 && !(p[k] & 0x80000000u)) << (2 * k + 1);
+    }
+    tr_store16(sm, dst, dstT, p, t, c0);
     return mask;
 }
 
-// acc . mask of 64 accumulator columns as BF16: row t of a [128][64] operand (dst != ~0u)
-// and column t of a [64][128] transposed one.
-__device__ __forceinline__ void tr_masked(unsigned char* sm, uint32_t dst, uint32_t dstT, uint32_t taddr, uint64_t mask,
-                                          uint32_t t) {
+// acc . mask of this thread's 16 accumulator columns as BF16 into both copies.
+__device__ __forceinline__ void tr_masked(unsigned char* sm, uint32_t dst, uint32_t dstT, uint32_t taddr, uint32_t mask,
+                                          uint32_t t, uint32_t c0) {
+    float v[16];
+    tmem_ld16(taddr + c0, v);
+    uint32_t p[8];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        float v[16];
-        tmem_ld16(taddr + 16u * q, v);
-        uint32_t p[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const uint32_t c = 16 * q + 2 * k;
-            p[k] = pack2(((mask >> c) & 1u) ? v[2 * k] : 0.0f, ((mask >> (c + 1)) & 1u) ? v[2 * k + 1] : 0.0f);
-            *reinterpret_cast<uint16_t*>(sm + dstT + cm_off_k(c, t, 128)) = (uint16_t)(p[k] & 0xFFFFu);
-            *reinterpret_cast<uint16_t*>(sm + dstT + cm_off_k(c + 1, t, 128)) = (uint16_t)(p[k] >> 16);
-        }
-        if (dst != ~0u) {
-            *reinterpret_cast<uint4*>(sm + dst + cm_off(t, 16 * q)) = make_uint4(p[0], p[1], p[2], p[3]);
-            *reinterpret_cast<uint4*>(sm + dst + cm_off(t, 16 * q + 8)) = make_uint4(p[4], p[5], p[6], p[7]);
-        }
-    }
+    for (int k = 0; k < 8; ++k)
+        p[k] = pack2(((mask >> (2 * k)) & 1u) ? v[2 * k] : 0.0f, ((mask >> (2 * k + 1)) & 1u) ? v[2 * k + 1] : 0.0f);
+    tr_store16(sm, dst, dstT, p, t, c0);
 }
 
 // Sum of row r of a [rows][128] BF16 operand (a bias gradient: a column sum over the batch).
@@ -623,7 +661,7 @@ __device__ __forceinline__ float tr_row_sum(const unsigned char* sm, uint32_t ba
     float s = 0.0f;
 #pragma unroll 4
     for (uint32_t c = 0; c < 128; c += 8) {
-        const uint4 w = *reinterpret_cast<const uint4*>(sm + base + cm_off_k(r, c, 128));
+        const uint4 w = *reinterpret_cast<const uint4*>(sm + base + cm_off_p(r, c, TR_SBO_T));
         const uint32_t x[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
         for (int k = 0; k < 4; ++k) s += __uint_as_float(x[k] << 16) + __uint_as_float(x[k] & 0xFFFF0000u);
@@ -631,211 +669,257 @@ __device__ __forceinline__ float tr_row_sum(const unsigned char* sm, uint32_t ba
     return s;
 }
 
+// One Adam update of weight w with moments m and v; the roundings are spelled out so that the
+// trained parameters do not depend on how the compiler contracts the sums.
+__device__ __forceinline__ float tr_adam(float w, float* m, float* v, float g, float lr_t, float bc1, float bc2) {
+    const float m1 = __fmaf_rn(0.1f, g, __fmul_rn(0.9f, *m));
+    const float m2 = __fmaf_rn(__fmul_rn(0.001f, g), g, __fmul_rn(0.999f, *v));
+    *m = m1;
+    *v = m2;
+    return w - lr_t * (m1 / bc1) / (sqrtf(m2 / bc2) + 1e-8f);
+}
+
+// Parameter index of entry e of the gradient stage St::grest.
+__device__ __forceinline__ uint32_t tr_rest_index(uint32_t e) {
+    return e < 192 ? P_W3 + e : e < 256 ? P_B1 + (e - 192) : e < 320 ? P_B2 + (e - 256) : P_B3 + (e - 320);
+}
+
+// The operands of parameter e of the stage (a weight of W3 or a bias).
+__device__ __forceinline__ void tr_put_rest(unsigned char* sm, uint32_t e, float w) {
+    float* bias = reinterpret_cast<float*>(sm + St::bias);
+    if (e < 192) {
+        const uint32_t in = e / 3u, out = e % 3u;
+        put_bf16(sm, St::w3t + cm_off_k(out, in, 64), w);
+        put_bf16(sm, St::w3n + cm_off_k(in, out, 16), w);
+    } else {
+        bias[e - 192] = w;   // b1, b2, b3 in the stage's order
+    }
+}
+
+// The operands of this thread's 16 weights W[in][c0 .. c0 + 15] of W1 (second = false) or W2.
+__device__ __forceinline__ void tr_put16(unsigned char* sm, bool second, uint32_t in, uint32_t c0, const float (&w)[16]) {
+    uint32_t p[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) p[k] = pack2(w[2 * k], w[2 * k + 1]);
+    const uint32_t wt = second ? St::w2t : St::w1t;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) {
+        *reinterpret_cast<uint16_t*>(sm + wt + cm_off_p(c0 + 2 * k, in, TR_SBO_W)) = (uint16_t)(p[k] & 0xFFFFu);
+        *reinterpret_cast<uint16_t*>(sm + wt + cm_off_p(c0 + 2 * k + 1, in, TR_SBO_W)) = (uint16_t)(p[k] >> 16);
+    }
+    if (second) {
+        *reinterpret_cast<uint4*>(sm + St::w2n + cm_off(in, c0)) = make_uint4(p[0], p[1], p[2], p[3]);
+        *reinterpret_cast<uint4*>(sm + St::w2n + cm_off(in, c0 + 8)) = make_uint4(p[4], p[5], p[6], p[7]);
+    }
+}
+
+// The data row of minibatch row t in step `step`: in order (gradient mode) or a fixed
+// per-epoch shuffle.
+__device__ __forceinline__ const float* tr_row(const TcTrainArgs& A, const float* data, uint32_t step, uint32_t t) {
+    const uint64_t k = A.sample0 + (uint64_t)step * TC_ROWS + t;
+    uint32_t row;
+    if (A.mode == 1) {
+        row = (uint32_t)k;
+    } else {
+        const uint32_t epoch = (uint32_t)(k >> (31 - __clz(A.n_data)));
+        row = (uint32_t)(k * 2654435761ull + (uint64_t)epoch * 0x9E3779B9ull) & (A.n_data - 1);
+    }
+    return data + (size_t)row * 5;
+}
+
 // One CTA per (split, material) runs `steps` minibatch steps of 128 rows.
-__global__ void __launch_bounds__(TC_ROWS) k_mlp_train_tc(TcTrainArgs A) {
+__global__ void __launch_bounds__(TR_T) k_mlp_train_tc(TcTrainArgs A) {
     extern __shared__ __align__(1024) unsigned char sm[];
-    const uint32_t t = threadIdx.x;
+    const uint32_t tid = threadIdx.x, warp = tid >> 5;
+    const uint32_t t = (warp & 3u) * 32u + (tid & 31u);   // row, and tensor-memory lane
+    const uint32_t cg = warp >> 2, c0 = 16u * cg;         // this thread's columns c0 .. c0 + 15
+    const bool second = t >= 64;                          // its weights: row t of W1, or row t - 64 of W2
+    const uint32_t in = t & 63u;
     const uint32_t base = smem_u32(sm), mbar = base + St::mbar;
     const uint32_t mat = blockIdx.y;
     const size_t pbase = (size_t)mat * MLP_PARAMS;
     const float* data = A.data + (size_t)mat * A.n_data * 5;
-    if (t == 0) {
+    if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (t < 32) {
+    if (tid < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + St::tmem),
                      "r"(TR_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    // the zero columns of dY and zero rows of dY^T stay zero: only outputs 0..2 are written
-    for (uint32_t i = t; i < 128u * 16u; i += TC_ROWS) {
-        *reinterpret_cast<uint16_t*>(sm + St::dy + cm_off_k(i >> 4, i & 15u, 16)) = 0;
-        *reinterpret_cast<uint16_t*>(sm + St::dyT + cm_off_k(i & 15u, i >> 4, 128)) = 0;
+    // the zero columns of dY and W3, and zero rows of dY^T and W3^T, stay zero: only outputs
+    // 0..2 are written
+    for (uint32_t i = tid; i < 4096u / 4; i += TR_T) *reinterpret_cast<uint32_t*>(sm + St::dy + 4 * i) = 0u;
+    for (uint32_t i = tid; i < 2u * TR_SBO_T / 4; i += TR_T) *reinterpret_cast<uint32_t*>(sm + St::dyT + 4 * i) = 0u;
+    for (uint32_t i = tid; i < 2048u / 4; i += TR_T) {
+        *reinterpret_cast<uint32_t*>(sm + St::w3t + 4 * i) = 0u;
+        *reinterpret_cast<uint32_t*>(sm + St::w3n + 4 * i) = 0u;
     }
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + St::tmem);
-    const uint32_t lane_addr = tmem + (((t >> 5) * 32u) << 16);
-    const float* bias = reinterpret_cast<const float*>(sm + St::bias);
-    const uint32_t log2n = 31 - __clz(A.n_data);
+    const uint32_t lane_addr = tmem + (((warp & 3u) * 32u) << 16);
+    float* bias = reinterpret_cast<float*>(sm + St::bias);
+    float* grest = reinterpret_cast<float*>(sm + St::grest);
+    float* sched = reinterpret_cast<float*>(sm + St::sched);
+    // this thread's masters and moments: 16 weights of a row of W1 or W2, and one parameter of
+    // the rest for the first 323 threads
+    const size_t own = pbase + (second ? P_W2 : P_W1) + in * 64u + c0;
+    const size_t rest = pbase + tr_rest_index(min(tid, TR_REST - 1u));
+    const bool has_rest = tid < TR_REST;
+    float w[16], m[16], v[16], wr = 0.0f, mr = 0.0f, vr = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        w[k] = A.theta[own + k];
+        m[k] = A.mode == 0 ? A.adam_m[own + k] : 0.0f;
+        v[k] = A.mode == 0 ? A.adam_v[own + k] : 0.0f;
+    }
+    if (has_rest) {
+        wr = A.theta[rest];
+        if (A.mode == 0) {
+            mr = A.adam_m[rest];
+            vr = A.adam_v[rest];
+        }
+        tr_put_rest(sm, tid, wr);
+    }
+    tr_put16(sm, second, in, c0, w);
     uint32_t phase = 0;
     float loss = 0.0f;
     bool ok = true;
-    tr_load_weights(sm, A.theta + pbase);   // later steps update the operands in place
-    __syncthreads();
-    for (uint32_t s = 0; s < A.steps && ok; ++s) {
+    // the coordinate and the targets of the first step's row; a later step's are loaded while
+    // the one before it runs
+    const float* d = tr_row(A, data, blockIdx.x, t);
+    float x = d[cg >> 1], tg0 = d[2], tg1 = d[3], tg2 = d[4];
+    const TrOp opA0{base + St::a0, 128, 1024}, opA1{base + St::a1, 128, 1024}, opDz2{base + St::dz2, 128, 1024};
+    const TrOp opDy{base + St::dy, 128, 256}, opW3n{base + St::w3n, 128, 256}, opW3t{base + St::w3t, 128, 1024};
+    const TrOp opW1t{base + St::w1t, TR_LBO, TR_SBO_W}, opW2t{base + St::w2t, TR_LBO, TR_SBO_W};
+    const TrOp opW2n{base + St::w2n, 128, 1024};
+    const TrOp opGT{base + St::gT, TR_LBO, TR_SBO_T}, opH1T{base + St::h1T, TR_LBO, TR_SBO_T};
+    const TrOp opDzT{base + St::dz1T, TR_LBO, TR_SBO_T}, opDyT{base + St::dyT, TR_LBO, TR_SBO_T};
+    for (uint32_t s = 0; s < A.steps; ++s) {
         const uint32_t step = s * gridDim.x + blockIdx.x;
-        // ---- row t of the minibatch: in order (gradient mode) or a fixed per-epoch shuffle
-        const uint64_t k = A.sample0 + (uint64_t)step * TC_ROWS + t;
-        uint32_t row;
-        if (A.mode == 1) {
-            row = (uint32_t)k;
-        } else {
-            const uint32_t epoch = (uint32_t)(k >> log2n);
-            row = (uint32_t)(k * 2654435761ull + (uint64_t)epoch * 0x9E3779B9ull) & (A.n_data - 1);
-        }
-        const float* d = data + (size_t)row * 5;
-        const float u = d[0], v = d[1], tg0 = d[2], tg1 = d[3], tg2 = d[4];
         // ---- features: row t of G, column t of G^T
-        tc_features(sm, t, u, v);
-        for (uint32_t c = 0; c < 64; c += 8) {
-            const uint4 w = *reinterpret_cast<const uint4*>(sm + St::a0 + cm_off(t, c));
-            const uint32_t x[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                *reinterpret_cast<uint16_t*>(sm + St::gT + cm_off_k(c + 2 * q, t, 128)) = (uint16_t)(x[q] & 0xFFFFu);
-                *reinterpret_cast<uint16_t*>(sm + St::gT + cm_off_k(c + 2 * q + 1, t, 128)) = (uint16_t)(x[q] >> 16);
-            }
+        tr_features(sm, t, x, cg & 1u, 32u * (cg >> 1) + 8u * (cg & 1u));
+        const float y0 = tg0, y1 = tg1, y2 = tg2;
+        if (s + 1 < A.steps) {
+            const float* dn = tr_row(A, data, step + gridDim.x, t);
+            x = dn[cg >> 1];
+            tg0 = dn[2];
+            tg1 = dn[3];
+            tg2 = dn[4];
         }
         // ---- forward
-        ok = tr_mma(mbar, &phase, tmem + 0u, base + St::a0, 64, base + St::w1t, 64, idesc(128, 64), 4);
-        if (!ok) break;
-        const uint64_t mask1 = tr_hidden(sm, St::a1, St::h1T, lane_addr + 0u, bias, t);
-        fence_before();
-        ok = tr_mma(mbar, &phase, tmem + 64u, base + St::a1, 64, base + St::w2t, 64, idesc(128, 64), 4);
-        if (!ok) break;
-        const uint64_t mask2 = tr_hidden(sm, St::a0, St::h2T, lane_addr + 64u, bias + 64, t);
-        fence_before();
-        ok = tr_mma(mbar, &phase, tmem + 128u, base + St::a0, 64, base + St::w3t, 64, idesc(128, 16), 4);
-        if (!ok) break;
+        ok &= tr_mma(mbar, &phase, tmem + 0u, opA0, opW1t, idesc(128, 64), 4);
+        const uint32_t mask1 = tr_hidden(sm, St::a1, St::h1T, lane_addr + 0u, bias, t, c0);
+        ok &= tr_mma(mbar, &phase, tmem + 64u, opA1, opW2t, idesc(128, 64), 4);
+        const uint32_t mask2 = tr_hidden(sm, St::a0, St::h2T, lane_addr + 64u, bias + 64, t, c0);
+        ok &= tr_mma(mbar, &phase, tmem + 128u, opA0, opW3t, idesc(128, 16), 4);
         // ---- dL/dy and the loss
-        {
+        if (cg == 0) {
             float o[4];
             tmem_ld4(lane_addr + 128u, o);
-            const float e[3] = {o[0] + bias[128] - tg0, o[1] + bias[129] - tg1, o[2] + bias[130] - tg2};
+            const float e[3] = {o[0] + bias[128] - y0, o[1] + bias[129] - y1, o[2] + bias[130] - y2};
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 loss += e[q] * e[q];
                 const float g = A.grad_scale * e[q];
                 put_bf16(sm, St::dy + cm_off_k(t, q, 16), g);
-                put_bf16(sm, St::dyT + cm_off_k(q, t, 128), g);
+                put_bf16(sm, St::dyT + cm_off_p(q, t, TR_SBO_T), g);
             }
         }
-        fence_before();
         // ---- dH2 = dY W3^T, masked
-        ok = tr_mma(mbar, &phase, tmem + 0u, base + St::dy, 16, base + St::w3n, 16, idesc(128, 64), 1);
-        if (!ok) break;
-        tr_masked(sm, St::dz2, St::dz2T, lane_addr + 0u, mask2, t);
-        fence_before();
+        ok &= tr_mma(mbar, &phase, tmem + 0u, opDy, opW3n, idesc(128, 64), 1);
+        tr_masked(sm, St::dz2, St::dz2T, lane_addr + 0u, mask2, t, c0);
         // ---- dH1 = dZ2 W2^T, masked
-        ok = tr_mma(mbar, &phase, tmem + 64u, base + St::dz2, 64, base + St::w2n, 64, idesc(128, 64), 4);
-        if (!ok) break;
-        tr_masked(sm, ~0u, St::dz1T, lane_addr + 64u, mask1, t);
-        fence_before();
+        ok &= tr_mma(mbar, &phase, tmem + 64u, opDz2, opW2n, idesc(128, 64), 4);
+        tr_masked(sm, ~0u, St::dz1T, lane_addr + 64u, mask1, t, c0);
         // ---- weight gradients: [G^T; H1^T] x [dZ1^T; dZ2^T]^T and [H1^T; H2^T] x dY
         fence_async_smem();
         fence_before();
         __syncthreads();
-        if (t == 0) {
+        if (tid == 0) {
             fence_after();
-            for (uint32_t q = 0; q < 8; ++q)
-                mma_bf16(tmem + 0u, sdesc_k(base + St::gT + 256u * q, 128), sdesc_k(base + St::dz1T + 256u * q, 128),
-                         idesc(128, 128), q > 0);
-            for (uint32_t q = 0; q < 8; ++q)
-                mma_bf16(tmem + 128u, sdesc_k(base + St::h1T + 256u * q, 128), sdesc_k(base + St::dyT + 256u * q, 128),
-                         idesc(128, 16), q > 0);
+            tr_issue(tmem + 0u, opGT, opDzT, idesc(128, 128), 8);
+            tr_issue(tmem + 128u, opH1T, opDyT, idesc(128, 16), 8);
             mma_commit(mbar);
         }
-        // bias gradients while the tensor cores run: column sums of dZ1, dZ2 and dY
-        const float gb = t < 64 ? tr_row_sum(sm, St::dz1T, t) : tr_row_sum(sm, St::dz2T, t - 64);
-        const float gb3 = t < 3 ? tr_row_sum(sm, St::dyT, t) : 0.0f;
-        const bool done = mbar_wait(mbar, phase);
+        // while the tensor cores run: the bias gradients (column sums of dZ1, dZ2 and dY) in four
+        // warps, the step's learning rate and bias corrections in another
+        if (tid < 128) {
+            grest[192 + tid] = tid < 64 ? tr_row_sum(sm, St::dz1T, tid) : tr_row_sum(sm, St::dz2T, tid - 64);
+            if (tid < 3) grest[320 + tid] = tr_row_sum(sm, St::dyT, tid);
+        } else if (tid == 256 && A.mode == 0) {
+            const uint32_t adam_t = A.step0 + step + 1;
+            const float frac = A.total_steps > 1 ? (float)(A.step0 + step) / (float)(A.total_steps - 1) : 0.0f;
+            sched[0] = A.lr * (0.05f + 0.95f * 0.5f * (1.0f + cospif(fminf(frac, 1.0f))));
+            sched[1] = 1.0f - powf(0.9f, (float)adam_t);
+            sched[2] = 1.0f - powf(0.999f, (float)adam_t);
+        }
+        __syncwarp();
+        ok &= mbar_wait(mbar, phase);
         phase ^= 1u;
-        if (__syncthreads_or(!done)) {
+        fence_after();
+        // ---- this thread's gradients: row t of dW1 (columns 0..63) or row t - 64 of dW2 (columns
+        // 64..127); rows 64.. of the second product hold dW3 (columns 128..130)
+        float g[16];
+        tmem_ld16(lane_addr + (second ? 64u : 0u) + c0, g);
+        if (second && cg == 0) {
+            float g3[4];
+            tmem_ld4(lane_addr + 128u, g3);
+            for (uint32_t o = 0; o < 3; ++o) grest[in * 3 + o] = g3[o];
+        }
+        fence_before();
+        if (__syncthreads_or(!ok)) {   // a wait ran out somewhere: every thread leaves
             ok = false;
             break;
         }
-        fence_after();
-        // ---- the step's gradient into shared memory: thread t < 64 holds row t of dW1 (tensor-
-        // memory lane t, columns 0..63), thread t >= 64 row t - 64 of dW2 (columns 64..127)
-        // and of dW3 (columns 128..130)
-        float* gw1 = reinterpret_cast<float*>(sm + St::gw1);
-        float* gw2 = reinterpret_cast<float*>(sm + St::gw2);
-        float* grest = reinterpret_cast<float*>(sm + St::grest);
-        {
-            float* row = t < 64 ? gw1 + t * St::GROW : gw2 + (t - 64) * St::GROW;
-            const uint32_t col0 = t < 64 ? 0u : 64u;
+        // ---- Adam (or gradient accumulation); the updated weights go straight into the BF16
+        // operands of the next step
+        if (A.mode == 1) {
 #pragma unroll
-            for (uint32_t q = 0; q < 4; ++q) {
-                float g[16];
-                tmem_ld16(lane_addr + col0 + 16u * q, g);
+            for (int k = 0; k < 16; ++k) atomicAdd(&A.grad[own + k], g[k]);
+            if (has_rest) atomicAdd(&A.grad[rest], grest[tid]);
+        } else {
+            const float lr_t = sched[0], bc1 = sched[1], bc2 = sched[2];
 #pragma unroll
-                for (int k = 0; k < 16; k += 4)
-                    *reinterpret_cast<float4*>(row + 16 * q + k) = make_float4(g[k], g[k + 1], g[k + 2], g[k + 3]);
-            }
-            if (t >= 64) {
-                float g3[4];
-                tmem_ld4(lane_addr + 128u, g3);
-                for (uint32_t o = 0; o < 3; ++o) grest[(t - 64) * 3 + o] = g3[o];
-            }
-            grest[192 + t] = gb;                  // b1 (t < 64), then b2
-            if (t < 3) grest[320 + t] = gb3;
-        }
-        fence_before();
-        __syncthreads();
-        // ---- Adam (or gradient accumulation) over the parameters in order, coalesced; the
-        // updated weights go straight into the BF16 operands of the next step
-        const uint32_t adam_t = A.step0 + step + 1;
-        const float frac = A.total_steps > 1 ? (float)(A.step0 + step) / (float)(A.total_steps - 1) : 0.0f;
-        const float lr_t = A.lr * (0.05f + 0.95f * 0.5f * (1.0f + cospif(fminf(frac, 1.0f))));
-        const float bc1 = 1.0f - powf(0.9f, (float)adam_t), bc2 = 1.0f - powf(0.999f, (float)adam_t);
-        float* bias_w = reinterpret_cast<float*>(sm + St::bias);
-#pragma unroll 4
-        for (uint32_t i = t; i < MLP_PARAMS; i += TC_ROWS) {
-            float g;
-            if (i < (uint32_t)P_B1) g = gw1[(i >> 6) * St::GROW + (i & 63u)];
-            else if (i < (uint32_t)P_W2) g = grest[192 + (i - P_B1)];
-            else if (i < (uint32_t)P_B2) g = gw2[((i - P_W2) >> 6) * St::GROW + ((i - P_W2) & 63u)];
-            else if (i < (uint32_t)P_W3) g = grest[256 + (i - P_B2)];
-            else if (i < (uint32_t)P_B3) g = grest[i - P_W3];
-            else g = grest[320 + (i - P_B3)];
-            const size_t k = pbase + i;
-            if (A.mode == 1) {
-                atomicAdd(&A.grad[k], g);
-                continue;
-            }
-            const float m1 = 0.9f * A.adam_m[k] + 0.1f * g;
-            const float m2 = 0.999f * A.adam_v[k] + 0.001f * g * g;
-            A.adam_m[k] = m1;
-            A.adam_v[k] = m2;
-            const float w = A.theta[k] - lr_t * (m1 / bc1) / (sqrtf(m2 / bc2) + 1e-8f);
-            A.theta[k] = w;
-            if (i < (uint32_t)P_B1) {
-                put_bf16(sm, St::w1t + cm_off(i & 63u, i >> 6), w);
-            } else if (i < (uint32_t)P_W2) {
-                bias_w[i - P_B1] = w;
-            } else if (i < (uint32_t)P_B2) {
-                const uint32_t j = i - P_W2, in = j >> 6, out = j & 63u;
-                put_bf16(sm, St::w2t + cm_off(out, in), w);
-                put_bf16(sm, St::w2n + cm_off(in, out), w);
-            } else if (i < (uint32_t)P_W3) {
-                bias_w[64 + (i - P_B2)] = w;
-            } else if (i < (uint32_t)P_B3) {
-                const uint32_t j = i - P_W3, in = j / 3u, out = j % 3u;
-                put_bf16(sm, St::w3t + cm_off_k(out, in, 64), w);
-                put_bf16(sm, St::w3n + cm_off_k(in, out, 16), w);
-            } else {
-                bias_w[128 + (i - P_B3)] = w;
+            for (int k = 0; k < 16; ++k) w[k] = tr_adam(w[k], &m[k], &v[k], g[k], lr_t, bc1, bc2);
+            tr_put16(sm, second, in, c0, w);
+            if (has_rest) {
+                wr = tr_adam(wr, &mr, &vr, grest[tid], lr_t, bc1, bc2);
+                tr_put_rest(sm, tid, wr);
             }
         }
-        fence_before();
-        __syncthreads();   // the next step reads the updated operands
+        // the next step's first product is issued behind a block barrier, and its stores to the
+        // stage come after that: the updated operands and the stage's reads are ordered by it
+    }
+    if (A.mode == 0 && ok) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            A.theta[own + k] = w[k];
+            A.adam_m[own + k] = m[k];
+            A.adam_v[own + k] = v[k];
+        }
+        if (has_rest) {
+            A.theta[rest] = wr;
+            A.adam_m[rest] = mr;
+            A.adam_v[rest] = vr;
+        }
     }
     if (!ok) {
-        if (t == 0) {
+        if (tid == 0) {
             if (A.err) atomicOr(A.err, ERR_TIMEOUT);
             atomicExch(&A.loss[mat], __int_as_float(0x7FC00000));
         }
-    } else {
+    } else if (cg == 0) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, o);
-        if ((t & 31u) == 0) atomicAdd(&A.loss[mat], loss);
+        if ((tid & 31u) == 0) atomicAdd(&A.loss[mat], loss);
     }
     fence_before();
     __syncthreads();
-    if (t < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TR_COLS));
+    if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TR_COLS));
 }
 
 }  // namespace
@@ -848,7 +932,7 @@ cudaError_t launch_mlp_train(float* theta, float* adam_m, float* adam_v, float* 
                   grad_scale, mode};
     cudaError_t e = cudaFuncSetAttribute(k_mlp_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)St::end);
     if (e != cudaSuccess) return e;
-    k_mlp_train_tc<<<dim3(splits, n_mats), TC_ROWS, St::end, s>>>(A);
+    k_mlp_train_tc<<<dim3(splits, n_mats), TR_T, St::end, s>>>(A);
     return cudaGetLastError();
 }
 
