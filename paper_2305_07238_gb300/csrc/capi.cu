@@ -1015,14 +1015,14 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     for (uint32_t i = 0; i < L; ++i) init_theta(d->seed * 0x100000001B3ull + train[i] + 1, th.data() + (size_t)i * MLP_PARAMS);
     float* theta = c->d_surr_theta + (size_t)s0 * MLP_PARAMS;
     cudaError_t e = cudaMemcpyAsync(theta, th.data(), th.size() * sizeof(float), cudaMemcpyHostToDevice, s);
-    // temporaries: Adam moments, pairs, losses, validation predictions
-    float *m1 = nullptr, *m2 = nullptr, *data = nullptr, *loss = nullptr, *pred = nullptr;
+    // temporaries: Adam moments, pairs, losses
+    float *m1 = nullptr, *m2 = nullptr, *data = nullptr, *loss = nullptr;
     uint32_t* groots = nullptr;
     const uint32_t nv = d->n_valid;
     if ((st = dalloc(&m1, th.size())) != PMC_OK || (st = dalloc(&m2, th.size())) != PMC_OK ||
         (st = dalloc(&data, (size_t)L * std::max(d->n_train, nv) * 5)) != PMC_OK || (st = dalloc(&loss, L)) != PMC_OK ||
-        (st = dalloc(&pred, (size_t)3 * nv)) != PMC_OK || (st = dalloc(&groots, L)) != PMC_OK) {
-        dfree(&m1); dfree(&m2); dfree(&data); dfree(&loss); dfree(&pred); dfree(&groots);
+        (st = dalloc(&groots, L)) != PMC_OK) {
+        dfree(&m1); dfree(&m2); dfree(&data); dfree(&loss); dfree(&groots);
         return st;
     }
     std::vector<uint32_t> gr(L);
@@ -1045,38 +1045,21 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
                              total, lr, 2.0f / (3.0f * 128.0f), 0, 1, s);
         done += chunk;
     }
-    // validation against held-out exact values
-    std::vector<float> valid((size_t)nv * 5), out((size_t)3 * nv);
+    // validation against held-out exact values, all networks in one launch
     if (e == cudaSuccess)
         e = launch_root_samples(c->d_prog, c->d_params, c->d_rinfo, groots, L, nv, d->seed ^ 0x5DEECE66Dull, data,
                                 c->max_slots_roots ? c->max_slots_roots : 1, c->num_sms, s);
-    std::vector<float> host_data((size_t)L * nv * 5);
+    const uint32_t parts = mlp_validate_parts(L, nv, c->num_sms);
+    double* d_sum = nullptr;
+    std::vector<double> sums((size_t)L * parts);
+    if (e == cudaSuccess && dalloc(&d_sum, sums.size()) != PMC_OK) e = cudaErrorMemoryAllocation;
+    if (e == cudaSuccess) e = launch_mlp_validate(theta, data, L, nv, d_sum, &c->d_ctl->err, c->num_sms, s);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(host_data.data(), data, host_data.size() * sizeof(float), cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpyAsync(sums.data(), d_sum, sums.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    // the validation (u, v) live inside `data`: run the network on copies of them
-    float *du = nullptr, *dv = nullptr;
-    if (e == cudaSuccess && (dalloc(&du, nv) != PMC_OK || dalloc(&dv, nv) != PMC_OK)) e = cudaErrorMemoryAllocation;
-    std::vector<float> uu(nv), vv(nv);
     for (uint32_t i = 0; e == cudaSuccess && i < L; ++i) {
-        const float* hd = host_data.data() + (size_t)i * nv * 5;
-        for (uint32_t r = 0; r < nv; ++r) {
-            uu[r] = hd[5 * r];
-            vv[r] = hd[5 * r + 1];
-        }
-        e = cudaMemcpy(du, uu.data(), nv * sizeof(float), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(dv, vv.data(), nv * sizeof(float), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = launch_mlp_forward_tc(theta + (size_t)i * MLP_PARAMS, du, dv, nv, pred, 1, &c->d_ctl->err, c->num_sms, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(out.data(), pred, out.size() * sizeof(float), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) break;
         double se = 0.0;
-        for (uint32_t r = 0; r < nv; ++r)
-            for (int k = 0; k < 3; ++k) {
-                const double df = (double)out[(size_t)k * nv + r] - (double)hd[5 * r + 2 + k];
-                se += df * df;
-            }
+        for (uint32_t p = 0; p < parts; ++p) se += sums[(size_t)i * parts + p];
         const float err = (float)std::sqrt(se / (3.0 * nv));
         const uint32_t m = train[i];
         c->surr_slot[m] = (int32_t)(s0 + i);
@@ -1087,8 +1070,8 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
             for (size_t k = 0; k < list.size(); ++k)
                 if (list[k] == m) rmse[k] = err;
     }
-    dfree(&du); dfree(&dv);
-    dfree(&m1); dfree(&m2); dfree(&data); dfree(&loss); dfree(&pred); dfree(&groots);
+    dfree(&d_sum);
+    dfree(&m1); dfree(&m2); dfree(&data); dfree(&loss); dfree(&groots);
     if (e != cudaSuccess) return cuda_fail(c, e);
     c->n_surr_slots = s0 + L;
     e = upload_surrogate_maps(c);

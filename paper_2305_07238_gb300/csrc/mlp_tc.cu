@@ -15,6 +15,7 @@
 // activations rounded to BF16, FP32 accumulation).
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "nodes.cuh"
@@ -380,6 +381,47 @@ __global__ void __launch_bounds__(TC_ROWS) k_mlp_forward_tc(const float* __restr
                 for (int k = 0; k < 3; ++k) out[(size_t)k * n + r] = __int_as_float(0x7FC00000);
         }
         if (err && t == 0) atomicOr(err, ERR_TIMEOUT);
+    }
+    tc_teardown(tmem);
+}
+
+// Validation of freshly trained networks against exact values: the CTAs of row y of the grid
+// run network y over its n rows (u, v, r, g, b) in tiles of 128 and sum the squared errors
+// of the clamped outputs in FP64, one partial sum per CTA (added up by the host in a fixed
+// order; NaN if a wait for the tensor cores ran out).
+__global__ void __launch_bounds__(TC_ROWS) k_mlp_validate_tc(const float* __restrict__ theta,
+                                                             const float* __restrict__ data, uint32_t n, double* sum,
+                                                             uint32_t* err) {
+    extern __shared__ __align__(1024) unsigned char sm[];
+    __shared__ double s_part[TC_ROWS / 32];
+    const uint32_t t = threadIdx.x;
+    const uint32_t tmem = tc_setup(sm);
+    tc_load_weights(sm, theta + (size_t)blockIdx.y * MLP_PARAMS);
+    const float* rows = data + (size_t)blockIdx.y * n * 5;
+    uint32_t phase = 0;
+    bool ok = true;
+    double se = 0.0;
+    for (uint32_t r0 = blockIdx.x * TC_ROWS; r0 < n && ok; r0 += gridDim.x * TC_ROWS) {
+        const uint32_t r = r0 + t;
+        float d[5] = {};
+        if (r < n)
+            for (int k = 0; k < 5; ++k) d[k] = rows[(size_t)r * 5 + k];
+        float y[3];
+        ok = tc_forward(sm, tmem, t, d[0], d[1], y, &phase);
+        if (ok && r < n)
+            for (int k = 0; k < 3; ++k) {
+                const double df = (double)__saturatef(y[k]) - (double)d[2 + k];
+                se += df * df;
+            }
+    }
+    for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xFFFFFFFFu, se, o);
+    if ((t & 31u) == 0) s_part[t >> 5] = se;
+    __syncthreads();
+    if (t == 0) {
+        se = 0.0;
+        for (uint32_t k = 0; k < TC_ROWS / 32; ++k) se += s_part[k];
+        sum[blockIdx.y * gridDim.x + blockIdx.x] = ok ? se : __longlong_as_double(0x7FF8000000000000ll);
+        if (!ok && err) atomicOr(err, ERR_TIMEOUT);
     }
     tc_teardown(tmem);
 }
@@ -933,6 +975,22 @@ cudaError_t launch_mlp_train(float* theta, float* adam_m, float* adam_v, float* 
     cudaError_t e = cudaFuncSetAttribute(k_mlp_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)St::end);
     if (e != cudaSuccess) return e;
     k_mlp_train_tc<<<dim3(splits, n_mats), TR_T, St::end, s>>>(A);
+    return cudaGetLastError();
+}
+
+// The partial sums go to sum[n_nets][*n_part]; the caller provides room for
+// mlp_validate_parts(n_nets, n, num_sms) of them per network.
+uint32_t mlp_validate_parts(uint32_t n_nets, uint32_t n, int num_sms) {
+    const uint32_t tiles = (n + TC_ROWS - 1) / TC_ROWS, room = (uint32_t)num_sms * TC_CTAS_PER_SM / n_nets;
+    return std::max(1u, std::min(tiles, room));
+}
+
+cudaError_t launch_mlp_validate(const float* theta, const float* data, uint32_t n_nets, uint32_t n, double* sum,
+                                uint32_t* err, int num_sms, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_validate_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sm::end);
+    if (e != cudaSuccess) return e;
+    k_mlp_validate_tc<<<dim3(mlp_validate_parts(n_nets, n, num_sms), n_nets), TC_ROWS, Sm::end, s>>>(theta, data, n, sum,
+                                                                                                 err);
     return cudaGetLastError();
 }
 

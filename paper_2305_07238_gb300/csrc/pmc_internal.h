@@ -275,6 +275,10 @@ cudaError_t launch_mlp_train(float* theta, float* adam_m, float* adam_v, float* 
 // Tensor-core (tcgen05) inference (mlp_tc.cu); err may be null.
 cudaError_t launch_mlp_forward_tc(const float* theta, const float* u, const float* v, uint32_t n, float* out, int clamp,
                                   uint32_t* err, int num_sms, cudaStream_t s);
+// Squared errors of n_nets networks over their n validation rows, in partial sums per network.
+uint32_t mlp_validate_parts(uint32_t n_nets, uint32_t n, int num_sms);
+cudaError_t launch_mlp_validate(const float* theta, const float* data, uint32_t n_nets, uint32_t n, double* sum,
+                                uint32_t* err, int num_sms, cudaStream_t s);
 cudaError_t launch_root_samples(const uint4* prog, const float* params, const RootInfo* rinfo, const uint32_t* groots,
                                 uint32_t n_train_mats, uint32_t n_rows, uint64_t seed, float* data, uint32_t max_slots,
                                 int num_sms, cudaStream_t s);
