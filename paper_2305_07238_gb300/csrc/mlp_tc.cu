@@ -8,7 +8,12 @@
 //   layer 1: D1[128x64] = G[128x64] W1      (G: features, K = 64 in four K = 16 steps)
 //   layer 2: D2[128x64] = relu(D1 + b1) W2
 //   layer 3: D3[128x16] = relu(D2 + b2) W3  (outputs 0..2 used, W3 padded to 16 columns)
-// Operands live in shared memory in the no-swizzle K-major layout: 8x8 BF16 "core
+// The activations (operand A) live in tensor memory as BF16 pairs, 32 columns a row: a thread
+// writes its own row with tcgen05.st, and no shared memory is written or read for them.  (With
+// A in shared memory the products were bound by its bandwidth: 4 KB of A for 2 KB of B per
+// K = 16 step, and the tensor pipe was busy 54 % of the time at 23 % of the BF16 rate; a call
+// over 2^20 points took 43.0 us, and 33.2 us now.)  The
+// weights (operand B) live in shared memory in the no-swizzle K-major layout: 8x8 BF16 "core
 // matrices" of 128 contiguous bytes, core matrices adjacent along K 128 B apart (leading
 // byte offset) and 8-row groups 1024 B apart (stride byte offset).  The network and
 // its BF16 rounding points are those of mlp.cu (features, weights and hidden
@@ -27,30 +32,37 @@ namespace {
 
 constexpr int P_W1 = 0, P_B1 = 4096, P_W2 = 4160, P_B2 = 8256, P_W3 = 8320, P_B3 = 8512;
 constexpr uint32_t TC_ROWS = 128;
-constexpr uint32_t TC_COLS = 64;                // tensor-memory columns: D1, D2 and D3 all at column 0
-constexpr uint32_t TC_CTAS_PER_SM = 6;          // resident inference CTAs (shared memory and TMEM allow 6)
+// tensor-memory columns of a CTA, allocated in this order: D1, D2 and D3 in turn, then the
+// activations
+constexpr uint32_t TC_COLS = 64, TC_ACOLS = 32;
+// Resident inference CTAs per SM: five have their 96 columns among the SM's 512.  Their shared
+// memory is asked for in a size of which five fit and six do not, so that a sixth never waits
+// for columns while it holds some: with at most five holders of 64, the 32 each needs then
+// are always there.
+constexpr uint32_t TC_CTAS_PER_SM = 5;
+constexpr uint32_t TC_SMEM = 40 * 1024;
 constexpr uint32_t WAIT_POLLS = 1u << 22;       // bound of every mbarrier wait
 
 // One activation operand serves the three layers: a layer's epilogue overwrites it only after
 // the product that read it has completed (the mbarrier wait), and likewise one 64-column
-// accumulator, read out completely before the next product is issued.  35 KB of shared
-// memory and 64 TMEM columns per CTA let six CTAs share an SM.
+// accumulator, read out completely before the next product is issued.
 struct Sm {                                     // byte offsets into dynamic shared memory
-    static constexpr uint32_t a0 = 0;           // 128 x 64 BF16: features, then layer-1, then layer-2 output
-    static constexpr uint32_t w1 = 16384;       // 64 x 64 BF16: W1 transposed (n rows, k columns)
-    static constexpr uint32_t w2 = 24576;       // 64 x 64 BF16: W2 transposed
-    static constexpr uint32_t w3 = 32768;       // 16 x 64 BF16: W3 transposed, rows 3..15 zero
-    static constexpr uint32_t bias = 34816;     // b1[64], b2[64], b3[4] FP32
-    static constexpr uint32_t mbar = 35344;     // 8-byte mbarrier of the products
-    static constexpr uint32_t mbar_w = 35352;   // 8-byte mbarrier of the operand-image copy
-    static constexpr uint32_t tmem = 35360;     // tensor-memory base written by tcgen05.alloc
-    static constexpr uint32_t end = 35368;
+    static constexpr uint32_t w1 = 0;           // 64 x 64 BF16: W1 transposed (n rows, k columns)
+    static constexpr uint32_t w2 = 8192;        // 64 x 64 BF16: W2 transposed
+    static constexpr uint32_t w3 = 16384;       // 16 x 64 BF16: W3 transposed, rows 3..15 zero
+    static constexpr uint32_t bias = 18432;     // b1[64], b2[64], b3[4] FP32
+    static constexpr uint32_t mbar = 18960;     // 8-byte mbarrier of the products
+    static constexpr uint32_t mbar_w = 18968;   // 8-byte mbarrier of the operand-image copy
+    static constexpr uint32_t tmem = 18976;     // tensor-memory bases written by tcgen05.alloc: D, A
+    static constexpr uint32_t end = 18984;
 };
 // the operand image of a network is shared memory [w1, bias end), in that layout
 static_assert(Sm::bias + 132 * 4 - Sm::w1 == SURR_IMG_BYTES, "operand image = weights and biases of Sm");
 static_assert(Sm::w1 % 16 == 0, "bulk copies land on 16-byte boundaries");
-static_assert(TC_CTAS_PER_SM * (Sm::end + 1024) <= 228 * 1024, "inference CTAs per SM by shared memory");
-static_assert(TC_CTAS_PER_SM * TC_COLS <= 512, "inference CTAs per SM by tensor memory");
+static_assert(Sm::end <= TC_SMEM, "inference shared memory");
+static_assert(TC_CTAS_PER_SM * (TC_SMEM + 1024) <= 228 * 1024 && (TC_CTAS_PER_SM + 1) * (TC_SMEM + 1024) > 228 * 1024,
+              "exactly TC_CTAS_PER_SM inference CTAs fit an SM's shared memory");
+static_assert(TC_CTAS_PER_SM * (TC_COLS + TC_ACOLS) <= 512, "inference CTAs per SM by tensor memory");
 
 // Byte offset of element (r, c) of a 64-column operand in the core-matrix layout.
 __device__ __forceinline__ uint32_t cm_off(uint32_t r, uint32_t c) {
@@ -82,6 +94,14 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
         "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
         "l"(a), "l"(b), "r"(id), "r"(acc));
+}
+
+// The same with operand A in tensor memory (lane = row, one 32-bit column per pair along K).
+__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t id, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b), "r"(id), "r"(acc));
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
@@ -130,6 +150,33 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = __uint_as_float(r[k]);
 }
+
+// 32 consecutive accumulator columns of this thread's lane.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int k = 0; k < 32; ++k) v[k] = __uint_as_float(r[k]);
+}
+
+// Sixteen words into consecutive columns of this thread's lane (complete only after tmem_st_wait).
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};\n" ::"r"(r[0]),
+        "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+        "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -207,19 +254,20 @@ __device__ __forceinline__ uint32_t pack2_relu(float lo, float hi) {
     return r;
 }
 
-// Row t of the feature matrix: [sin pi k u, cos pi k u, sin pi k v, cos pi k v], k = 1..16.
-// sincospif gives the anchors k = 1 and k = 9 of both coordinates; from each anchor, seven
-// steps of the angle-addition formulas
+// Row t of the feature matrix: [sin pi k u, cos pi k u, sin pi k v, cos pi k v], k = 1..16, into
+// the 32 activation columns of this thread's lane.  sincospif gives the anchors k = 1 and k = 9
+// of both coordinates; from each anchor, seven steps of the angle-addition formulas
 //   sin(a + b) = sin a cos b + cos a sin b,  cos(a + b) = cos a cos b - sin a sin b
 // with b = pi x give the next seven frequencies.  Every quantity is a (u, v) pair, so one
 // packed instruction steps both coordinates.  A step adds about an ulp of error, so every
 // feature is within a few ulps of sincospif's, far below the BF16 rounding the features
 // then take.  The features are packed to BF16 as soon as two neighbours exist.
-__device__ __forceinline__ void tc_features(unsigned char* sm, uint32_t t, float u, float v) {
+__device__ __forceinline__ void tc_features(uint32_t lane_a, float u, float v) {
     float s1u, c1u, s1v, c1v;
     sincospif(u, &s1u, &c1u);
     sincospif(v, &s1v, &c1v);
     const float2 S1 = f2(s1u, s1v), C1 = f2(c1u, c1v), nS1 = f2(-s1u, -s1v);
+    uint32_t wu[16], wv[16];   // words of u: eight of sin, eight of cos; and of v
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
         float2 sk, ck;
@@ -233,96 +281,99 @@ __device__ __forceinline__ void tc_features(unsigned char* sm, uint32_t t, float
             sk = f2(su, sv);
             ck = f2(cu, cv);
         }
-        uint32_t wsu[4], wcu[4], wsv[4], wcv[4];
 #pragma unroll
         for (int j = 0; j < 8; j += 2) {
             const float2 sn = fma2(sk, C1, mul2(ck, S1));
             const float2 cn = fma2(ck, C1, mul2(sk, nS1));
-            wsu[j / 2] = pack2(sk.x, sn.x);
-            wcu[j / 2] = pack2(ck.x, cn.x);
-            wsv[j / 2] = pack2(sk.y, sn.y);
-            wcv[j / 2] = pack2(ck.y, cn.y);
+            wu[4 * half + j / 2] = pack2(sk.x, sn.x);
+            wu[8 + 4 * half + j / 2] = pack2(ck.x, cn.x);
+            wv[4 * half + j / 2] = pack2(sk.y, sn.y);
+            wv[8 + 4 * half + j / 2] = pack2(ck.y, cn.y);
             if (j < 6) {
                 sk = fma2(sn, C1, mul2(cn, S1));
                 ck = fma2(cn, C1, mul2(sn, nS1));
             }
         }
-        const uint32_t k0 = 8u * half;   // first frequency of this anchor, minus one
-        *reinterpret_cast<uint4*>(sm + Sm::a0 + cm_off(t, k0)) = make_uint4(wsu[0], wsu[1], wsu[2], wsu[3]);
-        *reinterpret_cast<uint4*>(sm + Sm::a0 + cm_off(t, 16 + k0)) = make_uint4(wcu[0], wcu[1], wcu[2], wcu[3]);
-        *reinterpret_cast<uint4*>(sm + Sm::a0 + cm_off(t, 32 + k0)) = make_uint4(wsv[0], wsv[1], wsv[2], wsv[3]);
-        *reinterpret_cast<uint4*>(sm + Sm::a0 + cm_off(t, 48 + k0)) = make_uint4(wcv[0], wcv[1], wcv[2], wcv[3]);
     }
+    tmem_st16(lane_a, wu);
+    tmem_st16(lane_a + 16, wv);
+    tmem_st_wait();
 }
 
-// relu(acc + bias) of 64 accumulator columns -> row t of a BF16 operand.
-__device__ __forceinline__ void tc_hidden(unsigned char* sm, uint32_t dst, uint32_t taddr, const float* bias,
-                                          uint32_t t) {
+// relu(acc + bias) of 64 accumulator columns -> this thread's row of the activations.
+__device__ __forceinline__ void tc_hidden(uint32_t lane_a, uint32_t lane_d, const float* bias) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        float v[16];
-        tmem_ld16(taddr + 16u * q, v);
-        uint32_t p[8];
+    for (int h = 0; h < 2; ++h) {
+        float v[32];
+        tmem_ld32(lane_d + 32u * h, v);
+        uint32_t p[16];
 #pragma unroll
-        for (int k = 0; k < 8; k += 2) {
-            const float4 b = *reinterpret_cast<const float4*>(bias + 16 * q + 2 * k);
+        for (int k = 0; k < 16; k += 2) {
+            const float4 b = *reinterpret_cast<const float4*>(bias + 32 * h + 2 * k);
             const float2 x0 = add2(f2(v[2 * k], v[2 * k + 1]), f2(b.x, b.y));
             const float2 x1 = add2(f2(v[2 * k + 2], v[2 * k + 3]), f2(b.z, b.w));
             p[k] = pack2_relu(x0.x, x0.y);
             p[k + 1] = pack2_relu(x1.x, x1.y);
         }
-        *reinterpret_cast<uint4*>(sm + dst + cm_off(t, 16 * q)) = make_uint4(p[0], p[1], p[2], p[3]);
-        *reinterpret_cast<uint4*>(sm + dst + cm_off(t, 16 * q + 8)) = make_uint4(p[4], p[5], p[6], p[7]);
+        tmem_st16(lane_a + 16u * h, p);
     }
+    tmem_st_wait();
 }
 
 // Issues the four K = 16 steps of one layer (one thread).
-__device__ __forceinline__ void tc_layer(uint32_t d_tmem, uint32_t a_saddr, uint32_t b_saddr, uint32_t id) {
+__device__ __forceinline__ void tc_layer(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_saddr, uint32_t id) {
 #pragma unroll
-    for (uint32_t s = 0; s < 4; ++s) mma_bf16(d_tmem, sdesc(a_saddr + 256u * s), sdesc(b_saddr + 256u * s), id, s > 0);
+    for (uint32_t s = 0; s < 4; ++s) mma_bf16_ta(d_tmem, a_tmem + 8u * s, sdesc(b_saddr + 256u * s), id, s > 0);
 }
 
-// The network for this CTA's 128 rows (row t = this thread's point); y = raw outputs.
-// Every thread returns the same value: false if a wait for the tensor cores ran out.
-__device__ bool tc_forward(unsigned char* sm, uint32_t tmem, uint32_t t, float u, float v, float (&y)[3],
-                           uint32_t* phase) {
+struct TcTmem {
+    uint32_t d, a;   // first columns of the accumulator and of the activations
+};
+
+// The network for this CTA's 128 rows (row t = this thread's point); y = raw outputs.  *ok is
+// cleared if this thread's wait for the tensor cores ran out; every thread returns the same
+// value: false if any thread's *ok was cleared in an earlier call.
+__device__ __forceinline__ bool tc_forward(unsigned char* sm, TcTmem tm, uint32_t t, float u, float v, float (&y)[3],
+                                           uint32_t* phase, bool* ok) {
     const uint32_t base = smem_u32(sm), mbar = base + Sm::mbar;
-    const uint32_t lane_addr = tmem + (((t >> 5) * 32u) << 16);
+    const uint32_t lane = ((t >> 5) * 32u) << 16;
+    const uint32_t lane_d = tm.d + lane, lane_a = tm.a + lane;
     const float* bias = reinterpret_cast<const float*>(sm + Sm::bias);
-    tc_features(sm, t, u, v);
-    const uint32_t a0 = base + Sm::a0;
+    tc_features(lane_a, u, v);
     const uint32_t srcB[3] = {base + Sm::w1, base + Sm::w2, base + Sm::w3};
     const uint32_t ids[3] = {idesc(128, 64), idesc(128, 64), idesc(128, 16)};
 #pragma unroll
     for (int layer = 0; layer < 3; ++layer) {
-        // the operand rows written by every thread become visible to the tensor cores
-        fence_async_smem();
+        // the rows written by every thread, and its reads of the accumulator, come before the
+        // product; the first barrier of a call also brings the threads' waits together
         fence_before();
-        __syncthreads();
+        if (layer == 0) {
+            if (__syncthreads_or(!*ok)) return false;
+        } else {
+            __syncthreads();
+        }
         if (t == 0) {
             fence_after();
-            tc_layer(tmem, a0, srcB[layer], ids[layer]);
+            tc_layer(tm.d, tm.a, srcB[layer], ids[layer]);
             mma_commit(mbar);
         }
-        const bool done = mbar_wait(mbar, *phase);
+        *ok &= mbar_wait(mbar, *phase);
         *phase ^= 1u;
-        if (__syncthreads_or(!done)) return false;
         fence_after();
-        if (layer == 0) tc_hidden(sm, Sm::a0, lane_addr, bias, t);
-        else if (layer == 1) tc_hidden(sm, Sm::a0, lane_addr, bias + 64, t);
+        if (layer == 0) tc_hidden(lane_a, lane_d, bias);
+        else if (layer == 1) tc_hidden(lane_a, lane_d, bias + 64);
         else {
             float o[4];
-            tmem_ld4(lane_addr + 0u, o);
+            tmem_ld4(lane_d, o);
             y[0] = o[0] + bias[128];
             y[1] = o[1] + bias[129];
             y[2] = o[2] + bias[130];
         }
-        fence_before();
     }
     return true;
 }
 
-__device__ __forceinline__ uint32_t tc_setup(unsigned char* sm) {
+__device__ __forceinline__ TcTmem tc_setup(unsigned char* sm) {
     const uint32_t base = smem_u32(sm);
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(base + Sm::mbar));
@@ -332,56 +383,70 @@ __device__ __forceinline__ uint32_t tc_setup(unsigned char* sm) {
     if (threadIdx.x < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + Sm::tmem),
                      "r"(TC_COLS));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + Sm::tmem + 4),
+                     "r"(TC_ACOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     fence_before();
     __syncthreads();
     fence_after();
-    return *reinterpret_cast<volatile uint32_t*>(sm + Sm::tmem);
+    const volatile uint32_t* p = reinterpret_cast<volatile uint32_t*>(sm + Sm::tmem);
+    return TcTmem{p[0], p[1]};
 }
 
-__device__ __forceinline__ void tc_teardown(uint32_t tmem) {
+__device__ __forceinline__ void tc_teardown(TcTmem tm) {
     fence_before();
     __syncthreads();
-    if (threadIdx.x < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_COLS));
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm.d), "r"(TC_COLS));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm.a), "r"(TC_ACOLS));
+    }
 }
 
-// Stand-alone network over n points (planar 3 x n output).
-__global__ void __launch_bounds__(TC_ROWS) k_mlp_forward_tc(const float* __restrict__ theta, const float* __restrict__ u,
-                                                            const float* __restrict__ v, uint32_t n, float* out,
-                                                            int clamp, uint32_t* err) {
+// The operands written to shared memory by every thread (tc_load_weights) before the first product.
+__device__ __forceinline__ void tc_weights_ready() {
+    fence_async_smem();
+    __syncthreads();
+}
+
+// Stand-alone network over n points (planar 3 x n output).  A CTA whose wait for the tensor
+// cores ran out gives NaN for the rows of that tile and every later one of its own.
+__global__ void __launch_bounds__(TC_ROWS, TC_CTAS_PER_SM) k_mlp_forward_tc(const float* __restrict__ theta,
+                                                                            const float* __restrict__ u,
+                                                                            const float* __restrict__ v, uint32_t n,
+                                                                            float* out, int clamp, uint32_t* err) {
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t t = threadIdx.x;
-    const uint32_t tmem = tc_setup(sm);
+    const TcTmem tmem = tc_setup(sm);
     tc_load_weights(sm, theta);
+    tc_weights_ready();
     uint32_t phase = 0;
     bool ok = true;
     const uint32_t tiles = (n + TC_ROWS - 1) / TC_ROWS;
     // each tile's (u, v) is loaded while the previous tile runs through the network
     uint32_t r = blockIdx.x * TC_ROWS + t;
     float uu = r < n ? u[r] : 0.0f, vv = r < n ? v[r] : 0.0f;
-    for (uint32_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+    uint32_t tile = blockIdx.x;
+    for (; tile < tiles; tile += gridDim.x) {
         const uint32_t rn = r + gridDim.x * TC_ROWS;
         const float un = rn < n ? u[rn] : 0.0f, vn = rn < n ? v[rn] : 0.0f;
         float y[3];
-        ok = tc_forward(sm, tmem, t, uu, vv, y, &phase);
-        if (ok && r < n) {
+        if (!tc_forward(sm, tmem, t, uu, vv, y, &phase, &ok)) break;   // uniform
+        if (r < n) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) out[(size_t)k * n + r] = clamp ? __saturatef(y[k]) : y[k];
+            for (int k = 0; k < 3; ++k)
+                out[(size_t)k * n + r] = !ok ? __int_as_float(0x7FC00000) : clamp ? __saturatef(y[k]) : y[k];
         }
         r = rn;
         uu = un;
         vv = vn;
     }
-    if (!ok) {
-        // a wait for the tensor cores ran out: this CTA's remaining rows read NaN
-        for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-            const uint32_t r = tile * TC_ROWS + t;
-            if (r < n)
-                for (int k = 0; k < 3; ++k) out[(size_t)k * n + r] = __int_as_float(0x7FC00000);
-        }
-        if (err && t == 0) atomicOr(err, ERR_TIMEOUT);
+    for (; tile < tiles; tile += gridDim.x) {   // after a wait that ran out
+        r = tile * TC_ROWS + t;
+        if (r < n)
+            for (int k = 0; k < 3; ++k) out[(size_t)k * n + r] = __int_as_float(0x7FC00000);
     }
+    if (!ok && err) atomicOr(err, ERR_TIMEOUT);
     tc_teardown(tmem);
 }
 
@@ -389,30 +454,35 @@ __global__ void __launch_bounds__(TC_ROWS) k_mlp_forward_tc(const float* __restr
 // run network y over its n rows (u, v, r, g, b) in tiles of 128 and sum the squared errors
 // of the clamped outputs in FP64, one partial sum per CTA (added up by the host in a fixed
 // order; NaN if a wait for the tensor cores ran out).
-__global__ void __launch_bounds__(TC_ROWS) k_mlp_validate_tc(const float* __restrict__ theta,
-                                                             const float* __restrict__ data, uint32_t n, double* sum,
-                                                             uint32_t* err) {
+__global__ void __launch_bounds__(TC_ROWS, TC_CTAS_PER_SM) k_mlp_validate_tc(const float* __restrict__ theta,
+                                                                             const float* __restrict__ data, uint32_t n,
+                                                                             double* sum, uint32_t* err) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ double s_part[TC_ROWS / 32];
     const uint32_t t = threadIdx.x;
-    const uint32_t tmem = tc_setup(sm);
+    const TcTmem tmem = tc_setup(sm);
     tc_load_weights(sm, theta + (size_t)blockIdx.y * MLP_PARAMS);
+    tc_weights_ready();
     const float* rows = data + (size_t)blockIdx.y * n * 5;
     uint32_t phase = 0;
     bool ok = true;
     double se = 0.0;
-    for (uint32_t r0 = blockIdx.x * TC_ROWS; r0 < n && ok; r0 += gridDim.x * TC_ROWS) {
+    for (uint32_t r0 = blockIdx.x * TC_ROWS; r0 < n; r0 += gridDim.x * TC_ROWS) {
         const uint32_t r = r0 + t;
         float d[5] = {};
         if (r < n)
             for (int k = 0; k < 5; ++k) d[k] = rows[(size_t)r * 5 + k];
         float y[3];
-        ok = tc_forward(sm, tmem, t, d[0], d[1], y, &phase);
-        if (ok && r < n)
+        if (!tc_forward(sm, tmem, t, d[0], d[1], y, &phase, &ok)) break;   // uniform
+        if (r < n)
             for (int k = 0; k < 3; ++k) {
                 const double df = (double)__saturatef(y[k]) - (double)d[2 + k];
                 se += df * df;
             }
+    }
+    if (!ok) {
+        se = __longlong_as_double(0x7FF8000000000000ll);
+        if (err) atomicOr(err, ERR_TIMEOUT);
     }
     for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xFFFFFFFFu, se, o);
     if ((t & 31u) == 0) s_part[t >> 5] = se;
@@ -420,8 +490,7 @@ __global__ void __launch_bounds__(TC_ROWS) k_mlp_validate_tc(const float* __rest
     if (t == 0) {
         se = 0.0;
         for (uint32_t k = 0; k < TC_ROWS / 32; ++k) se += s_part[k];
-        sum[blockIdx.y * gridDim.x + blockIdx.x] = ok ? se : __longlong_as_double(0x7FF8000000000000ll);
-        if (!ok && err) atomicOr(err, ERR_TIMEOUT);
+        sum[blockIdx.y * gridDim.x + blockIdx.x] = se;
     }
     tc_teardown(tmem);
 }
@@ -429,10 +498,10 @@ __global__ void __launch_bounds__(TC_ROWS) k_mlp_validate_tc(const float* __rest
 // In-pass inference: contiguous ranges of 128-point items (grouped points of a material
 // whose cacheable node has a surrogate); the node's value goes into the points' probe
 // records as a value computed this pass.
-__global__ void __launch_bounds__(TC_ROWS) k_surrogate_tc(BatchArgs a) {
+__global__ void __launch_bounds__(TC_ROWS, TC_CTAS_PER_SM) k_surrogate_tc(BatchArgs a) {
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t t = threadIdx.x;
-    const uint32_t tmem = tc_setup(sm);
+    const TcTmem tmem = tc_setup(sm);
     const uint32_t n_items = a.ctl->n_surr_items;
     const uint32_t per = (n_items + gridDim.x - 1) / gridDim.x;
     const uint32_t i_end = min(n_items, (blockIdx.x + 1) * per);
@@ -444,7 +513,7 @@ __global__ void __launch_bounds__(TC_ROWS) k_surrogate_tc(BatchArgs a) {
     uint32_t m = 0, next_base = 0, ibase = 0, cnt = 0, s0 = 0, pre_item = 0xFFFFFFFFu;
     float uu = 0.0f, vv = 0.0f;
     size_t rbase = 0;   // the first probe record of the node's column in material m
-    for (uint32_t item = blockIdx.x * per; item < i_end && ok; ++item) {
+    for (uint32_t item = blockIdx.x * per; item < i_end; ++item) {
         if (item >= next_base) {
             uint32_t lo = 0, hi = a.n_mats;
             while (hi - lo > 1) {
@@ -468,6 +537,7 @@ __global__ void __launch_bounds__(TC_ROWS) k_surrogate_tc(BatchArgs a) {
                 }
             } else {
                 tc_load_weights(sm, a.surr_theta + (size_t)a.surr_slot[m] * MLP_PARAMS);
+                tc_weights_ready();
             }
             loaded = m;
         }
@@ -482,7 +552,7 @@ __global__ void __launch_bounds__(TC_ROWS) k_surrogate_tc(BatchArgs a) {
         const float un = (pre && jn < cnt) ? a.su[s0 + jn] : 0.0f, vn = (pre && jn < cnt) ? a.sv[s0 + jn] : 0.0f;
         pre_item = pre ? item + 1 : 0xFFFFFFFFu;
         float y[3];
-        ok = tc_forward(sm, tmem, t, uu, vv, y, &phase);
+        if (!tc_forward(sm, tmem, t, uu, vv, y, &phase, &ok)) break;   // uniform
         if (ok && j < cnt) {
             const size_t rec = rbase + j;
             a.probes[rec] = make_float4(__saturatef(y[0]), __saturatef(y[1]), __saturatef(y[2]), __uint_as_float(3u));
@@ -491,7 +561,7 @@ __global__ void __launch_bounds__(TC_ROWS) k_surrogate_tc(BatchArgs a) {
         uu = un;
         vv = vn;
     }
-    if (!ok && t == 0) atomicOr(&a.ctl->err, ERR_TIMEOUT);
+    if (!ok) atomicOr(&a.ctl->err, ERR_TIMEOUT);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) n_eval += __shfl_xor_sync(0xFFFFFFFFu, n_eval, o);
     if ((t & 31u) == 0 && n_eval) atomicAdd(&a.stats[ST_SURR], n_eval);
@@ -987,18 +1057,17 @@ uint32_t mlp_validate_parts(uint32_t n_nets, uint32_t n, int num_sms) {
 
 cudaError_t launch_mlp_validate(const float* theta, const float* data, uint32_t n_nets, uint32_t n, double* sum,
                                 uint32_t* err, int num_sms, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_validate_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sm::end);
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_validate_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
     if (e != cudaSuccess) return e;
-    k_mlp_validate_tc<<<dim3(mlp_validate_parts(n_nets, n, num_sms), n_nets), TC_ROWS, Sm::end, s>>>(theta, data, n, sum,
+    k_mlp_validate_tc<<<dim3(mlp_validate_parts(n_nets, n, num_sms), n_nets), TC_ROWS, TC_SMEM, s>>>(theta, data, n, sum,
                                                                                                  err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_surrogate(const BatchArgs& a, int num_sms, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_surrogate_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sm::end);
+    cudaError_t e = cudaFuncSetAttribute(k_surrogate_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
     if (e != cudaSuccess) return e;
-    // six CTAs per SM: their tensor-memory allocations (6 x 64 columns) fit the SM's 512
-    k_surrogate_tc<<<num_sms * TC_CTAS_PER_SM, TC_ROWS, Sm::end, s>>>(a);
+    k_surrogate_tc<<<num_sms * TC_CTAS_PER_SM, TC_ROWS, TC_SMEM, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1014,9 +1083,9 @@ cudaError_t launch_mlp_forward_tc(const float* theta, const float* u, const floa
     const uint32_t full = (uint32_t)num_sms * TC_CTAS_PER_SM;
     uint32_t blocks = tiles < full ? tiles : full;
     if (blocks == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sm::end);
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
     if (e != cudaSuccess) return e;
-    k_mlp_forward_tc<<<blocks, TC_ROWS, Sm::end, s>>>(theta, u, v, n, out, clamp, err);
+    k_mlp_forward_tc<<<blocks, TC_ROWS, TC_SMEM, s>>>(theta, u, v, n, out, clamp, err);
     return cudaGetLastError();
 }
 
