@@ -1,6 +1,7 @@
 // cache_impl.h -- the library's definition of the opaque pmc_cache object.
 #pragma once
 
+#include <algorithm>
 #include <vector>
 
 #include "pmc_internal.h"
@@ -47,7 +48,6 @@ struct pmc_cache {
     uint32_t* d_miss_cnt = nullptr;       // roots + MAX_LEVELS
     uint32_t* d_root_items = nullptr;     // roots + 1, then MAX_LEVELS + 1 level item starts
     uint32_t* d_root_order = nullptr;     // roots by ascending level, then MAX_LEVELS + 1 starts
-    uint32_t n_bins = 0;                  // cell-grouped insert bins
     bool table_empty = true;              // nothing inserted since creation or reset
     bool last_all_miss = false;           // the last batch ran on an empty table
     bool last_unsorted = false;           // the last batch kept no probe records
@@ -65,7 +65,7 @@ struct pmc_cache {
     uint32_t* d_surr_items = nullptr;     // n_mats + 1
     bool any_surr_on = false;
     bool all_roots_surr = false;   // every material's cacheable nodes are all surrogates' (>= one)
-    uint32_t* d_bins = nullptr;           // counts (n_bins) | bases (n_bins + 1)
+    uint32_t* d_bins = nullptr;           // counts (n_bins) | bases (n_bins + 1) | list (n_bins)
     // per-batch scratch, grown on demand
     uint64_t cap_points = 0;
     uint64_t cap_probes = 0;
@@ -109,4 +109,15 @@ struct pmc_cache {
 inline bool insert_lists(const pmc_cache* c) {
     return c->use_cache && c->desc.n_entries <= 8 &&
            !(c->desc.flags & (PMC_INSERT_ROUNDS | PMC_ALG1 | PMC_REPLACE_VISIBILITY)) && !c->insert_binned;
+}
+
+// The bins of the cell-grouped insert for the batch in *a (n and probe_cap set).
+inline void set_bins(const pmc_cache* c, pmc::BatchArgs* a) {
+    const uint64_t cells = c->use_cache ? c->desc.n_cells : 0;
+    const uint64_t probes = std::min<uint64_t>((uint64_t)a->n * c->max_roots, a->probe_cap);
+    a->bin_shift = pmc::insert_bin_shift(cells, probes);
+    a->n_bins = pmc::insert_bins(cells, a->bin_shift);
+    a->bin_cnt = c->d_bins;
+    a->bin_base = c->d_bins + a->n_bins;
+    a->bin_list = c->d_bins + 2 * (size_t)a->n_bins + 1;
 }

@@ -353,7 +353,6 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
     pmc_status s = PMC_OK;
     const uint64_t slots = c->use_cache ? desc->n_cells * desc->n_entries : 0;
     const uint64_t cells = c->use_cache ? desc->n_cells : 0;
-    c->n_bins = c->use_cache ? (uint32_t)((desc->n_cells + INSERT_BIN_CELLS - 1) / INSERT_BIN_CELLS) : 0;
     if ((s = dalloc(&c->d_mats, n_mats)) != PMC_OK ||
         (s = dalloc(&c->d_prog, prog.size())) != PMC_OK ||
         (s = dalloc(&c->d_params, params.size())) != PMC_OK ||
@@ -368,7 +367,7 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
         (s = dalloc(&c->d_miss_cnt, c->root_info.size() + MAX_LEVELS)) != PMC_OK ||
         (s = dalloc(&c->d_root_items, c->root_info.size() + 1 + MAX_LEVELS + 1)) != PMC_OK ||
         (s = dalloc(&c->d_root_order, c->root_info.size() + MAX_LEVELS + 1)) != PMC_OK ||
-        (s = dalloc(&c->d_bins, 3 * (size_t)c->n_bins + 1)) != PMC_OK ||
+        (s = dalloc(&c->d_bins, 3 * (size_t)(c->use_cache ? insert_bins_max(desc->n_cells) : 0) + 1)) != PMC_OK ||
         (s = dalloc(&c->d_surr_slot, n_mats)) != PMC_OK ||
         (s = dalloc(&c->d_surr_ord, n_mats)) != PMC_OK ||
         (s = dalloc(&c->d_surr_items, (size_t)n_mats + 1)) != PMC_OK) {
@@ -487,8 +486,7 @@ pmc_status enqueue_batch(pmc_cache* c, const pmc_points* pts, float* out_rgb, ui
     a.ctl = c->d_ctl; a.stats = c->d_stats;
     a.split = c->use_cache && c->split;
     a.insert_rounds = (c->desc.flags & PMC_INSERT_ROUNDS) ? 1 : 0;
-    a.n_bins = c->n_bins; a.bin_cnt = c->d_bins; a.bin_base = c->d_bins + c->n_bins;
-    a.bin_list = c->d_bins + 2 * (size_t)c->n_bins + 1;
+    set_bins(c, &a);
     a.cands_binned = c->d_cands_binned;
     a.insert_lists = insert_lists(c) ? 1 : 0;
     a.chain_head = c->d_chain_head;

@@ -1593,10 +1593,10 @@ __global__ void __launch_bounds__(256) k_insert(BatchArgs a) {
 }
 
 // ---- cell-grouped insert: the same (point, node) order per cell, without rounds.
-// Candidates are partitioned into bins of INS_CELLS consecutive cells (count, scan,
+// Candidates are partitioned into bins of 2^bin_shift consecutive cells (count, scan,
 // scatter: coalesced), then one block per bin groups its candidates by cell in shared
 // memory and one thread per cell inserts that cell's candidates in ascending order.
-constexpr uint32_t INS_CELLS = INSERT_BIN_CELLS;   // cells per bin (a multiple of 256)
+constexpr uint32_t INS_CELLS = INSERT_BIN_CELLS;   // most cells per bin (a multiple of 256)
 constexpr uint32_t INS_SMEM_BINS = 8192;  // bins counted in shared memory by the partition
 constexpr uint32_t INS_WARP_MAX = 256;     // a bin with at most this many candidates: one warp
 constexpr uint32_t INS_MID = 2048;         // at most this many: one block, staged in one pass
@@ -1653,7 +1653,7 @@ __device__ __forceinline__ void insert_one(const BatchArgs& a, const Candidate& 
     }
 }
 
-__device__ __forceinline__ uint32_t bin_of(uint32_t cell) { return cell / INS_CELLS; }
+__device__ __forceinline__ uint32_t bin_of(const BatchArgs& a, uint32_t cell) { return cell >> a.bin_shift; }
 
 // Candidates per bin, counted from the compact cell array the evaluation wrote.
 __global__ void __launch_bounds__(256) k_bin_count(BatchArgs a) {
@@ -1677,7 +1677,7 @@ __global__ void __launch_bounds__(256) k_bin_count(BatchArgs a) {
         for (uint32_t k = 0; k < 4; ++k) c[k] = i0 + k * stride < n_in ? cc[i0 + k * stride] : 0u;
 #pragma unroll
         for (uint32_t k = 0; k < 4; ++k)
-            if (i0 + k * stride < n_in) atomicAdd(local ? &s_cnt[bin_of(c[k])] : &a.bin_cnt[bin_of(c[k])], 1u);
+            if (i0 + k * stride < n_in) atomicAdd(local ? &s_cnt[bin_of(a, c[k])] : &a.bin_cnt[bin_of(a, c[k])], 1u);
     }
     if (local) {
         __syncthreads();
@@ -1775,7 +1775,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter(BatchArgs a) {
             for (uint32_t k = 0; k < U; ++k) c[k] = i0 + k * T < hi ? cc[i0 + k * T] : 0u;
 #pragma unroll
             for (uint32_t k = 0; k < U; ++k)
-                if (i0 + k * T < hi) atomicAdd(&s_cnt[bin_of(c[k])], 1u);
+                if (i0 + k * T < hi) atomicAdd(&s_cnt[bin_of(a, c[k])], 1u);
         }
         __syncthreads();
         for (uint32_t b = threadIdx.x; b < nb; b += T)
@@ -1800,7 +1800,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter(BatchArgs a) {
         for (uint32_t k = 0; k < U; ++k) {
             const uint32_t i = i0 + k * T;
             if (i < hi) {
-                const uint32_t b = bin_of(c[k]);
+                const uint32_t b = bin_of(a, c[k]);
                 const uint32_t pos = atomicAdd(local ? &s_cnt[b] : &a.bin_cnt[b], 1u);
                 dst[2 * (size_t)pos] = x[k][0];
                 dst[2 * (size_t)pos + 1] = x[k][1];
@@ -2003,7 +2003,7 @@ __global__ void __launch_bounds__(INS_WARPS * 32, 6) k_bin_insert_warp(BatchArgs
     for (uint32_t x = blockIdx.x * INS_WARPS + w; x < n_list; x += gridDim.x * INS_WARPS) {
         const uint32_t bin = a.bin_list[x];
         const uint32_t lo = a.bin_base[bin], hi = a.bin_base[bin + 1];
-        const uint32_t c0 = bin * INS_CELLS;
+        const uint32_t c0 = bin << a.bin_shift;
 #pragma unroll
         for (uint32_t q = 0; q < 8; ++q) st.cnt[8 * lane + q] = 0;
         __syncwarp();
@@ -2160,7 +2160,7 @@ __global__ void __launch_bounds__(INS_MID_T, 4) k_bin_insert_mid(BatchArgs a) {
     for (uint32_t x = blockIdx.x; x < n_list; x += gridDim.x) {
         const uint32_t bin = a.bin_list[first + x];
         const uint32_t lo = a.bin_base[bin], hi = a.bin_base[bin + 1];
-        const uint32_t c0 = bin * INS_CELLS;
+        const uint32_t c0 = bin << a.bin_shift;
         s_cnt[t] = 0;
         __syncthreads();
         // ---- count per cell; each candidate's rank of arrival among its cell's
@@ -2405,7 +2405,7 @@ __global__ void __launch_bounds__(256, 6) k_bin_insert(BatchArgs a) {
     for (uint32_t x = blockIdx.x; x < n_list; x += gridDim.x) {
         const uint32_t bin = a.bin_list[first + x];
         const uint32_t lo = a.bin_base[bin], hi = a.bin_base[bin + 1];
-        const uint32_t c0 = bin * INS_CELLS;
+        const uint32_t c0 = bin << a.bin_shift;
         // ---- per-cell counts and their exclusive scan
         for (uint32_t k = t; k < INS_CELLS; k += T) s_cnt[k] = 0;
         __syncthreads();

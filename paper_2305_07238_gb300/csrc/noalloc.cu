@@ -148,8 +148,7 @@ extern "C" pmc_status pmc_eval_batch_noalloc(pmc_cache* c, const pmc_points* pts
     a.ctl = c->d_ctl; a.stats = c->d_stats;
     a.split = c->use_cache && c->split;
     a.insert_rounds = (c->desc.flags & PMC_INSERT_ROUNDS) ? 1 : 0;
-    a.n_bins = c->n_bins; a.bin_cnt = c->d_bins; a.bin_base = c->d_bins + c->n_bins;
-    a.bin_list = c->d_bins + 2 * (size_t)c->n_bins + 1;
+    set_bins(c, &a);
     a.cands_binned = reinterpret_cast<Candidate*>(base + OFF_BINNED);
     a.insert_lists = insert_lists(c) ? 1 : 0;
     a.chain_head = c->d_chain_head;

@@ -220,7 +220,8 @@ struct BatchArgs {
     uint32_t* surr_item_base;  // n_mats + 1 (computed by k_scan)
     int all_surr;              // 1: every cacheable node of every material is a surrogate's:
                                // no lookup, no batched misses, no insert
-    uint32_t n_bins;           // cell-grouped insert: ceil(n_cells / INSERT_BIN_CELLS) bins
+    uint32_t n_bins;           // cell-grouped insert: ceil(n_cells / 2^bin_shift) bins
+    uint32_t bin_shift;        // log2 of the cells per bin, at most log2(INSERT_BIN_CELLS)
     uint32_t* bin_cnt;         // n_bins
     uint32_t* bin_base;        // n_bins + 1
     uint32_t* bin_list;        // n_bins: the non-empty bins by resolving kernel (warp, block,
@@ -245,7 +246,30 @@ struct BatchArgs {
     uint8_t* slot_cls;
 };
 
-constexpr uint32_t INSERT_BIN_CELLS = 256;
+constexpr uint32_t INSERT_BIN_SHIFT = 8;
+constexpr uint32_t INSERT_BIN_CELLS = 1u << INSERT_BIN_SHIFT;   // most cells per bin
+constexpr uint32_t INSERT_SMALL_BINS = 8192;                    // most bins of fewer cells
+
+// Bins of the cell-grouped insert for a batch that can offer up to `probes` candidates.  A bin
+// is resolved fastest by a block that stages all of its candidates at once (up to 2048); larger
+// ones are re-read for every range of cells that fits.  So bins shrink below 256 cells while
+// a bin could get more than 1024 on average and their number stays within what one block
+// scans quickly and the partition counts in shared memory.  (403 k points x 6.3 cacheable nodes
+// on 65,536 cells: 256 bins of 256 cells take 412 us per pass, 4096 bins of 16 cells 131 us.)
+inline uint32_t insert_bin_shift(uint64_t n_cells, uint64_t probes) {
+    uint32_t s = INSERT_BIN_SHIFT;
+    while (s > 0 && (n_cells >> (s - 1)) < INSERT_SMALL_BINS && probes >> 10 > (n_cells >> s)) --s;
+    return s;
+}
+inline uint32_t insert_bins(uint64_t n_cells, uint32_t shift) {
+    return (uint32_t)((n_cells + (1ull << shift) - 1) >> shift);
+}
+// Bins to reserve room for, whatever the batch.
+inline uint32_t insert_bins_max(uint64_t n_cells) {
+    const uint64_t most = n_cells < INSERT_SMALL_BINS ? n_cells : INSERT_SMALL_BINS;
+    const uint32_t wide = insert_bins(n_cells, INSERT_BIN_SHIFT);
+    return wide > most ? wide : (uint32_t)most;
+}
 
 
 // Phases timed by the optional CUDA events of a batch.
