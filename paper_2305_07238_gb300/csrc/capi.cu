@@ -404,8 +404,8 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
     c->surr_on.assign(n_mats, 0);
     if (e == cudaSuccess) e = cudaMemset(c->d_surr_slot, 0xFF, n_mats * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(c->d_surr_ord, 0xFF, n_mats * sizeof(int32_t));
-    if (e == cudaSuccess) e = launch_reset(c->d_table, table_units(c), c->d_claims, c->d_chain_head, cells, c->d_ctl, c->d_stats, 0,
-                                           (desc->flags & PMC_INSERT_ROUNDS) != 0);
+    if (e == cudaSuccess) e = launch_reset(c->d_table, table_units(c), c->d_claims, c->d_chain_head, cells, c->d_ctl, c->d_stats,
+                                           c->num_sms, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         cuda_fail(nullptr, e);
@@ -833,7 +833,7 @@ pmc_status pmc_reset(pmc_cache* c, void* stream) {
     DeviceGuard g(c->desc.device);
     const uint64_t cells = c->use_cache ? c->desc.n_cells : 0;
     cudaError_t e = launch_reset(c->d_table, table_units(c), c->d_claims, c->d_chain_head, cells, c->d_ctl, c->d_stats,
-                                 (cudaStream_t)stream, (c->desc.flags & PMC_INSERT_ROUNDS) != 0);
+                                 c->num_sms, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(c, e);
     c->epoch_host = 0;
     c->table_empty = true;
@@ -1261,7 +1261,8 @@ pmc_status pmc_graph_create(pmc_cache* c, const pmc_points* passes, uint32_t n_p
         const uint64_t slots = c->use_cache ? c->desc.n_cells * ne : 0;
         const uint64_t cells = c->use_cache ? c->desc.n_cells : 0;
         if (flags & PMC_GRAPH_RESET) {
-            e = launch_reset(c->d_table, table_units(c), c->d_claims, c->d_chain_head, cells, c->d_ctl, c->d_stats, s, rounds);
+            e = launch_reset(c->d_table, table_units(c), c->d_claims, c->d_chain_head, cells, c->d_ctl, c->d_stats,
+                             c->num_sms, s);
             c->table_empty = true;
         } else {
             c->table_empty = false;   // the table's contents at replay time are unknown

@@ -1,11 +1,12 @@
 // kernels.cu -- sm_103a kernels of one progressive pass (Sec. 3, Alg. 1).
 //
-//   k_hist     material histogram of the batch (+ range check of material indices)
-//   k_scan     per-material segment offsets, probe offsets and warp work items
+//   k_begin    clears the batch's counters
+//   k_hist     material histogram of the batch (+ range check of material indices); its last
+//              block lays out the per-material segments, probe offsets and warp work items
 //   k_scatter  groups the points by material into structure-of-arrays copies
 //   k_lookup   probes of every (point, cacheable node) against the table as it was
 //              when the pass started (Sec. 3.2, Fig. 3); several probes in flight per lane
-//   k_scan_roots / k_eval_roots
+//   k_eval_roots
 //              the missed cacheable nodes, listed per node by k_lookup, evaluated 32 at a
 //              time with each node's standalone program; values go back into the probe
 //              records and become insert candidates (Sec. 3)
@@ -15,7 +16,6 @@
 //              targets the first slot of its cell holding its hash2 (duplicate) or 0
 //              (free, Alg. 1); the smallest (point index, node ID) per cell wins by
 //              atomicMin and writes its slot
-//   k_finish   advances the claim epoch and the batch counters
 #include <algorithm>
 #include <cstddef>
 #include <cstdio>
@@ -117,6 +117,39 @@ __device__ __forceinline__ U block_incl_scan(U v, U* tmp, U* total) {
     return r;
 }
 
+// Clears the counters of a batch (one launch instead of a memset for each of the regions; a pass of
+// 4,096 points is bound by its launches: reset and four passes took 299 us with four memsets,
+// separate scans and a closing kernel per pass, 254 us with this and the scans run by the last
+// block of k_hist and k_lookup): the
+// control block's per-batch part, the material and miss counts with the work-item counters
+// behind them, and the round counters of the claim-round insert.  Counts the batch.
+__global__ void __launch_bounds__(256) k_begin(BatchArgs a) {
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, T = gridDim.x * blockDim.x;
+    uint32_t* ctl = reinterpret_cast<uint32_t*>(a.ctl);
+    for (uint32_t i = t; i < offsetof(Control, epoch) / 4; i += T) ctl[i] = 0u;
+    if (a.insert_rounds)
+        for (uint32_t i = t; i < 2 * (MAX_ENTRIES + 2); i += T) a.ctl->mid_count[i] = 0u;   // and out_count behind it
+    for (uint32_t i = t; i <= a.n_mats; i += T) a.counts[i] = 0u;
+    if (a.split)
+        for (uint32_t i = t; i < a.n_roots_total + MAX_LEVELS; i += T) a.miss_cnt[i] = 0u;
+    if (t == 0) a.stats[ST_BATCHES] += 1ull;
+}
+
+// True in every thread of the block that arrives last of the grid's blocks (after its threads'
+// writes and atomics are visible to the device): the block that runs a kernel's epilogue.
+__device__ __forceinline__ bool last_block(uint32_t* ticket) {
+    __shared__ uint32_t s_ticket;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_ticket = atomicAdd(ticket, 1u);
+    __syncthreads();
+    if (s_ticket != gridDim.x - 1) return false;
+    __threadfence();
+    return true;
+}
+
+__device__ __forceinline__ void scan_materials(const BatchArgs& a);
+
 __global__ void __launch_bounds__(256) k_hist(BatchArgs a) {
     __shared__ uint32_t s_cnt[GROUP_SMEM_MATS];
     const bool local = a.n_mats <= GROUP_SMEM_MATS;
@@ -165,10 +198,12 @@ __global__ void __launch_bounds__(256) k_hist(BatchArgs a) {
         atomicAdd(&a.stats[ST_BAD], tot);
         atomicOr(&a.ctl->err, ERR_BAD_MAT);
     }
+    // the block that finishes last lays out the materials' segments
+    if (last_block(&a.ctl->hist_done)) scan_materials(a);
 }
 
 // One block: exclusive scans of counts, counts * roots and ceil(counts / 32).
-__global__ void k_scan(BatchArgs a) {
+__device__ __forceinline__ void scan_materials(const BatchArgs& a) {
     __shared__ uint32_t s_tmp[33];
     const uint32_t T = blockDim.x, t = threadIdx.x;
     const uint32_t per = (a.n_mats + T - 1) / T;
@@ -177,8 +212,9 @@ __global__ void k_scan(BatchArgs a) {
     // the surrogate instead of a lookup)
     const bool surr = a.surr_slot != nullptr;
     uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
+#pragma unroll 4
     for (uint32_t m = lo; m < hi; ++m) {
-        uint32_t c = a.counts[m];
+        uint32_t c = __ldcg(&a.counts[m]);
         uint32_t k = (a.use_cache || surr) ? a.mats[m].n_roots : 0u;
         c0 += c;
         c1 += c * k;
@@ -190,8 +226,9 @@ __global__ void k_scan(BatchArgs a) {
     uint32_t b1 = block_incl_scan(c1, s_tmp, &tot1) - c1;
     uint32_t b2 = block_incl_scan(c2, s_tmp, &tot2) - c2;
     uint32_t b3 = block_incl_scan(c3, s_tmp, &tot3) - c3;
+#pragma unroll 4
     for (uint32_t m = lo; m < hi; ++m) {
-        uint32_t c = a.counts[m];
+        uint32_t c = __ldcg(&a.counts[m]);
         uint32_t k = (a.use_cache || surr) ? a.mats[m].n_roots : 0u;
         a.seg_start[m] = b0;
         a.cursor[m] = b0;
@@ -347,6 +384,39 @@ __device__ __forceinline__ int scan_words(const uint4 (&w)[NQ], uint32_t h2, uin
     return first;
 }
 
+// Work items of the batched evaluation: ceil(misses / 32) per cacheable node, laid out in
+// ascending nesting level (root_order), with the first item of each level after them.
+__device__ __forceinline__ void scan_roots(const BatchArgs& a) {
+    __shared__ uint32_t s_tmp[33];
+    const uint32_t T = blockDim.x, t = threadIdx.x, N = a.n_roots_total;
+    const uint32_t per = (N + T - 1) / T;
+    const uint32_t lo = min(t * per, N), hi = min(lo + per, N);
+    uint32_t c = 0;
+#pragma unroll 4
+    for (uint32_t q = lo; q < hi; ++q) c += (__ldcg(&a.miss_cnt[a.root_order[q]]) + 31u) >> 5;
+    uint32_t tot;
+    uint32_t b = block_incl_scan(c, s_tmp, &tot) - c;
+#pragma unroll 4
+    for (uint32_t q = lo; q < hi; ++q) {
+        a.root_item_base[q] = b;
+        b += (__ldcg(&a.miss_cnt[a.root_order[q]]) + 31u) >> 5;
+    }
+    __syncthreads();
+    if (t == T - 1) {
+        a.root_item_base[N] = tot;
+        a.ctl->n_root_items = tot;
+    }
+    __syncthreads();
+    uint32_t* level_items = a.root_item_base + N + 1;
+    for (uint32_t l = t; l <= MAX_LEVELS; l += T) level_items[l] = a.root_item_base[a.level_start[l]];
+}
+
+__global__ void __launch_bounds__(1024) k_scan_roots(BatchArgs a) { scan_roots(a); }
+
+// Up to this many cacheable nodes the last block of the lookup lays out the items itself (a
+// few per thread); above, a launch of its own with four times the threads is the faster way.
+constexpr uint32_t SCAN_IN_LOOKUP = 2048;
+
 // NQ = 16-byte words of hash2 per cell (ceil(N_e / 4)); RB probes in flight per lane; POS:
 // the cache has the world-position descriptor (a separate instantiation, so that caches
 // without it keep the registers the position keys would take).
@@ -457,6 +527,7 @@ __global__ void __launch_bounds__(256, 4) k_lookup(BatchArgs a) {
     warp_add_u64(&a.stats[ST_HITS], n_hit);
     warp_add_u64(&a.stats[ST_MISSES], n_look - n_hit);
     warp_add_u64(&a.stats[ST_SLOTS], n_slots);
+    if (a.split && a.n_roots_total <= SCAN_IN_LOOKUP && last_block(&a.ctl->lookup_done)) scan_roots(a);
 }
 
 // =======================================================================================
@@ -1256,31 +1327,6 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_fused(BatchArgs a, uin
         warp_add_u64(&a.stats[ST_BAD], n_bad);
         if (__any_sync(FULL_MASK, n_bad != 0) && lane == 0) atomicOr(&a.ctl->err, ERR_BAD_MAT);
     }
-}
-
-// Work items of the batched evaluation: ceil(misses / 32) per cacheable node, laid out in
-// ascending nesting level (root_order), with the first item of each level after them.
-__global__ void k_scan_roots(BatchArgs a) {
-    __shared__ uint32_t s_tmp[33];
-    const uint32_t T = blockDim.x, t = threadIdx.x, N = a.n_roots_total;
-    const uint32_t per = (N + T - 1) / T;
-    const uint32_t lo = min(t * per, N), hi = min(lo + per, N);
-    uint32_t c = 0;
-    for (uint32_t q = lo; q < hi; ++q) c += (a.miss_cnt[a.root_order[q]] + 31u) >> 5;
-    uint32_t tot;
-    uint32_t b = block_incl_scan(c, s_tmp, &tot) - c;
-    for (uint32_t q = lo; q < hi; ++q) {
-        a.root_item_base[q] = b;
-        b += (a.miss_cnt[a.root_order[q]] + 31u) >> 5;
-    }
-    __syncthreads();
-    if (t == T - 1) {
-        a.root_item_base[N] = tot;
-        a.ctl->n_root_items = tot;
-    }
-    __syncthreads();
-    uint32_t* level_items = a.root_item_base + N + 1;
-    for (uint32_t l = t; l <= MAX_LEVELS; l += T) level_items[l] = a.root_item_base[a.level_start[l]];
 }
 
 // Batched evaluation of the missed cacheable nodes (the "missed sub-graphs" of Sec. 3):
@@ -2759,11 +2805,9 @@ __global__ void __launch_bounds__(256, 4) k_chain_resolve(BatchArgs a) {
     warp_add_u64(&a.stats[ST_INSERTED], n_ins);
 }
 
-__global__ void k_finish(BatchArgs a) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        if (a.use_cache) a.ctl->epoch += a.n_entries + 1u;
-        a.stats[ST_BATCHES] += 1ull;
-    }
+// Advances the claim epoch past the rounds of this batch.
+__global__ void k_next_epoch(BatchArgs a) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) a.ctl->epoch += a.n_entries + 1u;
 }
 
 // =======================================================================================
@@ -2816,19 +2860,33 @@ cudaError_t launch_keys(const uint32_t* mat, const uint32_t* node, const float* 
     return cudaGetLastError();
 }
 
+// Empties a cache: zeros over the table (16-byte units), all-ones over the claim words (the
+// largest claim of the atomicMin rounds) and over the list heads (the per-cell-list insert
+// leaves every list empty after a batch; this only repairs lists left by a batch that
+// failed), zeros over the control block and the counters.  One launch instead of five memsets:
+// a small table's reset is launch time.
+__global__ void __launch_bounds__(256) k_reset(uint4* table, size_t units, unsigned long long* claims,
+                                               uint32_t* chain_head, size_t cells, Control* ctl,
+                                               unsigned long long* stats) {
+    const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, T = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = t; i < units; i += T) table[i] = make_uint4(0, 0, 0, 0);
+    ulonglong2* c2 = reinterpret_cast<ulonglong2*>(claims);
+    for (size_t i = t; i < cells / 2; i += T) c2[i] = make_ulonglong2(~0ull, ~0ull);
+    uint4* h4 = reinterpret_cast<uint4*>(chain_head);
+    for (size_t i = t; i < cells / 4; i += T) h4[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    if (t == 0 && (cells & 1)) claims[cells - 1] = ~0ull;
+    if (t < (cells & 3)) chain_head[cells - 1 - t] = ~0u;
+    for (size_t i = t; i < sizeof(Control) / 4; i += T) reinterpret_cast<uint32_t*>(ctl)[i] = 0u;
+    for (size_t i = t; i < ST_COUNT; i += T) stats[i] = 0ull;
+}
+
 cudaError_t launch_reset(uint4* table, size_t units, unsigned long long* claims, uint32_t* chain_head, size_t cells,
-                         Control* ctl, unsigned long long* stats, cudaStream_t s, bool claim_words) {
-    cudaError_t e;
-    if (units && (e = cudaMemsetAsync(table, 0, (units + 16) * sizeof(uint4), s)) != cudaSuccess) return e;
-    // all-ones: the largest claim word of the atomicMin rounds, and an empty list per cell
-    // for the per-cell-list insert (which leaves every list empty after a batch; this only
-    // repairs lists left by a batch that failed)
-    (void)claim_words;
-    if (cells && (e = cudaMemsetAsync(claims, 0xFF, cells * sizeof(unsigned long long), s)) != cudaSuccess) return e;
-    if (cells && chain_head && (e = cudaMemsetAsync(chain_head, 0xFF, cells * sizeof(uint32_t), s)) != cudaSuccess)
-        return e;
-    if ((e = cudaMemsetAsync(ctl, 0, sizeof(Control), s)) != cudaSuccess) return e;
-    return cudaMemsetAsync(stats, 0, ST_COUNT * sizeof(unsigned long long), s);
+                         Control* ctl, unsigned long long* stats, int num_sms, cudaStream_t s) {
+    const size_t all = units ? units + 16 : 0;   // the table's padding too
+    const size_t want = (std::max(all, cells) + 1023) / 1024;   // four units a thread, or more
+    const unsigned blocks = (unsigned)std::min<size_t>(std::max<size_t>(want, 1), (size_t)num_sms * 8);
+    k_reset<<<blocks, 256, 0, s>>>(table, all, claims, chain_head, cells, ctl, stats);
+    return cudaGetLastError();
 }
 
 int insert_grid(int num_sms) {
@@ -2851,7 +2909,8 @@ static cudaError_t launch_insert(const BatchArgs& a, cudaStream_t s, int num_sms
         if ((e = cudaLaunchCooperativeKernel((const void*)k_insert, dim3(insert_grid(num_sms)), dim3(256), params, 0, s)) !=
             cudaSuccess)
             return e;
-        *nl += 1;
+        k_next_epoch<<<1, 32, 0, s>>>(a);
+        *nl += 2;
     } else if (a.n > 0 && a.use_cache && a.insert_lists) {
         static int per_sm = 0;
         if (per_sm == 0) {
@@ -2903,33 +2962,35 @@ void launch_lookup(const BatchArgs& a, uint32_t ne, uint32_t rb, unsigned lb, cu
     }
 }
 
+// Blocks of the grouping kernels: one per 256 points at most (a block without points still
+// takes part in a kernel's end), and at least one.
+static unsigned group_blocks(uint32_t n, int num_sms) {
+    return std::max(1u, std::min((n + 255u) / 256u, (unsigned)num_sms * GROUP_BLOCKS_PER_SM));
+}
+
 cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEvent_t* ev,
                          uint64_t* launches) {
     cudaError_t e;
     uint64_t nl = 0;
     auto mark = [&](int k) { return ev ? cudaEventRecord(ev[k], s) : cudaSuccess; };
     if ((e = mark(0)) != cudaSuccess) return e;
-    // per-batch counters (epoch, errors and the barrier persist)
-    if ((e = cudaMemsetAsync(a.ctl, 0, offsetof(Control, epoch), s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.ctl->mid_count, 0, 2 * (MAX_ENTRIES + 2) * sizeof(uint32_t), s)) != cudaSuccess) return e;
-    // counts has n_mats + 1 entries; the last one is the evaluation's work-item counter
-    if ((e = cudaMemsetAsync(a.counts, 0, (a.n_mats + 1) * sizeof(uint32_t), s)) != cudaSuccess) return e;
-    if (a.split && (e = cudaMemsetAsync(a.miss_cnt, 0, (a.n_roots_total + MAX_LEVELS) * sizeof(uint32_t), s)) != cudaSuccess)
-        return e;
+    // per-batch counters (epoch, errors and the barrier persist); counts has n_mats + 1 entries,
+    // the last one the evaluation's work-item counter
+    {
+        const uint32_t words = a.n_mats + (a.split ? a.n_roots_total : 0u);
+        k_begin<<<std::min<uint32_t>(1u + words / 1024u, 64u), 256, 0, s>>>(a);
+        nl++;
+    }
     uint32_t* item_ctr = a.counts + a.n_mats;
     if (a.alg1 && a.use_cache) {
         // the paper's concurrent update: lookups and inserts inside the evaluator, no
         // lookup kernel, no insert phase; grouped by material unless unsorted
-        if (!a.unsorted && a.n > 0) {
-            k_hist<<<num_sms * GROUP_BLOCKS_PER_SM, 256, 0, s>>>(a);
-            nl++;
-        }
         if (!a.unsorted) {
-            k_scan<<<1, 1024, 0, s>>>(a);
+            k_hist<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
             nl++;
         }
         if (!a.unsorted && a.n > 0) {
-            k_scatter<<<num_sms * GROUP_BLOCKS_PER_SM, 256, 0, s>>>(a);
+            k_scatter<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
             nl++;
         }
         if ((e = mark(1)) != cudaSuccess) return e;
@@ -2958,8 +3019,6 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
         }
         if ((e = mark(4)) != cudaSuccess) return e;
         if ((e = mark(5)) != cudaSuccess) return e;
-        k_finish<<<1, 32, 0, s>>>(a);
-        nl++;
         if ((e = mark(6)) != cudaSuccess) return e;
         if (launches) *launches += nl;
         return cudaGetLastError();
@@ -2981,20 +3040,14 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
         if ((e = mark(4)) != cudaSuccess) return e;
         if ((e = launch_insert(a, s, num_sms, &nl)) != cudaSuccess) return e;
         if ((e = mark(5)) != cudaSuccess) return e;
-        k_finish<<<1, 32, 0, s>>>(a);
-        nl++;
         if ((e = mark(6)) != cudaSuccess) return e;
         if (launches) *launches += nl;
         return cudaGetLastError();
     }
-    if (a.n > 0) {
-        k_hist<<<num_sms * GROUP_BLOCKS_PER_SM, 256, 0, s>>>(a);
-        nl++;
-    }
-    k_scan<<<1, 1024, 0, s>>>(a);
+    k_hist<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
     nl++;
     if (a.n > 0) {
-        k_scatter<<<num_sms * GROUP_BLOCKS_PER_SM, 256, 0, s>>>(a);
+        k_scatter<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
         nl++;
     }
     if ((e = mark(1)) != cudaSuccess) return e;
@@ -3054,8 +3107,10 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
                 cudaSuccess)
             return e;
         if (a.use_cache && a.split && !a.keys_inline && !a.all_surr) {
-            k_scan_roots<<<1, 1024, 0, s>>>(a);
-            nl++;
+            if (a.n_roots_total > SCAN_IN_LOOKUP) {
+                k_scan_roots<<<1, 1024, 0, s>>>(a);
+                nl++;
+            }
             // the level counters live after the per-root miss counters
             for (uint32_t lv = 0; lv <= a.max_level; ++lv) {
                 kroots<<<num_sms * 16, EVAL_WARPS * 32, smem_kroots, s>>>(a, lv, a.miss_cnt + a.n_roots_total + lv);
@@ -3072,8 +3127,6 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
     // with every cacheable node a surrogate's there is nothing to insert
     if (!a.all_surr && (e = launch_insert(a, s, num_sms, &nl)) != cudaSuccess) return e;
     if ((e = mark(5)) != cudaSuccess) return e;
-    k_finish<<<1, 32, 0, s>>>(a);
-    nl++;
     if ((e = mark(6)) != cudaSuccess) return e;
     if (launches) *launches += nl;
     return cudaGetLastError();

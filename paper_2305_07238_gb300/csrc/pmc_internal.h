@@ -138,7 +138,8 @@ struct Control {
     uint32_t bins_big;
     uint32_t n_lists;           // cells with candidates (per-cell-list insert)
     uint32_t w_cand;            // candidates emitted for the insert, shadows included
-    uint32_t pad1;
+    uint32_t hist_done;         // blocks done of k_hist and k_lookup (the last runs the scans)
+    uint32_t lookup_done;
     // persistent
     uint32_t epoch;             // claim epoch of round 0 of the current batch
     uint32_t err;               // ERR_* bits
@@ -217,7 +218,7 @@ struct BatchArgs {
     // ordinal; FP32 parameters per slot; work items of 128 points per material
     const int32_t* surr_slot; const int32_t* surr_ord; const float* surr_theta;
     const unsigned char* surr_img;   // per slot SURR_IMG_BYTES (16-byte aligned), or null
-    uint32_t* surr_item_base;  // n_mats + 1 (computed by k_scan)
+    uint32_t* surr_item_base;  // n_mats + 1 (computed by k_hist)
     int all_surr;              // 1: every cacheable node of every material is a surrogate's:
                                // no lookup, no batched misses, no insert
     uint32_t n_bins;           // cell-grouped insert: ceil(n_cells / 2^bin_shift) bins
@@ -280,7 +281,7 @@ enum { PH_SORT = 0, PH_LOOKUP, PH_MISSED, PH_EVAL, PH_INSERT, PH_FINISH, PH_COUN
 cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEvent_t* ev,
                          uint64_t* launches);
 cudaError_t launch_reset(uint4* table, size_t units, unsigned long long* claims, uint32_t* chain_head, size_t cells,
-                         Control* ctl, unsigned long long* stats, cudaStream_t s, bool claim_words);
+                         Control* ctl, unsigned long long* stats, int num_sms, cudaStream_t s);
 cudaError_t launch_levels(const float* g1u, const float* g1v, const float* g2u, const float* g2v, uint64_t n,
                           int32_t offset, uint32_t* level, cudaStream_t s);
 cudaError_t launch_keys(const uint32_t* mat, const uint32_t* node, const float* u,
