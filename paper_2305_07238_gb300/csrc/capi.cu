@@ -14,27 +14,24 @@ using namespace pmc;
 
 namespace {
 
-// The device form of a compiled instruction: slots become byte offsets into the slot file,
-// a MIX reading its factor from a node gets FLAG_IN2, parameter offsets move by the
-// material's base in the pool.  *ok is cleared if a slot is beyond the 16-bit offsets.
-uint4 device_ins(uint4 ins, uint32_t pbase, bool* ok) {
-    const uint32_t op = ins.x & 0xFFu;
-    auto off = [&](uint32_t slot) -> uint32_t {
-        if (slot == 0xFFFFu) return 0u;   // no such input
-        if (slot > MAX_DEVICE_SLOTS) *ok = false;
-        return slot * SLOT_BYTES;
-    };
-    if (op == OP_ROOT_BEGIN || op == OP_LOAD_ROOT) {
+// The device form of a compacted instruction: rows become byte offsets into the slot file, and
+// parameter offsets move by the material's base in the pool.
+uint4 device_ins(uint4 ins, uint32_t pbase) {
+    auto off = [](uint32_t row) -> uint32_t { return row == 0xFFFFu ? 0u : row * ROW_BYTES; };   // 0xFFFF: no such input
+    if ((ins.x & 0xFFu) >= OP_CONTROL) {
         ins.y = off(ins.y & 0xFFFFu) | (ins.y & 0xFFFF0000u);   // out | ordinal
         return ins;
     }
-    uint32_t flags = (ins.x >> 8) & 0xFFu;
-    if (op == PMC_OP_MIX && (ins.z >> 16) != 0xFFFFu) flags |= FLAG_IN2;
-    ins.x = (ins.x & ~0xFF00u) | (flags << 8);
     ins.y = off(ins.y & 0xFFFFu) | (off(ins.y >> 16) << 16);
     ins.z = off(ins.z & 0xFFFFu) | (off(ins.z >> 16) << 16);
     ins.w += pbase;
     return ins;
+}
+
+// Appends a program to the pool, with its end.
+void push_program(const std::vector<uint4>& code, uint32_t pbase, std::vector<uint4>* pool) {
+    for (uint4 ins : code) pool->push_back(device_ins(ins, pbase));
+    pool->push_back(make_uint4(OP_END, 0, 0, 0));
 }
 
 // Nodes and FP32 operations of one run of a program in which every node instruction runs.
@@ -42,7 +39,7 @@ void program_totals(const std::vector<uint4>& prog, uint32_t* nodes, uint32_t* f
     uint64_t n = 0, f = 0;
     for (const uint4& ins : prog) {
         const uint32_t op = ins.x & 0xFFu;
-        if (op == OP_ROOT_BEGIN || op == OP_LOAD_ROOT) continue;
+        if (op >= OP_CONTROL) continue;
         n++;
         f += ins.x >> 16;
     }
@@ -264,6 +261,7 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
 
     std::vector<uint4> prog;
     std::vector<float> params;
+    uint32_t point_slots = 0, root_slots = 0;   // largest programs in slots of three channels
     for (uint32_t m = 0; m < n_mats; ++m) {
         CompiledMaterial cm;
         const char* why = "";
@@ -278,13 +276,12 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
         mi.prog_len = (uint32_t)cm.prog.size();
         mi.root_base = (uint32_t)c->roots.size();
         mi.n_roots = (uint32_t)cm.roots.size();
-        mi.out_slot = cm.out_slot;
+        mi.out_row = cm.out_row;
         mi.n_slots = cm.n_slots;
         mi.n_nodes = cm.n_nodes;
         params.resize((params.size() + 3) & ~size_t(3), 0.0f);   // 16-byte aligned per material
         const uint32_t pbase = (uint32_t)params.size();
-        bool slots_ok = true;
-        for (uint4 ins : cm.prog) prog.push_back(device_ins(ins, pbase, &slots_ok));
+        push_program(cm.prog, pbase, &prog);
         program_totals(cm.prog, &mi.full_nodes, &mi.full_flops);
         program_totals(cm.outer_prog, &mi.outer_nodes, &mi.outer_flops);
         int32_t cand = -1;
@@ -299,10 +296,11 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
         c->surr_cand.push_back(cand);
         mi.outer_start = (uint32_t)prog.size();
         mi.outer_len = (uint32_t)cm.outer_prog.size();
-        mi.outer_out_slot = cm.outer_out_slot;
+        mi.outer_out_row = cm.outer_out_row;
         mi.outer_slots = cm.outer_slots;
-        for (uint4 ins : cm.outer_prog) prog.push_back(device_ins(ins, pbase, &slots_ok));
-        c->max_slots_outer = std::max(c->max_slots_outer, cm.outer_slots);
+        push_program(cm.outer_prog, pbase, &prog);
+        c->max_rows_outer = std::max(c->max_rows_outer, cm.outer_rows);
+        uint32_t most_slots = std::max(cm.n_slots, cm.outer_slots);
         for (size_t r = 0; r < cm.roots.size(); ++r) {
             RootInfo ri{};
             ri.prog_start = (uint32_t)prog.size();
@@ -312,14 +310,16 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
             ri.level = cm.root_level[r];
             ri.n_slots = cm.root_slots[r];
             ri.node = cm.roots[r];
-            ri.out_slot = cm.root_out_slot[r];
+            ri.out_row = cm.root_out_row[r];
             program_totals(cm.root_progs[r], &ri.nodes, &ri.flops);
-            for (uint4 ins : cm.root_progs[r]) prog.push_back(device_ins(ins, pbase, &slots_ok));
+            push_program(cm.root_progs[r], pbase, &prog);
             c->root_info.push_back(ri);
             c->max_level = std::max(c->max_level, ri.level);
-            c->max_slots_roots = std::max(c->max_slots_roots, ri.n_slots);
+            c->max_rows_roots = std::max(c->max_rows_roots, cm.root_rows[r]);
+            root_slots = std::max(root_slots, ri.n_slots);
+            most_slots = std::max(most_slots, ri.n_slots);
         }
-        if (!slots_ok) {
+        if (most_slots > MAX_DEVICE_SLOTS + 1) {   // slots are numbered from 0
             fprintf(stderr, "pmc: material %u needs more than %u live values\n", m, MAX_DEVICE_SLOTS);
             delete c;
             return PMC_ERR_UNSUPPORTED;
@@ -330,7 +330,8 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
             c->roots_dev.push_back(cm.roots[r] | (cm.root_pos[r] ? ROOT_POS_BIT : 0u));
         c->mat_info.push_back(mi);
         c->max_roots = std::max(c->max_roots, mi.n_roots);
-        c->max_slots = std::max(c->max_slots, mi.n_slots);
+        c->max_rows = std::max(c->max_rows, cm.rows);
+        point_slots = std::max(point_slots, mi.n_slots);
     }
     // the interpreters fetch one instruction ahead of the one they run: a zero instruction
     // past the last program keeps that read inside the pool
@@ -339,9 +340,9 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
     // the interpreters fetch eight parameters ahead of a node, even one without any
     params.resize(((params.size() + 3) & ~size_t(3)) + 8, 0.0f);
     if (c->max_level >= MAX_LEVELS) c->split = 0;   // deeper nesting: evaluate misses inline
-    if (eval_smem_bytes(std::max(c->max_slots, c->max_slots_roots)) > 200u * 1024u) {
+    if (eval_smem_bytes(3 * std::max(point_slots, root_slots)) > 200u * 1024u) {
         fprintf(stderr, "pmc: a material needs %u live values; this build supports %zu\n",
-                std::max(c->max_slots, c->max_slots_roots), (size_t)(200u * 1024u) / eval_smem_bytes(1));
+                std::max(point_slots, root_slots), (size_t)(200u * 1024u) / eval_smem_bytes(3));
         delete c;
         return PMC_ERR_UNSUPPORTED;
     }
@@ -460,9 +461,9 @@ pmc_status enqueue_batch(pmc_cache* c, const pmc_points* pts, float* out_rgb, ui
     a.out_rgb = out_rgb; a.out_hits = out_hits;
     a.mats = c->d_mats; a.n_mats = c->n_mats;
     a.prog = c->d_prog; a.params = c->d_params; a.roots = c->d_roots;
-    a.max_slots = c->max_slots ? c->max_slots : 1;
-    a.max_slots_roots = c->max_slots_roots ? c->max_slots_roots : 1;
-    a.max_slots_outer = c->max_slots_outer ? c->max_slots_outer : 1;
+    a.max_rows = c->max_rows ? c->max_rows : 1;
+    a.max_rows_roots = c->max_rows_roots ? c->max_rows_roots : 1;
+    a.max_rows_outer = c->max_rows_outer ? c->max_rows_outer : 1;
     const size_t M1 = (size_t)c->n_mats + 1;
     a.counts = c->d_seg; a.seg_start = c->d_seg + M1; a.probe_base = c->d_seg + 2 * M1;
     a.item_base = c->d_seg + 3 * M1; a.cursor = c->d_seg + 4 * M1;
@@ -1036,7 +1037,7 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     // training pairs from the exact evaluator
     if (e == cudaSuccess)
         e = launch_root_samples(c->d_prog, c->d_params, c->d_rinfo, groots, L, d->n_train, d->seed, data,
-                                c->max_slots_roots ? c->max_slots_roots : 1, c->num_sms, s);
+                                c->max_rows_roots ? c->max_rows_roots : 1, c->num_sms, s);
     const uint32_t steps_per_epoch = d->n_train / 128u;
     const uint32_t total = steps_per_epoch * d->epochs;
     const float lr = d->lr > 0.0f ? d->lr : 1e-2f;
@@ -1050,7 +1051,7 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     // validation against held-out exact values, all networks in one launch
     if (e == cudaSuccess)
         e = launch_root_samples(c->d_prog, c->d_params, c->d_rinfo, groots, L, nv, d->seed ^ 0x5DEECE66Dull, data,
-                                c->max_slots_roots ? c->max_slots_roots : 1, c->num_sms, s);
+                                c->max_rows_roots ? c->max_rows_roots : 1, c->num_sms, s);
     const uint32_t parts = mlp_validate_parts(L, nv, c->num_sms);
     double* d_sum = nullptr;
     std::vector<double> sums((size_t)L * parts);

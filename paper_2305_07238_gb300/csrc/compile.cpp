@@ -158,6 +158,14 @@ bool fold(const pmc_node& nd, const std::vector<pmc_node>& g, pmc_node* out) {
     return true;
 }
 
+// The coordinates below which freq x coordinate stays under 2^22 in magnitude, whatever the
+// rounding of the frequency in FP32 (a margin of 2^-10); 0, so that no coordinate is, for a
+// frequency too large or not a number.
+float noise_limit(double freq) {
+    if (!(freq < 1e30)) return 0.0f;
+    return (float)std::min(4194304.0 * (1.0 - 0x1p-10) / std::max(freq, 1e-30), 1e38);
+}
+
 // Appends a node's parameters to the pool.  Every node's parameters start on a 16-byte
 // boundary so that an interpreter can fetch the first eight with two vector loads.
 void pack_params(const pmc_node& nd, std::vector<float>* pool) {
@@ -173,11 +181,13 @@ void pack_params(const pmc_node& nd, std::vector<float>* pool) {
     case PMC_OP_FBM: {
         double norm = 0.0, amp = 1.0;
         for (int k = 0; k < nd.ip[0]; ++k) { norm += amp; amp *= (double)p[2]; }
-        pool->insert(pool->end(), {p[0], p[1], p[2], (float)(1.0 / norm), bits(nd.ip[0]), bits(nd.ip[1])});
+        double top = 0.0, freq = p[0];   // the largest |frequency| of an octave
+        for (int k = 0; k < nd.ip[0]; ++k, freq *= (double)p[1]) top = std::fabs(freq) <= top ? top : std::fabs(freq);
+        pool->insert(pool->end(), {p[0], p[1], p[2], (float)(1.0 / norm), bits(nd.ip[0]), bits(nd.ip[1]), noise_limit(top)});
         break;
     }
     case PMC_OP_VORONOI:
-        pool->insert(pool->end(), {p[0], bits(nd.ip[1])});
+        pool->insert(pool->end(), {p[0], bits(nd.ip[1]), noise_limit(std::fabs((double)p[0]))});
         break;
     case PMC_OP_CHECKER:
         pool->insert(pool->end(), {p[0], p[1], p[2], p[3], p[4], p[5], p[6]});
@@ -214,6 +224,17 @@ void pack_params(const pmc_node& nd, std::vector<float>* pool) {
 }
 
 
+// The nodes whose last use is at a place of the program, as a list per place (filled from the
+// last node to the first, so that each lists its nodes in ascending order).
+struct ReleaseLists {
+    std::vector<uint32_t> head, next;
+    ReleaseLists(size_t places, size_t nodes) : head(places + 1, ~0u), next(nodes, ~0u) {}
+    void add(size_t place, uint32_t x) {
+        next[x] = head[place];
+        head[place] = x;
+    }
+};
+
 // Emits a linear program for `order` (nodes in topological order; entries flagged as
 // loads take a cacheable node's value from its probe record instead of evaluating it)
 // with linear-scan slot allocation.  `keep` is the node whose value must survive to the
@@ -234,9 +255,9 @@ uint32_t emit_standalone(const std::vector<pmc_node>& g, const std::vector<std::
         }
     }
     last_use[keep] = (int64_t)L;
-    std::vector<std::vector<uint32_t>> release_at(L + 1);
-    for (uint32_t x = 0; x < g.size(); ++x)
-        if (in_order[x] && last_use[x] >= 0 && last_use[x] < (int64_t)L) release_at[last_use[x]].push_back(x);
+    ReleaseLists release_at(L, g.size());
+    for (uint32_t x = (uint32_t)g.size(); x-- > 0;)
+        if (in_order[x] && last_use[x] >= 0 && last_use[x] < (int64_t)L) release_at.add((size_t)last_use[x], x);
     std::vector<uint32_t> slot(g.size(), 0xFFFFu), free_slots;
     uint32_t n_slots = 0;
     auto take = [&]() {
@@ -250,7 +271,7 @@ uint32_t emit_standalone(const std::vector<pmc_node>& g, const std::vector<std::
         uint32_t x = order[p].first;
         uint4 ins;
         if (order[p].second) {
-            for (uint32_t y : release_at[p]) free_slots.push_back(slot[y]);
+            for (uint32_t y = release_at.head[p]; y != ~0u; y = release_at.next[y]) free_slots.push_back(slot[y]);
             slot[x] = take();
             ins.x = OP_LOAD_ROOT;
             ins.y = slot[x] | (ordinal[x] << 16);
@@ -262,7 +283,7 @@ uint32_t emit_standalone(const std::vector<pmc_node>& g, const std::vector<std::
         uint32_t in_slot[3] = {0xFFFFu, 0xFFFFu, 0xFFFFu};
         for (int k = 0; k < 3; ++k)
             if (g[x].in[k] >= 0) in_slot[k] = slot[g[x].in[k]];
-        for (uint32_t y : release_at[p]) free_slots.push_back(slot[y]);
+        for (uint32_t y = release_at.head[p]; y != ~0u; y = release_at.next[y]) free_slots.push_back(slot[y]);
         slot[x] = take();
         const uint32_t flags = (x == keep && keep_is_root) ? FLAG_ROOT : 0u;
         const uint32_t cost = std::min<uint32_t>(node_cost(g[x]), 0xFFFFu);
@@ -299,6 +320,156 @@ uint32_t node_cost(const pmc_node& nd) {
     case PMC_OP_FACING: return 8;                         // dot (mul + 2 fma), abs, clamp
     default: return 0;
     }
+}
+
+namespace {
+
+// The operators of device programs without kinds of rows (DOP_*); the others are chosen by kind.
+uint32_t device_op(uint32_t op, bool w0, bool w1, bool wide, bool in2) {
+    switch (op) {
+    case PMC_OP_UV: return DOP_UV;
+    case PMC_OP_POSITION: return DOP_POSITION;
+    case PMC_OP_NORMAL: return DOP_NORMAL;
+    case PMC_OP_CONST: return wide ? DOP_CONST : DOP_CONST_1;
+    case PMC_OP_UV_AFFINE: return DOP_AFFINE;
+    case PMC_OP_FBM: return DOP_FBM;
+    case PMC_OP_VORONOI: return DOP_VORONOI;
+    case PMC_OP_CHECKER: return DOP_CHECKER;
+    case PMC_OP_RAMP: return DOP_RAMP;
+    case PMC_OP_MIX: return (in2 ? DOP_MIXN_33 : DOP_MIX_33) + (w0 ? 0 : 2) + (w1 ? 0 : 1);
+    case PMC_OP_ADD: return w0 && w1 ? DOP_ADD_33 : w0 || w1 ? DOP_ADD_31 : DOP_ADD_11;
+    case PMC_OP_MUL: return w0 && w1 ? DOP_MUL_33 : w0 || w1 ? DOP_MUL_31 : DOP_MUL_11;
+    case PMC_OP_POW: return w0 ? DOP_POW_3 : DOP_POW_1;
+    default: return DOP_FACING;
+    }
+}
+
+// Rows in use, as bits: the first run of `width` (1 or 3) free ones.
+struct RowSet {
+    std::vector<uint64_t> bits;
+    uint32_t take(uint32_t width) {
+        for (uint32_t w = 0;; ++w) {
+            if (bits.size() < w + 2) bits.resize(w + 2, 0);
+            uint64_t f = ~bits[w];
+            if (width == 3) {
+                const uint64_t n = ~bits[w + 1];
+                f &= ((f >> 1) | (n << 63)) & ((f >> 2) | (n << 62));
+            }
+            if (!f) continue;
+            const uint32_t r = 64 * w + (uint32_t)__builtin_ctzll(f);
+            for (uint32_t k = 0; k < width; ++k) bits[(r + k) >> 6] |= 1ull << ((r + k) & 63);
+            return r;
+        }
+    }
+    void give(uint32_t r, uint32_t width) {
+        for (uint32_t k = 0; k < width; ++k) bits[(r + k) >> 6] &= ~(1ull << ((r + k) & 63));
+    }
+};
+
+}  // namespace
+
+uint32_t compact_rows(std::vector<uint4>* prog, const std::vector<float>& params, uint32_t n_slots, uint32_t out_slot,
+                      uint32_t* out_row) {
+    // the program's values: one per definition (a cacheable node's block begins with its
+    // definition and ends with another write to it); `next`: the value ending at the same place
+    struct Value {
+        uint32_t def, last, row;
+        int next;
+        bool wide;   // three rows
+    };
+    struct Refs {
+        int out, in[3];
+    };
+    const uint32_t L = (uint32_t)prog->size();
+    std::vector<Value> val;
+    val.reserve(L);
+    std::vector<Refs> refs(L);
+    std::vector<int> cur(n_slots, -1);   // value now in each slot
+    for (uint32_t p = 0; p < L; ++p) {
+        const uint4 ins = (*prog)[p];
+        const uint32_t op = ins.x & 0xFFu, out = ins.y & 0xFFFFu;
+        Refs& r = refs[p];
+        r = Refs{-1, {-1, -1, -1}};
+        bool wide = op >= OP_CONTROL || op == PMC_OP_UV || op == PMC_OP_POSITION || op == PMC_OP_NORMAL ||
+                    op == PMC_OP_UV_AFFINE || op == PMC_OP_CHECKER || op == PMC_OP_RAMP;
+        if (op < OP_CONTROL) {
+            const uint32_t s[3] = {ins.y >> 16, ins.z & 0xFFFFu, ins.z >> 16};
+            for (int k = 0; k < 3; ++k)
+                if (s[k] != NO_SLOT) {
+                    r.in[k] = cur[s[k]];
+                    val[r.in[k]].last = p;
+                }
+            if (op == PMC_OP_CONST)
+                wide = float_bits(params[ins.w]) != float_bits(params[ins.w + 1]) ||
+                       float_bits(params[ins.w]) != float_bits(params[ins.w + 2]);
+            if (op == PMC_OP_ADD || op == PMC_OP_MUL || op == PMC_OP_MIX) wide = val[r.in[0]].wide || val[r.in[1]].wide;
+            if (op == PMC_OP_POW) wide = val[r.in[0]].wide;
+            if ((ins.x >> 8) & FLAG_ROOT) {
+                // a cacheable node's value is read by channel elsewhere (offers, records)
+                wide = true;
+                const int v = cur[out];
+                if (v >= 0 && ((*prog)[val[v].def].x & 0xFFu) == OP_ROOT_BEGIN) {
+                    r.out = v;   // the end of its block
+                    val[v].last = std::max(val[v].last, p);
+                    continue;
+                }
+            }
+        }
+        r.out = cur[out] = (int)val.size();
+        val.push_back({p, p, 0, -1, wide});
+    }
+    const int result = cur[out_slot];
+    val[result].last = L;
+    val[result].wide = true;   // read by channel after the program
+    // rows by first fit; an instruction's inputs that end there are free for its output
+    std::vector<int> ends(L + 1, -1);
+    for (size_t i = val.size(); i-- > 0;) {
+        val[i].next = ends[val[i].last];
+        ends[val[i].last] = (int)i;
+    }
+    RowSet set;
+    uint32_t rows = 0;
+    for (uint32_t p = 0; p < L; ++p) {
+        for (int i = ends[p]; i >= 0; i = val[i].next)
+            if (val[i].def < p) set.give(val[i].row, val[i].wide ? 3 : 1);
+        Value& v = val[refs[p].out];
+        if (v.def == p) {
+            v.row = set.take(v.wide ? 3 : 1);
+            rows = std::max(rows, v.row + (v.wide ? 3u : 1u));
+            if (v.last == p) set.give(v.row, v.wide ? 3 : 1);   // never read
+        }
+    }
+    if (rows > 3 * n_slots) {   // fragmentation: the slots as they were, three rows each
+        rows = 3 * n_slots;
+        for (uint32_t p = 0; p < L; ++p) val[refs[p].out].row = 3u * ((*prog)[p].y & 0xFFFFu);
+    }
+    for (uint32_t p = 0; p < L; ++p) {
+        uint4& ins = (*prog)[p];
+        const uint32_t op = ins.x & 0xFFu;
+        const Refs& r = refs[p];
+        const Value& v = val[r.out];
+        if (op >= OP_CONTROL) {
+            ins.y = v.row | (ins.y & 0xFFFF0000u);
+            continue;
+        }
+        uint32_t in[3];
+        bool w[3];
+        for (int k = 0; k < 3; ++k) {
+            in[k] = r.in[k] >= 0 ? val[r.in[k]].row : NO_SLOT;
+            w[k] = r.in[k] < 0 || val[r.in[k]].wide;
+        }
+        if ((op == PMC_OP_ADD || op == PMC_OP_MUL) && !w[0] && w[1]) {   // either order gives the same bits
+            std::swap(in[0], in[1]);
+            std::swap(w[0], w[1]);
+        }
+        const bool reads_pair = op == PMC_OP_UV_AFFINE || op == PMC_OP_FBM || op == PMC_OP_VORONOI || op == PMC_OP_FACING;
+        const uint32_t flags = (v.wide ? 0u : FLAG_ONE_ROW) | (reads_pair && !w[0] ? FLAG_ONE_IN : 0u);
+        ins.x = (ins.x & ~0xFFu) | device_op(op, w[0], w[1], v.wide, r.in[2] >= 0) | (flags << 8);
+        ins.y = v.row | (in[0] << 16);
+        ins.z = in[1] | (in[2] << 16);
+    }
+    *out_row = val[result].row;
+    return rows;
 }
 
 bool compile_material(const pmc_node* nodes_in, uint32_t n, uint32_t min_root_nodes, uint32_t min_root_cost,
@@ -377,25 +548,21 @@ bool compile_material(const pmc_node* nodes_in, uint32_t n, uint32_t min_root_no
         if (reach[i])
             for (int k = 0; k < 4; ++k)
                 if (g[i].in[k] >= 0) reach[g[i].in[k]] = 1;
-    std::vector<std::vector<uint32_t>> consumers(n);
-    for (uint32_t i = 0; i < n; ++i)
-        if (reach[i])
-            for (int k = 0; k < 4; ++k)
-                if (g[i].in[k] >= 0) consumers[g[i].in[k]].push_back(i);
-
     // ---- skip sets: -1 = always evaluate, r = skipped whenever root r hits -----------
-    const int32_t NEVER = -1;
-    std::vector<int32_t> guard(n, NEVER);
+    // every consumer of a node comes after it, so one sweep from the output down has each
+    // node's answers complete when it is reached
+    const int32_t NEVER = -1, NONE = -2;   // -2 = nothing seen yet
+    std::vector<int32_t> guard(n, NONE);
     for (int32_t i = (int32_t)n - 1; i >= 0; --i) {
-        if (!reach[i] || (uint32_t)i == out_node) continue;
-        int32_t gset = -2;  // -2 = nothing seen yet
-        for (uint32_t c : consumers[i]) {
-            int32_t contrib = is_root[c] ? (int32_t)c : guard[c];
-            if (contrib == NEVER) { gset = NEVER; break; }
-            if (gset == -2) gset = contrib;
-            else if (gset != contrib) { gset = NEVER; break; }  // shared by two roots
+        if (!reach[i]) continue;
+        if (guard[i] == NONE || (uint32_t)i == out_node) guard[i] = NEVER;
+        const int32_t contrib = is_root[i] ? i : guard[i];
+        for (int k = 0; k < 4; ++k) {
+            const int32_t y = g[i].in[k];
+            if (y < 0) continue;
+            if (guard[y] == NONE) guard[y] = contrib;
+            else if (guard[y] != contrib) guard[y] = NEVER;   // shared by two roots
         }
-        guard[i] = (gset == -2) ? NEVER : gset;
     }
     // block id of each node: the root whose block it belongs to, or -1
     std::vector<int32_t> block(n, -1);
@@ -497,9 +664,9 @@ bool compile_material(const pmc_node* nodes_in, uint32_t n, uint32_t min_root_no
     std::vector<uint32_t> slot(n, NO_SLOT);
     std::vector<uint32_t> free_slots;
     uint32_t n_slots = 0;
-    std::vector<std::vector<uint32_t>> release_at(L + 1);
-    for (uint32_t x = 0; x < n; ++x)
-        if (last_use[x] >= 0 && last_use[x] < (int64_t)L) release_at[last_use[x]].push_back(x);
+    ReleaseLists release_at(L, n);
+    for (uint32_t x = n; x-- > 0;)
+        if (last_use[x] >= 0 && last_use[x] < (int64_t)L) release_at.add((size_t)last_use[x], x);
     auto take = [&]() {
         if (free_slots.empty()) return n_slots++;
         auto it = std::min_element(free_slots.begin(), free_slots.end());
@@ -528,7 +695,7 @@ bool compile_material(const pmc_node* nodes_in, uint32_t n, uint32_t min_root_no
         uint32_t in_slot[3] = {NO_SLOT, NO_SLOT, NO_SLOT};
         for (int k = 0; k < 3; ++k)
             if (g[x].in[k] >= 0) in_slot[k] = slot[g[x].in[k]];
-        for (uint32_t y : release_at[p]) free_slots.push_back(slot[y]);
+        for (uint32_t y = release_at.head[p]; y != ~0u; y = release_at.next[y]) free_slots.push_back(slot[y]);
         if (!is_root[x]) slot[x] = take();
         uint4 ins;
         uint32_t flags = is_root[x] ? FLAG_ROOT : 0;
@@ -616,6 +783,16 @@ bool compile_material(const pmc_node* nodes_in, uint32_t n, uint32_t min_root_no
         out->outer_out_slot = os;
         if (out->outer_slots >= NO_SLOT) { *why = "too many live values"; return false; }
     }
+
+    // ---- rows of the slot file ----------------------------------------------------------
+    out->rows = compact_rows(&out->prog, out->params, out->n_slots, out->out_slot, &out->out_row);
+    out->outer_rows =
+        compact_rows(&out->outer_prog, out->params, out->outer_slots, out->outer_out_slot, &out->outer_out_row);
+    out->root_rows.assign(out->roots.size(), 0);
+    out->root_out_row.assign(out->roots.size(), 0);
+    for (size_t ri = 0; ri < out->roots.size(); ++ri)
+        out->root_rows[ri] = compact_rows(&out->root_progs[ri], out->params, out->root_slots[ri], out->root_out_slot[ri],
+                                          &out->root_out_row[ri]);
     return true;
 }
 

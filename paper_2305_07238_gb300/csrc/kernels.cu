@@ -536,13 +536,13 @@ __global__ void __launch_bounds__(256, 4) k_lookup(BatchArgs a) {
 constexpr uint32_t PROBE_COMPUTED = 3u;   // record {r, g, b, 3}: a miss evaluated this pass
 constexpr uint32_t EVAL_WARPS = 4;
 
-size_t eval_smem_bytes(uint32_t max_slots) {
-    return (size_t)EVAL_WARPS * max_slots * 3u * 32u * sizeof(float);
-}
+size_t eval_smem_bytes(uint32_t rows) { return (size_t)EVAL_WARPS * rows * ROW_BYTES; }
 
-// Largest slot file (bytes per block) with which the two-points-per-lane evaluator runs:
-// six blocks of its size fit an SM's shared memory.
-constexpr size_t EVAL2_MAX_SMEM = 36 * 1024;
+// Largest slot file (bytes per block) with which two points per lane run: four blocks of that size
+// fit an SM's shared memory.  Plain evaluation of 2 M points, two points against one per lane:
+// 42 KB 336 vs 388 us, 54 KB 458 vs 502, 66 KB 651 vs 654, 90 KB 998 vs 992: from there on the
+// warps that no longer fit cost what the shared decode saves.
+constexpr size_t EVAL2_MAX_SMEM = 56 * 1024;
 
 // Offers the lanes' freshly evaluated cacheable-node values to the table (Sec. 3).
 // `full`: the cell cannot take the value in this batch, so it is counted as dropped
@@ -602,17 +602,17 @@ struct FillStats {
 };
 
 // Offers the value (r, g, b) of cacheable node `node` at grouped point s (act: a valid
-// point); the point's level, texel and batch index are read here, where they are needed.
+// point); the point's inputs, level, texel and batch index are read here, where they are needed.
 __device__ __forceinline__ void fill_offer(const BatchArgs& a, bool act, uint32_t s, uint32_t m, uint32_t node, bool pos,
-                                           const PointIn& p, float r, float g, float b, FillStats* fs) {
+                                           float r, float g, float b, FillStats* fs) {
     uint32_t cell = 0, h2 = 0, orig = 0;
     if (act) {
         uint64_t key;
         if (pos) {
-            key = d_key_pos(m, node, (uint32_t)a.pos_level, p.px, p.py, p.pz);
+            key = d_key_pos(m, node, (uint32_t)a.pos_level, a.spx[s], a.spy[s], a.spz[s]);
         } else {
             const uint32_t lev = a.g1u ? (uint32_t)a.slev[s] : a.level;
-            key = d_key(m, node, lev, d_texel(p.u, lev), d_texel(p.v, lev));
+            key = d_key(m, node, lev, d_texel(a.su[s], lev), d_texel(a.sv[s], lev));
         }
         d_address(key, a.n_cells, a.cells_pow2_mask, &cell, &h2);
         orig = a.sidx[s];
@@ -621,30 +621,27 @@ __device__ __forceinline__ void fill_offer(const BatchArgs& a, bool act, uint32_
     offer(a, act, orig, node, cell, h2, 0u, false, r, g, b, &fs->n_cand, &fs->n_full);
 }
 
-// Per-point interpreter: one warp runs one material's program for 32 grouped points.
+// Per-point interpreter: one warp runs one material's program for 32 or 64 grouped points.
 // EVAL_OUTER: every cacheable node already has its value in its probe record (a hit, a
 //   value computed by k_eval_roots or a learned surrogate), so the outer program runs:
 //   each block replaced by a load of its node's record.
 // EVAL_PLAIN: the cache is off; the whole program runs for every point.
-// EVAL_FILL: the first pass on an empty table without surrogates (two points per lane only;
-//   see fill_offer).
-// EVAL_GENERIC: the whole program with per-lane skipping: the first pass on an empty table
-//   (descriptors formed here, every cacheable node offered), the inline evaluation of
-//   misses (a lane whose lookup hit skips the block), learned surrogates on that pass.
-// In the first two modes every lane runs every instruction: a lane past the end of its
+// EVAL_FILL: the first pass on an empty table without surrogates (see fill_offer).
+// In these modes every lane runs every instruction: a lane past the end of its
 // material's points shadows the segment's last point and stores nothing, and the node and
 // operation counts come from the program's totals.
-enum { EVAL_OUTER = 0, EVAL_PLAIN = 1, EVAL_GENERIC = 2, EVAL_FILL = 3 };
+// k_eval is the general form: the whole program with per-lane skipping, one point per lane: the
+//   inline evaluation of misses (a lane whose lookup hit skips the block), learned surrogates
+//   beside other cacheable nodes on the empty table (descriptors formed here).
+enum { EVAL_OUTER = 0, EVAL_PLAIN = 1, EVAL_FILL = 2 };
 
-template <int MODE>
 __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval(BatchArgs a, uint32_t* item_ctr) {
     extern __shared__ float s_val[];
     __shared__ float2 s_grad[8];
     init_gradients(s_grad);
     __syncthreads();
     const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-    constexpr bool outer = MODE == EVAL_OUTER;
-    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * (outer ? a.max_slots_outer : a.max_slots) * 96u + lane);
+    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * a.max_rows * 32u + lane);
     const uint32_t n_items = a.ctl->n_items;
     unsigned long long n_nodes = 0, n_flops = 0, n_cand = 0, n_full = 0, n_look = 0;
     for (;;) {
@@ -664,116 +661,85 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval(BatchArgs a, uint32_t*
         pt.nx = a.snx[s]; pt.ny = a.sny[s]; pt.nz = a.snz[s];
         const uint32_t orig = a.sidx[s];
         const MatInfo mi = a.mats[m];
-        const uint4* prog = a.prog + (outer ? mi.outer_start : mi.prog_start);
-        const uint32_t out_off = (outer ? mi.outer_out_slot : mi.out_slot) * SLOT_BYTES;
+        const uint4* prog = a.prog + mi.prog_start;
+        const uint32_t out_off = mi.out_row * ROW_BYTES;
         const uint32_t pbase = __ldg(&a.probe_base[m]);
-        const int len = (int)(outer ? mi.outer_len : mi.prog_len);
+        const int len = (int)mi.prog_len;
         uint32_t hits = 0;
-        if (outer) {
-            // the point's cacheable-node records, read by the program's loads: fetched into
-            // L1 now, so that the loads find them there instead of waiting on memory
-            const float4* rec0 = a.probes + (size_t)pbase + jj;
-            const uint32_t nr = min(mi.n_roots, 16u);
-            for (uint32_t r = 0; r < nr; ++r)
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(rec0 + (size_t)r * cnt));
-        }
         // the next instruction is fetched while the current one executes (the pool ends
         // with a padding instruction)
         uint4 nxt = __ldg(&prog[0]);
-        if (MODE != EVAL_GENERIC) {
-            for (int pc = 0; pc < len; ++pc) {
-                const uint4 ins = nxt;
-                nxt = __ldg(&prog[pc + 1]);
-                const uint32_t op = ins.x & 0xFFu;
-                if (outer && op == OP_LOAD_ROOT) {
-                    const float4 rec = a.probes[(size_t)pbase + (size_t)(ins.y >> 16) * cnt + jj];
+        int skip_end = -1;          // lane inactive while pc <= skip_end
+        uint32_t cand_cell = 0, cand_h2 = 0, cand_node = 0, cand_start = 0;
+        bool cand_full = false;
+        uint32_t iu = 0, iv = 0, lev = a.level;
+        if (a.keys_inline && valid) {
+            if (a.g1u) lev = a.slev[s];
+            iu = d_texel(pt.u, lev);
+            iv = d_texel(pt.v, lev);
+        }
+        for (int pc = 0; pc < len; ++pc) {
+            const uint4 ins = nxt;
+            nxt = __ldg(&prog[pc + 1]);
+            const uint32_t op = ins.x & 0xFFu;
+            if (op == OP_ROOT_BEGIN) {
+                const uint32_t off = ins.y & 0xFFFFu, r = ins.y >> 16;
+                bool need = valid;
+                // the node's probe record: a hit, a miss, or a value computed this pass
+                float4 rec = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (valid && ((a.use_cache && !a.keys_inline) || a.surr_ord))
+                    rec = a.probes[(size_t)pbase + (size_t)r * cnt + j];
+                if (a.surr_ord && a.surr_ord[m] == (int32_t)r) {
+                    // the learned surrogate already wrote this node's value
+                    if (valid) slot_store(Vb, off, rec.x, rec.y, rec.z);
+                    need = false;
+                } else if (a.keys_inline) {
+                    // empty table: every probe misses at slot 0, so the descriptor is all
+                    // the insert needs (no lookup kernel, no probe record)
+                    if (valid) {
+                        const uint64_t key = ((ins.x >> 8) & FLAG_POSROOT)
+                                                 ? d_key_pos(m, ins.z, (uint32_t)a.pos_level, pt.px, pt.py, pt.pz)
+                                                 : d_key(m, ins.z, lev, iu, iv);
+                        d_address(key, a.n_cells, a.cells_pow2_mask, &cand_cell, &cand_h2);
+                        cand_start = 0;
+                        cand_full = false;
+                        cand_node = ins.z;
+                        n_look++;
+                    }
+                } else if (a.use_cache && valid) {
                     const uint32_t state = __float_as_uint(rec.w);
-                    slot_store(Vb, ins.y & 0xFFFFu, rec.x, rec.y, rec.z);
-                    hits += state == PROBE_HIT ? 1u : 0u;
-                    // the batched evaluation or the surrogate must have given it a value
-                    if (valid && state != PROBE_HIT && state != PROBE_COMPUTED) atomicOr(&a.ctl->err, ERR_BOUNDS);
-                    continue;
-                }
-                if (!outer && op == OP_ROOT_BEGIN) continue;   // a block marker: nothing to skip
-                exec_node(op, ins, Vb, pt, a.params, s_grad);
-            }
-            if (valid) {
-                n_nodes += outer ? mi.outer_nodes : mi.full_nodes;
-                n_flops += outer ? mi.outer_flops : mi.full_flops;
-            }
-        } else {
-            int skip_end = -1;          // lane inactive while pc <= skip_end
-            uint32_t cand_cell = 0, cand_h2 = 0, cand_node = 0, cand_start = 0;
-            bool cand_full = false;
-            uint32_t iu = 0, iv = 0, lev = a.level;
-            if (a.keys_inline && valid) {
-                if (a.g1u) lev = a.slev[s];
-                iu = d_texel(pt.u, lev);
-                iv = d_texel(pt.v, lev);
-            }
-            for (int pc = 0; pc < len; ++pc) {
-                const uint4 ins = nxt;
-                nxt = __ldg(&prog[pc + 1]);
-                const uint32_t op = ins.x & 0xFFu;
-                if (op == OP_ROOT_BEGIN) {
-                    const uint32_t off = ins.y & 0xFFFFu, r = ins.y >> 16;
-                    bool need = valid;
-                    // the node's probe record: a hit, a miss, or a value computed this pass
-                    float4 rec = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (valid && ((a.use_cache && !a.keys_inline) || a.surr_ord))
-                        rec = a.probes[(size_t)pbase + (size_t)r * cnt + j];
-                    if (a.surr_ord && a.surr_ord[m] == (int32_t)r) {
-                        // the learned surrogate already wrote this node's value
-                        if (valid) slot_store(Vb, off, rec.x, rec.y, rec.z);
+                    if (state == PROBE_HIT || state == PROBE_COMPUTED) {
+                        slot_store(Vb, off, rec.x, rec.y, rec.z);
+                        hits += state == PROBE_HIT ? 1u : 0u;
                         need = false;
-                    } else if (a.keys_inline) {
-                        // empty table: every probe misses at slot 0, so the descriptor is all
-                        // the insert needs (no lookup kernel, no probe record)
-                        if (valid) {
-                            const uint64_t key = ((ins.x >> 8) & FLAG_POSROOT)
-                                                     ? d_key_pos(m, ins.z, (uint32_t)a.pos_level, pt.px, pt.py, pt.pz)
-                                                     : d_key(m, ins.z, lev, iu, iv);
-                            d_address(key, a.n_cells, a.cells_pow2_mask, &cand_cell, &cand_h2);
-                            cand_start = 0;
-                            cand_full = false;
-                            cand_node = ins.z;
-                            n_look++;
-                        }
-                    } else if (a.use_cache && valid) {
-                        const uint32_t state = __float_as_uint(rec.w);
-                        if (state == PROBE_HIT || state == PROBE_COMPUTED) {
-                            slot_store(Vb, off, rec.x, rec.y, rec.z);
-                            hits += state == PROBE_HIT ? 1u : 0u;
-                            need = false;
-                        } else if (a.split) {
-                            atomicOr(&a.ctl->err, ERR_BOUNDS);   // the batched evaluation missed it
-                            need = false;
-                        } else {
-                            cand_cell = __float_as_uint(rec.x);
-                            cand_h2 = __float_as_uint(rec.y);
-                            cand_start = __float_as_uint(rec.z);
-                            cand_full = state == PROBE_FULL;
-                            cand_node = ins.z;
-                        }
+                    } else if (a.split) {
+                        atomicOr(&a.ctl->err, ERR_BOUNDS);   // the batched evaluation missed it
+                        need = false;
+                    } else {
+                        cand_cell = __float_as_uint(rec.x);
+                        cand_h2 = __float_as_uint(rec.y);
+                        cand_start = __float_as_uint(rec.z);
+                        cand_full = state == PROBE_FULL;
+                        cand_node = ins.z;
                     }
-                    if (!need) skip_end = pc + (int)ins.w;
-                    if (__all_sync(FULL_MASK, !need)) {
-                        pc += (int)ins.w;
-                        nxt = __ldg(&prog[pc + 1]);
-                    }
-                    continue;
                 }
-                const bool act = valid && pc > skip_end;
-                if (act) {
-                    exec_node(op, ins, Vb, pt, a.params, s_grad);
-                    n_nodes++;
-                    n_flops += ins.x >> 16;
+                if (!need) skip_end = pc + (int)ins.w;
+                if (__all_sync(FULL_MASK, !need)) {
+                    pc += (int)ins.w;
+                    nxt = __ldg(&prog[pc + 1]);
                 }
-                if (a.use_cache && ((ins.x >> 8) & FLAG_ROOT)) {
-                    const uint32_t out = ins.y & 0xFFFFu;
-                    offer(a, act, orig, cand_node, cand_cell, cand_h2, cand_start, cand_full, slot_ch(Vb, out, 0),
-                          slot_ch(Vb, out, 1), slot_ch(Vb, out, 2), &n_cand, &n_full);
-                }
+                continue;
+            }
+            const bool act = valid && pc > skip_end;
+            if (act) {
+                exec_points<float>(ins, Vb, PointRegs{pt}, PointRegs{pt}, a.params, s_grad);
+                n_nodes++;
+                n_flops += ins.x >> 16;
+            }
+            if (a.use_cache && ((ins.x >> 8) & FLAG_ROOT)) {
+                const uint32_t out = ins.y & 0xFFFFu;
+                offer(a, act, orig, cand_node, cand_cell, cand_h2, cand_start, cand_full, slot_ch(Vb, out, 0),
+                      slot_ch(Vb, out, 1), slot_ch(Vb, out, 2), &n_cand, &n_full);
             }
         }
         if (valid) {
@@ -785,20 +751,25 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval(BatchArgs a, uint32_t*
     }
     warp_add_u64(&a.stats[ST_NODES], n_nodes);
     warp_add_u64(&a.stats[ST_FLOPS], n_flops);
-    if (MODE == EVAL_GENERIC) {
-        warp_add_u64(&a.stats[ST_CANDIDATES], n_cand);
-        warp_add_u64(&a.stats[ST_FULL], n_full);
-        warp_add_u32(&a.ctl->w_cand, (uint32_t)(n_cand - n_full));
-        if (a.keys_inline) {
-            warp_add_u64(&a.stats[ST_LOOKUPS], n_look);
-            warp_add_u64(&a.stats[ST_MISSES], n_look);
-            warp_add_u64(&a.stats[ST_SLOTS], n_look);   // one (empty) slot examined per probe
-        }
+    warp_add_u64(&a.stats[ST_CANDIDATES], n_cand);
+    warp_add_u64(&a.stats[ST_FULL], n_full);
+    warp_add_u32(&a.ctl->w_cand, (uint32_t)(n_cand - n_full));
+    if (a.keys_inline) {
+        warp_add_u64(&a.stats[ST_LOOKUPS], n_look);
+        warp_add_u64(&a.stats[ST_MISSES], n_look);
+        warp_add_u64(&a.stats[ST_SLOTS], n_look);   // one (empty) slot examined per probe
     }
 }
 
+// The eight inputs of grouped point s into L1, ahead of the program's input nodes.
+__device__ __forceinline__ void prefetch_point(const BatchArgs& a, uint32_t s) {
+    const float* f[8] = {a.su, a.sv, a.spx, a.spy, a.spz, a.snx, a.sny, a.snz};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) asm volatile("prefetch.global.L1 [%0];" ::"l"(f[k] + s));
+}
+
 // One 32-point item of the modes in which every lane runs every instruction (EVAL_OUTER,
-// EVAL_PLAIN, EVAL_FILL), one point per lane (Vb: the lane's base in a [slot][channel][lane]
+// EVAL_PLAIN, EVAL_FILL), one point per lane (Vb: the lane's base in a [row][lane]
 // file).
 template <int MODE>
 __device__ __forceinline__ void eval_item1(const BatchArgs& a, uint32_t item, uint32_t m, char* Vb, const float2* grad,
@@ -810,62 +781,62 @@ __device__ __forceinline__ void eval_item1(const BatchArgs& a, uint32_t item, ui
     const bool valid = j < cnt;
     const uint32_t jj = valid ? j : cnt - 1u;   // an idle lane shadows the segment's last point
     const uint32_t s = __ldg(&a.seg_start[m]) + jj;
-    PointIn pt;
-    pt.u = a.su[s]; pt.v = a.sv[s];
-    pt.px = a.spx[s]; pt.py = a.spy[s]; pt.pz = a.spz[s];
-    pt.nx = a.snx[s]; pt.ny = a.sny[s]; pt.nz = a.snz[s];
-    const uint32_t orig = a.sidx[s];
-    const MatInfo mi = a.mats[m];
-    const uint4* prog = a.prog + (outer ? mi.outer_start : mi.prog_start);
-    const uint32_t out_off = (outer ? mi.outer_out_slot : mi.out_slot) * SLOT_BYTES;
+    const PointMem pt{a, s};
+    prefetch_point(a, s);
+    const MatInfo* mi = a.mats + m;
     const uint32_t pbase = __ldg(&a.probe_base[m]);
-    const int len = (int)(outer ? mi.outer_len : mi.prog_len);
     uint32_t hits = 0;
     if (outer) {
+        // the point's cacheable-node records, read by the program's loads: fetched into
+        // L1 now, so that the loads find them there instead of waiting on memory
         const float4* rec0 = a.probes + (size_t)pbase + jj;
-        const uint32_t nr = min(mi.n_roots, 16u);
+        const uint32_t nr = min(mi->n_roots, 16u);
         for (uint32_t r = 0; r < nr; ++r) asm volatile("prefetch.global.L1 [%0];" ::"l"(rec0 + (size_t)r * cnt));
     }
     uint32_t cnode = 0;
     bool cpos = false;
-    uint4 nxt = __ldg(&prog[0]);   // the pool ends with a padding instruction
-    for (int pc = 0; pc < len; ++pc) {
+    // the next instruction is fetched while the current one executes (the pool ends
+    // with a padding instruction)
+    const uint4* pc = a.prog + (outer ? mi->outer_start : mi->prog_start);
+    uint4 nxt = __ldg(pc);
+    for (;;) {
         const uint4 ins = nxt;
-        nxt = __ldg(&prog[pc + 1]);
-        const uint32_t op = ins.x & 0xFFu;
-        if (outer && op == OP_LOAD_ROOT) {
-            const float4 rec = a.probes[(size_t)pbase + (size_t)(ins.y >> 16) * cnt + jj];
-            const uint32_t state = __float_as_uint(rec.w);
-            slot_store(Vb, ins.y & 0xFFFFu, rec.x, rec.y, rec.z);
-            hits += state == PROBE_HIT ? 1u : 0u;
-            if (valid && state != PROBE_HIT && state != PROBE_COMPUTED) atomicOr(&a.ctl->err, ERR_BOUNDS);
-            continue;
-        }
-        if (!outer && op == OP_ROOT_BEGIN) {
-            if (MODE == EVAL_FILL) {
+        nxt = __ldg(++pc);
+        if (ins.x & OP_CONTROL) {
+            if ((ins.x & 0xFFu) == OP_END) break;
+            if (outer) {   // OP_LOAD_ROOT
+                const float4 rec = a.probes[(size_t)pbase + (size_t)(ins.y >> 16) * cnt + jj];
+                const uint32_t state = __float_as_uint(rec.w);
+                slot_store(Vb, ins.y & 0xFFFFu, rec.x, rec.y, rec.z);
+                hits += state == PROBE_HIT ? 1u : 0u;
+                // the batched evaluation or the surrogate must have given it a value
+                if (valid && state != PROBE_HIT && state != PROBE_COMPUTED) atomicOr(&a.ctl->err, ERR_BOUNDS);
+            } else if (MODE == EVAL_FILL) {   // OP_ROOT_BEGIN
                 cnode = ins.z;
                 cpos = ((ins.x >> 8) & FLAG_POSROOT) != 0;
             }
             continue;
         }
-        exec_node(op, ins, Vb, pt, a.params, grad);
+        exec_points<float>(ins, Vb, pt, pt, a.params, grad);
         if (MODE == EVAL_FILL && ((ins.x >> 8) & FLAG_ROOT)) {
             const uint32_t o = ins.y & 0xFFFFu;
-            fill_offer(a, valid, s, m, cnode, cpos, pt, slot_ch(Vb, o, 0), slot_ch(Vb, o, 1), slot_ch(Vb, o, 2), fs);
+            fill_offer(a, valid, s, m, cnode, cpos, slot_ch(Vb, o, 0), slot_ch(Vb, o, 1), slot_ch(Vb, o, 2), fs);
         }
     }
+    const uint32_t out_off = (outer ? mi->outer_out_row : mi->out_row) * ROW_BYTES;
     if (valid) {
+        const uint32_t orig = a.sidx[s];
         a.out_rgb[orig] = slot_ch(Vb, out_off, 0);
         a.out_rgb[(size_t)a.n + orig] = slot_ch(Vb, out_off, 1);
         a.out_rgb[2 * (size_t)a.n + orig] = slot_ch(Vb, out_off, 2);
         if (a.out_hits) a.out_hits[orig] = (uint16_t)min(hits, 65535u);
-        *n_nodes += outer ? mi.outer_nodes : mi.full_nodes;
-        *n_flops += outer ? mi.outer_flops : mi.full_flops;
+        *n_nodes += outer ? mi->outer_nodes : mi->full_nodes;
+        *n_flops += outer ? mi->outer_flops : mi->full_flops;
     }
 }
 
 // Two consecutive 32-point items of one material, two points per lane (A from the first
-// item, B from the second; Vb: the lane's base in a [slot][channel][lane][2] file).
+// item, B from the second; Vb: the lane's base in a [row][lane][2] file).
 template <int MODE>
 __device__ __forceinline__ void eval_item2(const BatchArgs& a, uint32_t item, uint32_t m, char* Vb, const float2* grad,
                                            unsigned long long* n_nodes, unsigned long long* n_flops, FillStats* fs) {
@@ -877,21 +848,16 @@ __device__ __forceinline__ void eval_item2(const BatchArgs& a, uint32_t item, ui
     const uint32_t jA = vA ? j : cnt - 1u, jB = vB ? j + 32u : cnt - 1u;
     const uint32_t s0 = __ldg(&a.seg_start[m]);
     const uint32_t sA = s0 + jA, sB = s0 + jB;
-    PointIn A, B;
-    A.u = a.su[sA]; A.v = a.sv[sA]; A.px = a.spx[sA]; A.py = a.spy[sA]; A.pz = a.spz[sA];
-    A.nx = a.snx[sA]; A.ny = a.sny[sA]; A.nz = a.snz[sA];
-    B.u = a.su[sB]; B.v = a.sv[sB]; B.px = a.spx[sB]; B.py = a.spy[sB]; B.pz = a.spz[sB];
-    B.nx = a.snx[sB]; B.ny = a.sny[sB]; B.nz = a.snz[sB];
-    const MatInfo mi = a.mats[m];
-    const uint4* prog = a.prog + (outer ? mi.outer_start : mi.prog_start);
-    const uint32_t out_off = (outer ? mi.outer_out_slot : mi.out_slot) * SLOT_BYTES;
+    const PointMem A{a, sA}, B{a, sB};
+    prefetch_point(a, sA);
+    prefetch_point(a, sB);
+    const MatInfo* mi = a.mats + m;
     const uint32_t pbase = __ldg(&a.probe_base[m]);
-    const int len = (int)(outer ? mi.outer_len : mi.prog_len);
     uint32_t hA = 0, hB = 0;
     if (outer) {
         const float4* ra = a.probes + (size_t)pbase + jA;
         const float4* rb = a.probes + (size_t)pbase + jB;
-        const uint32_t nr = min(mi.n_roots, 16u);
+        const uint32_t nr = min(mi->n_roots, 16u);
         for (uint32_t r = 0; r < nr; ++r) {
             asm volatile("prefetch.global.L1 [%0];" ::"l"(ra + (size_t)r * cnt));
             asm volatile("prefetch.global.L1 [%0];" ::"l"(rb + (size_t)r * cnt));
@@ -899,37 +865,37 @@ __device__ __forceinline__ void eval_item2(const BatchArgs& a, uint32_t item, ui
     }
     uint32_t cnode = 0;
     bool cpos = false;
-    uint4 nxt = __ldg(&prog[0]);
-    for (int pc = 0; pc < len; ++pc) {
+    const uint4* pc = a.prog + (outer ? mi->outer_start : mi->prog_start);
+    uint4 nxt = __ldg(pc);
+    for (;;) {
         const uint4 ins = nxt;
-        nxt = __ldg(&prog[pc + 1]);
-        const uint32_t op = ins.x & 0xFFu;
-        if (outer && op == OP_LOAD_ROOT) {
-            const size_t rb = (size_t)pbase + (size_t)(ins.y >> 16) * cnt;
-            const float4 ra = a.probes[rb + jA], rc = a.probes[rb + jB];
-            const uint32_t sa = __float_as_uint(ra.w), sc = __float_as_uint(rc.w);
-            slot2_store(Vb, ins.y & 0xFFFFu, f2(ra.x, rc.x), f2(ra.y, rc.y), f2(ra.z, rc.z));
-            hA += sa == PROBE_HIT ? 1u : 0u;
-            hB += sc == PROBE_HIT ? 1u : 0u;
-            if ((vA && sa != PROBE_HIT && sa != PROBE_COMPUTED) || (vB && sc != PROBE_HIT && sc != PROBE_COMPUTED))
-                atomicOr(&a.ctl->err, ERR_BOUNDS);
-            continue;
-        }
-        if (!outer && op == OP_ROOT_BEGIN) {
-            if (MODE == EVAL_FILL) {
+        nxt = __ldg(++pc);
+        if (ins.x & OP_CONTROL) {
+            if ((ins.x & 0xFFu) == OP_END) break;
+            if (outer) {   // OP_LOAD_ROOT
+                const size_t rb = (size_t)pbase + (size_t)(ins.y >> 16) * cnt;
+                const float4 ra = a.probes[rb + jA], rc = a.probes[rb + jB];
+                const uint32_t sa = __float_as_uint(ra.w), sc = __float_as_uint(rc.w);
+                slot2_store(Vb, ins.y & 0xFFFFu, f2(ra.x, rc.x), f2(ra.y, rc.y), f2(ra.z, rc.z));
+                hA += sa == PROBE_HIT ? 1u : 0u;
+                hB += sc == PROBE_HIT ? 1u : 0u;
+                if ((vA && sa != PROBE_HIT && sa != PROBE_COMPUTED) || (vB && sc != PROBE_HIT && sc != PROBE_COMPUTED))
+                    atomicOr(&a.ctl->err, ERR_BOUNDS);
+            } else if (MODE == EVAL_FILL) {   // OP_ROOT_BEGIN
                 cnode = ins.z;
                 cpos = ((ins.x >> 8) & FLAG_POSROOT) != 0;
             }
             continue;
         }
-        exec_node2(op, ins, Vb, A, B, a.params, grad);
+        exec_points<float2>(ins, Vb, A, B, a.params, grad);
         if (MODE == EVAL_FILL && ((ins.x >> 8) & FLAG_ROOT)) {
             const uint32_t o = ins.y & 0xFFFFu;
             const float2 c0 = slot2(Vb, o, 0), c1 = slot2(Vb, o, 1), c2 = slot2(Vb, o, 2);
-            fill_offer(a, vA, sA, m, cnode, cpos, A, c0.x, c1.x, c2.x, fs);
-            fill_offer(a, vB, sB, m, cnode, cpos, B, c0.y, c1.y, c2.y, fs);
+            fill_offer(a, vA, sA, m, cnode, cpos, c0.x, c1.x, c2.x, fs);
+            fill_offer(a, vB, sB, m, cnode, cpos, c0.y, c1.y, c2.y, fs);
         }
     }
+    const uint32_t out_off = (outer ? mi->outer_out_row : mi->out_row) * ROW_BYTES;
     const float2 o0 = slot2(Vb, out_off, 0), o1 = slot2(Vb, out_off, 1), o2 = slot2(Vb, out_off, 2);
     const uint32_t nv = (vA ? 1u : 0u) + (vB ? 1u : 0u);
     if (vA) {
@@ -946,15 +912,58 @@ __device__ __forceinline__ void eval_item2(const BatchArgs& a, uint32_t item, ui
         a.out_rgb[2 * (size_t)a.n + ob] = o2.y;
         if (a.out_hits) a.out_hits[ob] = (uint16_t)min(hB, 65535u);
     }
-    *n_nodes += (unsigned long long)nv * (outer ? mi.outer_nodes : mi.full_nodes);
-    *n_flops += (unsigned long long)nv * (outer ? mi.outer_flops : mi.full_flops);
+    *n_nodes += (unsigned long long)nv * (outer ? mi->outer_nodes : mi->full_nodes);
+    *n_flops += (unsigned long long)nv * (outer ? mi->outer_flops : mi->full_flops);
 }
 
-// EVAL_OUTER and EVAL_PLAIN with two points per lane: a warp takes pairs of consecutive
+__device__ __forceinline__ void fill_stats(const BatchArgs& a, const FillStats& fs) {
+    warp_add_u64(&a.stats[ST_CANDIDATES], fs.n_cand);
+    warp_add_u64(&a.stats[ST_FULL], fs.n_full);
+    warp_add_u32(&a.ctl->w_cand, (uint32_t)(fs.n_cand - fs.n_full));
+    warp_add_u64(&a.stats[ST_LOOKUPS], fs.n_look);
+    warp_add_u64(&a.stats[ST_MISSES], fs.n_look);
+    warp_add_u64(&a.stats[ST_SLOTS], fs.n_look);   // one (empty) slot examined per probe
+}
+
+// EVAL_OUTER, EVAL_PLAIN and EVAL_FILL with one point per lane: every warp claims an item at a
+// time.
+template <int MODE>
+__global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval1(BatchArgs a, uint32_t* item_ctr) {
+    extern __shared__ float s_val[];
+    __shared__ float2 s_grad[8];
+    init_gradients(s_grad);
+    __syncthreads();
+    const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+    const uint32_t rows = MODE == EVAL_OUTER ? a.max_rows_outer : a.max_rows;
+    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * rows * 32u + lane);
+    const uint32_t n_items = a.ctl->n_items;
+    unsigned long long n_nodes = 0, n_flops = 0;
+    FillStats fs;
+    for (;;) {
+        uint32_t item = 0;
+        if (lane == 0) item = atomicAdd(item_ctr, 1u);
+        item = __shfl_sync(FULL_MASK, item, 0);
+        if (item >= n_items) break;
+        eval_item1<MODE>(a, item, find_material(a.item_base, a.n_mats, item), Vb, s_grad, &n_nodes, &n_flops, &fs);
+    }
+    warp_add_u64(&a.stats[ST_NODES], n_nodes);
+    warp_add_u64(&a.stats[ST_FLOPS], n_flops);
+    if (MODE == EVAL_FILL) fill_stats(a, fs);
+}
+
+// EVAL_OUTER, EVAL_PLAIN and EVAL_FILL with two points per lane: a warp takes pairs of consecutive
 // items; a pair that straddles two materials runs as two single items.  BLOCK: the block
 // claims a tile of EVAL_WARPS consecutive pairs at a time (block-per-material work: the
 // warps of a block run one material's program together and share its instruction and
 // parameter lines in L1); else every warp claims its own pair.
+// Bound by instruction issue (80 % of the issue slots in use), so what counts is instructions
+// per node: 74 per octave of noise and point (four lattice hashes, their integer work on the ALU
+// pipe), 197 per Worley node, about 29 around any node for fetch, decode and dispatch.  Hence:
+// no point data held across the program (72 registers hold seven blocks per SM; eight blocks at
+// 64 spill: 6,626 vs 6,250 us for the frame's evaluation), no operand kinds tested at run time, one
+// row for values with equal channels, floors through packed additions.  Measured, one pass of
+// 2.07 M points over 64 networks of 20-200 nodes: plain 753 -> 621 us (12.7 -> 15.4 TFLOP/s, 19 % of the
+// FP32 peak), outer programs 393 -> 357 us; 1024 networks of 5-2000 nodes, two passes 10,080 -> 7,816 us.
 template <int MODE, bool BLOCK>
 __global__ void __launch_bounds__(EVAL_WARPS * 32, MODE == EVAL_FILL ? 6 : 7) k_eval2(BatchArgs a, uint32_t* item_ctr) {
     extern __shared__ float s_val[];
@@ -963,9 +972,9 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32, MODE == EVAL_FILL ? 6 : 7) k_
     init_gradients(s_grad);
     __syncthreads();
     const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-    const uint32_t slots = MODE == EVAL_OUTER ? a.max_slots_outer : a.max_slots;
+    const uint32_t rows = MODE == EVAL_OUTER ? a.max_rows_outer : a.max_rows;
     FillStats fs;
-    char* Vw = reinterpret_cast<char*>(s_val + (size_t)warp * slots * 192u);
+    char* Vw = reinterpret_cast<char*>(s_val + (size_t)warp * rows * 64u);
     char* Vb2 = Vw + lane * 8u;
     char* Vb1 = Vw + lane * 4u;
     const uint32_t n_items = a.ctl->n_items;
@@ -1000,14 +1009,7 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32, MODE == EVAL_FILL ? 6 : 7) k_
     }
     warp_add_u64(&a.stats[ST_NODES], n_nodes);
     warp_add_u64(&a.stats[ST_FLOPS], n_flops);
-    if (MODE == EVAL_FILL) {
-        warp_add_u64(&a.stats[ST_CANDIDATES], fs.n_cand);
-        warp_add_u64(&a.stats[ST_FULL], fs.n_full);
-        warp_add_u32(&a.ctl->w_cand, (uint32_t)(fs.n_cand - fs.n_full));
-        warp_add_u64(&a.stats[ST_LOOKUPS], fs.n_look);
-        warp_add_u64(&a.stats[ST_MISSES], fs.n_look);
-        warp_add_u64(&a.stats[ST_SLOTS], fs.n_look);   // one (empty) slot examined per probe
-    }
+    if (MODE == EVAL_FILL) fill_stats(a, fs);
 }
 
 // Scans cell `cell` for h2 (Alg. 1's entry loop read as a lookup): the first slot that
@@ -1150,7 +1152,7 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_fused(BatchArgs a, uin
     init_gradients(s_grad);
     __syncthreads();
     const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * a.max_slots * 96u + lane);
+    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * a.max_rows * 32u + lane);
     const uint32_t n_chunks = GROUPED ? a.ctl->n_items : (a.n + 31u) >> 5;
     const uint32_t ne = a.n_entries;
     unsigned long long n_nodes = 0, n_flops = 0, n_cand = 0, n_full = 0;
@@ -1280,7 +1282,7 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_fused(BatchArgs a, uin
                 }
                 const bool act = mine && pc > skip_end;
                 if (act) {
-                    exec_node(op, ins, Vb, pt, a.params, s_grad);
+                    exec_points<float>(ins, Vb, PointRegs{pt}, PointRegs{pt}, a.params, s_grad);
                     n_nodes++;
                     n_flops += ins.x >> 16;
                 }
@@ -1299,7 +1301,7 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_fused(BatchArgs a, uin
                 }
             }
             if (mine) {
-                const uint32_t oo = mi.out_slot * SLOT_BYTES;
+                const uint32_t oo = mi.out_row * ROW_BYTES;
                 a.out_rgb[i] = slot_ch(Vb, oo, 0);
                 a.out_rgb[(size_t)a.n + i] = slot_ch(Vb, oo, 1);
                 a.out_rgb[2 * (size_t)a.n + i] = slot_ch(Vb, oo, 2);
@@ -1338,8 +1340,7 @@ struct RootStats {
 };
 
 // One item (32 misses of one cacheable node), one miss per lane (Vb: the lane's base in a
-// [slot][channel][lane] file).
-template <bool POS>
+// [row][lane] file).
 __device__ __forceinline__ void roots_item1(const BatchArgs& a, uint32_t item, uint32_t q, char* Vb, const float2* grad,
                                             RootStats* st) {
     const uint32_t lane = lane_id();
@@ -1354,30 +1355,23 @@ __device__ __forceinline__ void roots_item1(const BatchArgs& a, uint32_t item, u
     const size_t base = pbase + (size_t)r * cnt;
     const uint32_t j = a.misslist[base + (valid ? idx : nm - 1u)];
     const uint32_t s = __ldg(&a.seg_start[m]) + j;
-    PointIn pt{0, 0, 0, 0, 0, 0, 0, 0};
-    pt.u = a.su[s];
-    pt.v = a.sv[s];
-    if (POS) {   // a position-class node reads the position
-        pt.px = a.spx[s];
-        pt.py = a.spy[s];
-        pt.pz = a.spz[s];
-    }
+    const PointMem pt{a, s};
     const uint32_t orig = a.sidx[s];
     const float4 rec = a.probes[base + j];
-    const uint4* prog = a.prog + ri.prog_start;
-    uint4 nxt = __ldg(&prog[0]);   // the pool ends with a padding instruction
-    for (uint32_t pc = 0; pc < ri.prog_len; ++pc) {
+    const uint4* pc = a.prog + ri.prog_start;
+    uint4 nxt = __ldg(pc);   // the pool ends with a padding instruction
+    for (;;) {
         const uint4 ins = nxt;
-        nxt = __ldg(&prog[pc + 1]);
-        const uint32_t op = ins.x & 0xFFu;
-        if (op == OP_LOAD_ROOT) {
-            const float4 v = a.probes[pbase + (size_t)(ins.y >> 16) * cnt + j];
+        nxt = __ldg(++pc);
+        if (ins.x & OP_CONTROL) {
+            if ((ins.x & 0xFFu) == OP_END) break;
+            const float4 v = a.probes[pbase + (size_t)(ins.y >> 16) * cnt + j];   // OP_LOAD_ROOT
             slot_store(Vb, ins.y & 0xFFFFu, v.x, v.y, v.z);
             continue;
         }
-        exec_node(op, ins, Vb, pt, a.params, grad);
+        exec_points<float>(ins, Vb, pt, pt, a.params, grad);
     }
-    const uint32_t out_off = ri.out_slot * SLOT_BYTES;
+    const uint32_t out_off = ri.out_row * ROW_BYTES;
     const float v0 = slot_ch(Vb, out_off, 0), v1 = slot_ch(Vb, out_off, 1), v2 = slot_ch(Vb, out_off, 2);
     if (valid) {
         a.probes[base + j] = make_float4(v0, v1, v2, __uint_as_float(PROBE_COMPUTED));
@@ -1389,8 +1383,7 @@ __device__ __forceinline__ void roots_item1(const BatchArgs& a, uint32_t item, u
 }
 
 // Two consecutive items of one cacheable node, two misses per lane (A from the first item,
-// B from the second; Vb: the lane's base in a [slot][channel][lane][2] file).
-template <bool POS>
+// B from the second; Vb: the lane's base in a [row][lane][2] file).
 __device__ __forceinline__ void roots_item2(const BatchArgs& a, uint32_t item, uint32_t q, char* Vb, const float2* grad,
                                             RootStats* st) {
     const uint32_t lane = lane_id();
@@ -1406,31 +1399,25 @@ __device__ __forceinline__ void roots_item2(const BatchArgs& a, uint32_t item, u
     const uint32_t jA = a.misslist[base + (vA ? iA : nm - 1u)], jB = a.misslist[base + (vB ? iB : nm - 1u)];
     const uint32_t s0 = __ldg(&a.seg_start[m]);
     const uint32_t sA = s0 + jA, sB = s0 + jB;
-    PointIn A{0, 0, 0, 0, 0, 0, 0, 0}, B{0, 0, 0, 0, 0, 0, 0, 0};
-    A.u = a.su[sA]; A.v = a.sv[sA];
-    B.u = a.su[sB]; B.v = a.sv[sB];
-    if (POS) {
-        A.px = a.spx[sA]; A.py = a.spy[sA]; A.pz = a.spz[sA];
-        B.px = a.spx[sB]; B.py = a.spy[sB]; B.pz = a.spz[sB];
-    }
+    const PointMem A{a, sA}, B{a, sB};
     // the miss records and batch indices the offers need, loaded while the program runs
     const float4 recA = a.probes[base + jA], recB = a.probes[base + jB];
     const uint32_t oA = a.sidx[sA], oB = a.sidx[sB];
-    const uint4* prog = a.prog + ri.prog_start;
-    uint4 nxt = __ldg(&prog[0]);
-    for (uint32_t pc = 0; pc < ri.prog_len; ++pc) {
+    const uint4* pc = a.prog + ri.prog_start;
+    uint4 nxt = __ldg(pc);
+    for (;;) {
         const uint4 ins = nxt;
-        nxt = __ldg(&prog[pc + 1]);
-        const uint32_t op = ins.x & 0xFFu;
-        if (op == OP_LOAD_ROOT) {
-            const size_t rb = pbase + (size_t)(ins.y >> 16) * cnt;
+        nxt = __ldg(++pc);
+        if (ins.x & OP_CONTROL) {
+            if ((ins.x & 0xFFu) == OP_END) break;
+            const size_t rb = pbase + (size_t)(ins.y >> 16) * cnt;   // OP_LOAD_ROOT
             const float4 ra = a.probes[rb + jA], rc = a.probes[rb + jB];
             slot2_store(Vb, ins.y & 0xFFFFu, f2(ra.x, rc.x), f2(ra.y, rc.y), f2(ra.z, rc.z));
             continue;
         }
-        exec_node2(op, ins, Vb, A, B, a.params, grad);
+        exec_points<float2>(ins, Vb, A, B, a.params, grad);
     }
-    const uint32_t out_off = ri.out_slot * SLOT_BYTES;
+    const uint32_t out_off = ri.out_row * ROW_BYTES;
     const float2 o0 = slot2(Vb, out_off, 0), o1 = slot2(Vb, out_off, 1), o2 = slot2(Vb, out_off, 2);
     if (vA) {
         a.probes[base + jA] = make_float4(o0.x, o1.x, o2.x, __uint_as_float(PROBE_COMPUTED));
@@ -1457,14 +1444,13 @@ __device__ __forceinline__ void roots_stats(const BatchArgs& a, const RootStats&
     warp_add_u32(&a.ctl->w_cand, (uint32_t)(st.n_cand - st.n_full));
 }
 
-template <bool POS>
 __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_roots(BatchArgs a, uint32_t level, uint32_t* item_ctr) {
     extern __shared__ float s_val[];
     __shared__ float2 s_grad[8];
     init_gradients(s_grad);
     __syncthreads();
     const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * a.max_slots_roots * 96u + lane);
+    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * a.max_rows_roots * 32u + lane);
     // this level's items only: they are contiguous in the level-ordered item layout
     const uint32_t* level_items = a.root_item_base + a.n_roots_total + 1;
     const uint32_t first = level_items[level], end = level_items[level + 1];
@@ -1474,7 +1460,7 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_roots(BatchArgs a, uin
         if (lane == 0) item = first + atomicAdd(item_ctr, 1u);
         item = __shfl_sync(FULL_MASK, item, 0);
         if (item >= end) break;
-        roots_item1<POS>(a, item, find_material(a.root_item_base, a.n_roots_total, item), Vb, s_grad, &st);
+        roots_item1(a, item, find_material(a.root_item_base, a.n_roots_total, item), Vb, s_grad, &st);
     }
     roots_stats(a, st);
 }
@@ -1482,14 +1468,13 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_roots(BatchArgs a, uin
 // The same with two misses per lane: a warp takes pairs of consecutive items (the item
 // counter counts pairs); a pair whose items belong to two cacheable nodes runs as two
 // single items.
-template <bool POS>
 __global__ void __launch_bounds__(EVAL_WARPS * 32, 6) k_eval_roots2(BatchArgs a, uint32_t level, uint32_t* item_ctr) {
     extern __shared__ float s_val[];
     __shared__ float2 s_grad[8];
     init_gradients(s_grad);
     __syncthreads();
     const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-    char* Vw = reinterpret_cast<char*>(s_val + (size_t)warp * a.max_slots_roots * 192u);
+    char* Vw = reinterpret_cast<char*>(s_val + (size_t)warp * a.max_rows_roots * 64u);
     char* Vb2 = Vw + lane * 8u;
     char* Vb1 = Vw + lane * 4u;
     const uint32_t* level_items = a.root_item_base + a.n_roots_total + 1;
@@ -1503,11 +1488,11 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32, 6) k_eval_roots2(BatchArgs a,
         if (it >= end) break;
         const uint32_t q = find_material(a.root_item_base, a.n_roots_total, it);
         if (it + 1u < end && it + 1u < a.root_item_base[q + 1]) {
-            roots_item2<POS>(a, it, q, Vb2, s_grad, &st);
+            roots_item2(a, it, q, Vb2, s_grad, &st);
         } else {
-            roots_item1<POS>(a, it, q, Vb1, s_grad, &st);
+            roots_item1(a, it, q, Vb1, s_grad, &st);
             if (it + 1u < end)
-                roots_item1<POS>(a, it + 1u, find_material(a.root_item_base, a.n_roots_total, it + 1u), Vb1, s_grad,
+                roots_item1(a, it + 1u, find_material(a.root_item_base, a.n_roots_total, it + 1u), Vb1, s_grad,
                                  &st);
         }
     }
@@ -3001,7 +2986,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
         if ((e = mark(2)) != cudaSuccess) return e;
         if ((e = mark(3)) != cudaSuccess) return e;
         if (a.n > 0) {
-            const size_t smem = eval_smem_bytes(a.max_slots);
+            const size_t smem = eval_smem_bytes(a.max_rows);
             if (a.unsorted) {
                 if (smem > 48 * 1024 &&
                     (e = cudaFuncSetAttribute(k_eval_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -3029,7 +3014,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
         if ((e = mark(2)) != cudaSuccess) return e;
         if ((e = mark(3)) != cudaSuccess) return e;
         if (a.n > 0) {
-            const size_t smem = eval_smem_bytes(a.max_slots);
+            const size_t smem = eval_smem_bytes(a.max_rows);
             if (smem > 48 * 1024 &&
                 (e = cudaFuncSetAttribute(k_eval_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
                     cudaSuccess)
@@ -3068,7 +3053,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
     }
     if ((e = mark(2)) != cudaSuccess) return e;
     if (a.n > 0 && fused) {
-        const size_t smem = eval_smem_bytes(a.max_slots);
+        const size_t smem = eval_smem_bytes(a.max_rows);
         if (smem > 48 * 1024 &&
             (e = cudaFuncSetAttribute(k_eval_fused<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
                 cudaSuccess)
@@ -3079,11 +3064,11 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
     } else if (a.n > 0) {
         const bool outer = a.use_cache && a.split && !a.keys_inline;
         const bool plain = !a.use_cache && !a.surr_ord;
-        const size_t smem = eval_smem_bytes(outer ? a.max_slots_outer : a.max_slots),
-                     smem_roots = eval_smem_bytes(a.max_slots_roots);
+        const size_t smem = eval_smem_bytes(outer ? a.max_rows_outer : a.max_rows),
+                     smem_roots = eval_smem_bytes(a.max_rows_roots);
         // the first pass on an empty table without surrogates: every lane runs every node
         const bool fill = a.use_cache && a.keys_inline && !a.surr_ord;
-        auto keval = outer ? k_eval<EVAL_OUTER> : plain ? k_eval<EVAL_PLAIN> : k_eval<EVAL_GENERIC>;
+        auto keval = outer ? k_eval1<EVAL_OUTER> : plain ? k_eval1<EVAL_PLAIN> : fill ? k_eval1<EVAL_FILL> : k_eval;
         // two points per lane where every lane runs every instruction and the doubled slot
         // file leaves room for several blocks per SM; the item counter then counts pairs
         const bool two = (outer || plain || fill) && !a.one_point && 2 * smem <= EVAL2_MAX_SMEM;
@@ -3099,8 +3084,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
         // the batched misses: two misses per lane under the same conditions as the per-point
         // evaluator (the item counter then counts pairs)
         const bool two_roots = !a.one_point && 2 * smem_roots <= EVAL2_MAX_SMEM;
-        auto kroots = a.pos_level >= 0 ? (two_roots ? k_eval_roots2<true> : k_eval_roots<true>)
-                                       : (two_roots ? k_eval_roots2<false> : k_eval_roots<false>);
+        auto kroots = two_roots ? k_eval_roots2 : k_eval_roots;
         const size_t smem_kroots = two_roots ? 2 * smem_roots : smem_roots;
         if (smem_kroots > 48 * 1024 &&
             (e = cudaFuncSetAttribute(kroots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_kroots)) !=

@@ -15,13 +15,13 @@ namespace {
 __global__ void __launch_bounds__(128) k_root_samples(const uint4* __restrict__ prog, const float* __restrict__ params,
                                                       const RootInfo* __restrict__ rinfo, const uint32_t* __restrict__ groots,
                                                       uint32_t n_train_mats, uint32_t n_rows, uint64_t seed, float* data,
-                                                      uint32_t max_slots) {
+                                                      uint32_t max_rows) {
     extern __shared__ float s_val[];
     __shared__ float2 s_grad[8];
     init_gradients(s_grad);
     __syncthreads();
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * max_slots * 96u + lane);
+    char* Vb = reinterpret_cast<char*>(s_val + (size_t)warp * max_rows * 32u + lane);
     const uint32_t chunks = (n_rows + 31) / 32;
     for (uint32_t item = blockIdx.x * 4 + warp; item < n_train_mats * chunks; item += gridDim.x * 4) {
         const uint32_t mi = item / chunks, row = (item % chunks) * 32 + lane;
@@ -43,15 +43,15 @@ __global__ void __launch_bounds__(128) k_root_samples(const uint4* __restrict__ 
                 // such nodes are rejected when surrogates are chosen
                 continue;
             }
-            if (row < n_rows) exec_node(op, ins, Vb, pt, params, s_grad);
+            if (row < n_rows) exec_points<float>(ins, Vb, PointRegs{pt}, PointRegs{pt}, params, s_grad);
         }
         if (row < n_rows) {
             float* d = data + ((size_t)mi * n_rows + row) * 5;
             d[0] = pt.u;
             d[1] = pt.v;
-            d[2] = slot_ch(Vb, ri.out_slot * SLOT_BYTES, 0);
-            d[3] = slot_ch(Vb, ri.out_slot * SLOT_BYTES, 1);
-            d[4] = slot_ch(Vb, ri.out_slot * SLOT_BYTES, 2);
+            d[2] = slot_ch(Vb, ri.out_row * ROW_BYTES, 0);
+            d[3] = slot_ch(Vb, ri.out_row * ROW_BYTES, 1);
+            d[4] = slot_ch(Vb, ri.out_row * ROW_BYTES, 2);
         }
     }
 }
@@ -59,15 +59,15 @@ __global__ void __launch_bounds__(128) k_root_samples(const uint4* __restrict__ 
 }  // namespace
 
 cudaError_t launch_root_samples(const uint4* prog, const float* params, const RootInfo* rinfo, const uint32_t* groots,
-                                uint32_t n_train_mats, uint32_t n_rows, uint64_t seed, float* data, uint32_t max_slots,
+                                uint32_t n_train_mats, uint32_t n_rows, uint64_t seed, float* data, uint32_t max_rows,
                                 int num_sms, cudaStream_t s) {
-    const size_t smem = (size_t)4 * max_slots * 96u * sizeof(float);
+    const size_t smem = eval_smem_bytes(max_rows);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_root_samples, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     k_root_samples<<<num_sms * 16, 128, smem, s>>>(prog, params, rinfo, groots, n_train_mats, n_rows, seed, data,
-                                                   max_slots);
+                                                   max_rows);
     return cudaGetLastError();
 }
 

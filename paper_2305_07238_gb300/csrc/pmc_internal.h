@@ -25,16 +25,32 @@ namespace pmc {
 // A cacheable node r with the nodes only it needs (its exclusive sub-graph) forms a
 // contiguous block: ROOT_BEGIN(r), the exclusive nodes, then r flagged FLAG_ROOT.  A
 // lane whose lookup hit takes the cached value at ROOT_BEGIN and skips the block.
-constexpr uint32_t OP_ROOT_BEGIN = 32;
-constexpr uint32_t OP_LOAD_ROOT = 33;   // y: out slot | root ordinal; reads that node's probe record
+constexpr uint32_t OP_ROOT_BEGIN = 64;
+constexpr uint32_t OP_LOAD_ROOT = 65;   // y: out slot | root ordinal; reads that node's probe record
+constexpr uint32_t OP_END = 66;         // device programs only: the end of a program
+constexpr uint32_t OP_CONTROL = 64;     // operators from here on are no node's
 constexpr uint32_t FLAG_ROOT = 1;
 constexpr uint32_t FLAG_POSROOT = 2;    // ROOT_BEGIN of a node looked up under a position voxel
-constexpr uint32_t FLAG_IN2 = 4;        // MIX: the factor comes from in2 (else from fp0)
+constexpr uint32_t FLAG_ONE_ROW = 4;    // a node with equal channels: its value has one row, not three
+constexpr uint32_t FLAG_ONE_IN = 8;     // input 0 of an affine map, noise, Worley or facing node has one row
 
-// On the device, y and z of a node instruction hold byte offsets into the lane's slot
-// file (slot x SLOT_BYTES: the file is [slot][channel][lane] per warp), so an operand is one
-// add away from its address; 16-bit offsets allow MAX_DEVICE_SLOTS slots.
-constexpr uint32_t SLOT_BYTES = 3u * 32u * 4u;
+// Operators of device programs: the public ones, with the kinds of the operands' rows (three
+// or one; see compact_rows) spelled out where a node reads them by channel.  MIXN: the factor
+// comes from in2 (else it is a parameter).  ADD and MUL with one row of each kind have the
+// three-row input first.
+enum {
+    DOP_UV = 0, DOP_POSITION, DOP_NORMAL, DOP_CONST, DOP_CONST_1, DOP_AFFINE, DOP_FBM, DOP_VORONOI, DOP_CHECKER,
+    DOP_RAMP, DOP_MIX_33, DOP_MIX_31, DOP_MIX_13, DOP_MIX_11, DOP_MIXN_33, DOP_MIXN_31, DOP_MIXN_13, DOP_MIXN_11,
+    DOP_ADD_33, DOP_ADD_31, DOP_ADD_11, DOP_MUL_33, DOP_MUL_31, DOP_MUL_11, DOP_POW_3, DOP_POW_1, DOP_FACING
+};
+
+// The compiler allocates slots of three channels (networks needing more than MAX_DEVICE_SLOTS of
+// 3 x 32 floats per warp are refused) and then packs them into rows of one channel
+// (compact_rows): a value whose channels are all equal takes one row.  On the device, y and z of
+// a node instruction hold byte offsets into the lane's slot file (row x ROW_BYTES: the file is
+// [row][lane] per warp), so an operand is one add away from its address.
+constexpr uint32_t ROW_BYTES = 32u * 4u;
+constexpr uint32_t SLOT_BYTES = 3u * ROW_BYTES;
 constexpr uint32_t MAX_DEVICE_SLOTS = 0xFFFFu / SLOT_BYTES;
 constexpr uint32_t ROOT_POS_BIT = 1u << 31;   // device root table: node ID | this bit for such nodes
 
@@ -49,7 +65,7 @@ struct RootInfo {
     uint32_t level;
     uint32_t n_slots;
     uint32_t node;
-    uint32_t out_slot;
+    uint32_t out_row;
     uint32_t nodes;       // nodes and FP32 operations one run of the program evaluates
     uint32_t flops;
 };
@@ -59,12 +75,12 @@ struct MatInfo {
     uint32_t prog_len;
     uint32_t root_base;   // first entry in the root-node table
     uint32_t n_roots;
-    uint32_t out_slot;    // slot holding the material output after the program
+    uint32_t out_row;     // first of the three rows holding the material output after the program
     uint32_t n_slots;
     uint32_t n_nodes;
     uint32_t outer_start; // outer program: blocks replaced by loads of their node's record
     uint32_t outer_len;
-    uint32_t outer_out_slot;
+    uint32_t outer_out_row;
     uint32_t outer_slots;
     uint32_t pad;
     // nodes and FP32 operations one point evaluates with the whole program run (every
@@ -81,6 +97,9 @@ struct CompiledMaterial {
     std::vector<uint32_t> root_level;
     std::vector<uint32_t> root_slots;
     std::vector<uint32_t> root_out_slot;
+    // after compact_rows: the same programs' rows
+    uint32_t rows = 0, outer_rows = 0, out_row = 0, outer_out_row = 0;
+    std::vector<uint32_t> root_rows, root_out_row;
     std::vector<uint4> outer_prog;    // the program with each block replaced by OP_LOAD_ROOT
     uint32_t outer_slots = 0;
     uint32_t outer_out_slot = 0;
@@ -94,6 +113,13 @@ struct CompiledMaterial {
 // of the node cost model (node_cost), summed over the network as given; 0 = no threshold.
 bool compile_material(const pmc_node* nodes, uint32_t n, uint32_t min_root_nodes, uint32_t min_root_cost,
                       bool pos_desc, CompiledMaterial* out, const char** why);
+
+// Rewrites a program for the device: slots become rows, one per channel, or a single row for a
+// value whose channels are equal (params: the material's pool), and operators become DOP_*.
+// Returns the number of rows, at most 3 x n_slots; *out_row receives the first row of
+// out_slot's value (always three rows, like every cacheable node's).
+uint32_t compact_rows(std::vector<uint4>* prog, const std::vector<float>& params, uint32_t n_slots, uint32_t out_slot,
+                      uint32_t* out_row);
 
 // FP32 flops of one executed node (FMA counted as 2), from the device formulas: the node
 // cost model of include/pmc.h (pmc_node_cost).
@@ -178,9 +204,9 @@ struct BatchArgs {
     // materials
     const MatInfo* mats; uint32_t n_mats;
     const uint4* prog; const float* params; const uint32_t* roots;
-    uint32_t max_slots;        // value slots of the largest per-point program
-    uint32_t max_slots_roots;  // value slots of the largest standalone cacheable-node program
-    uint32_t max_slots_outer;  // value slots of the largest outer program
+    uint32_t max_rows;         // slot-file rows of the largest per-point program
+    uint32_t max_rows_roots;   // ... standalone cacheable-node program
+    uint32_t max_rows_outer;   // ... outer program
     // sort / segments
     uint32_t* counts; uint32_t* seg_start; uint32_t* probe_base; uint32_t* item_base;
     uint32_t* cursor;
@@ -287,7 +313,8 @@ cudaError_t launch_levels(const float* g1u, const float* g1v, const float* g2u, 
 cudaError_t launch_keys(const uint32_t* mat, const uint32_t* node, const float* u,
                         const float* v, uint64_t n, uint32_t level, uint64_t n_cells,
                         uint64_t* key, uint64_t* cell, uint32_t* h2, cudaStream_t s);
-size_t eval_smem_bytes(uint32_t max_slots);
+// Shared memory of an evaluator block with one point per lane; with two it is twice that.
+size_t eval_smem_bytes(uint32_t rows);
 
 // Training of the learned surrogates on the tcgen05 tensor cores (mlp_tc.cu): `steps`
 // minibatches of 128 rows per (split, material); mode 0 takes Adam steps, mode 1 adds the
@@ -305,7 +332,7 @@ uint32_t mlp_validate_parts(uint32_t n_nets, uint32_t n, int num_sms);
 cudaError_t launch_mlp_validate(const float* theta, const float* data, uint32_t n_nets, uint32_t n, double* sum,
                                 uint32_t* err, int num_sms, cudaStream_t s);
 cudaError_t launch_root_samples(const uint4* prog, const float* params, const RootInfo* rinfo, const uint32_t* groots,
-                                uint32_t n_train_mats, uint32_t n_rows, uint64_t seed, float* data, uint32_t max_slots,
+                                uint32_t n_train_mats, uint32_t n_rows, uint64_t seed, float* data, uint32_t max_rows,
                                 int num_sms, cudaStream_t s);
 cudaError_t launch_surrogate(const BatchArgs& a, int num_sms, cudaStream_t s);
 // Writes the operand images of slots 0 .. n_slots - 1 from their FP32 parameters.
