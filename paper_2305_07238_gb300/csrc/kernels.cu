@@ -2611,53 +2611,197 @@ __global__ void __launch_bounds__(256, 6) k_bin_insert(BatchArgs a) {
 //     priority is smallest, in that order, each with the value of that candidate;
 //   * a candidate with an inserted hash2 that is not its smallest is a duplicate; the
 //     candidates of every other hash2 find the cell full.
-// A first walk keeps the best F distinct keys seen so far in a buffer, each with the smallest
+// A walk keeps the best F distinct keys seen so far in a buffer, each with the smallest
 // priority seen for it; a new key pushes out the entry of largest priority when the buffer
 // is full and its own priority is smaller.  A key that belongs to the final F is never pushed
 // out (F better keys would have to exist) and enters at its smallest priority at the latest,
-// so the buffer ends as the inserted keys.  A second walk (lists of two or more) writes each
-// inserted key's candidate of smallest priority into the slot of its rank and sums the
-// weights (1 + shadows) of the inserted keys' candidates.  The rest are dropped full: the
-// evaluation counted the batch's emitted weight, which the resolution starts from, so a
-// cell without an empty slot is not walked at all.
+// so the buffer ends as the inserted keys, in the slots of their ranks.  If no key ever met a full
+// buffer, every candidate of the list has an inserted key; else a second walk sums the weights
+// (1 + shadows) of those that have.  The rest are dropped full: the evaluation counted the
+// batch's emitted weight, which the resolution starts from, so a cell without an empty slot is
+// not walked at all.
+//
+// Bound by memory: random 32-byte records and table sectors, and the latency between the steps of
+// a walk.  So a walk fetches the next record before it handles the current one, a list is walked
+// once unless it has more keys than the cell has room, a cell's words and an empty cell's
+// values are written as whole sectors (partial ones are fetched to be merged), and one atomic per
+// 256 candidates appends to the list of cells (one per 32, all on one address, took as long as the
+// rest of the linking).  Links in an array of their own, written in order, are slower: a second
+// random read per step (1,038 us).  Measured, the first pass of 2.07 M points with 6.7 cacheable nodes:
+// link 286 -> 157 us, resolve 798 -> 493 us (1.9 GB read: 3.8 TB/s); insert of four such passes 1,764 -> 1,282 us.
 constexpr uint32_t CHAIN_END = 0xFFFFFFFFu;
 
 __global__ void __launch_bounds__(256) k_chain_link(BatchArgs a) {
+    constexpr uint32_t PER = 8;   // candidates per lane and step: independent atomics in flight
     const uint32_t n_in = min(a.ctl->n_cand, a.probe_cap);
     const uint32_t* cc = a.lists[0];
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
-    // a warp takes 128 consecutive candidates per step: four independent atomics per lane
-    for (uint32_t b = warp * 128u; b < n_in; b += n_warps * 128u) {
-        uint32_t c[4];
-        bool first[4];
+    for (uint32_t b = warp * 32u * PER; b < n_in; b += n_warps * 32u * PER) {
+        uint32_t c[PER], prev[PER];
 #pragma unroll
-        for (uint32_t k = 0; k < 4; ++k) {
+        for (uint32_t k = 0; k < PER; ++k) {
             const uint32_t i = b + 32u * k + lane;
             c[k] = i < n_in ? __ldcg(&cc[i]) : 0u;
         }
 #pragma unroll
-        for (uint32_t k = 0; k < 4; ++k) {
+        for (uint32_t k = 0; k < PER; ++k) {
             const uint32_t i = b + 32u * k + lane;
-            first[k] = false;
-            if (i < n_in) {
-                const uint32_t prev = atomicExch(&a.chain_head[c[k]], i);
-                a.cands[i].cell = prev;   // the successor replaces the cell, known from the list
-                first[k] = prev == CHAIN_END;
+            prev[k] = i < n_in ? atomicExch(&a.chain_head[c[k]], i) : 0u;
+        }
+        uint32_t n_first = 0;   // cells first reached by this lane
+#pragma unroll
+        for (uint32_t k = 0; k < PER; ++k) {
+            const uint32_t i = b + 32u * k + lane;
+            if (i < n_in) a.cands[i].cell = prev[k];   // the successor replaces the cell, known from the list
+            n_first += prev[k] == CHAIN_END ? 1u : 0u;
+        }
+        uint32_t incl = n_first;
+#pragma unroll
+        for (uint32_t o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL_MASK, incl, o);
+            if (lane >= o) incl += y;
+        }
+        uint32_t x = 0;
+        if (lane == 31 && incl) x = atomicAdd(&a.ctl->n_lists, incl);
+        x = __shfl_sync(FULL_MASK, x, 31) + incl - n_first;
+#pragma unroll
+        for (uint32_t k = 0; k < PER; ++k)
+            if (prev[k] == CHAIN_END) a.lists[1][x++] = c[k];
+    }
+}
+
+// The best distinct keys of a cell seen so far: hash2, smallest priority and the candidate that
+// has it.  `lost`: a new key found the buffer full.
+struct CellBest {
+    uint32_t h[8], idx[8], nb;
+    unsigned long long p[8];
+    bool lost;
+    __device__ __forceinline__ void clear() {
+        nb = 0;
+        lost = false;
+#pragma unroll
+        for (uint32_t e = 0; e < 8; ++e) {
+            h[e] = idx[e] = 0u;
+            p[e] = 0ull;
+        }
+    }
+    // F: empty slots of the cell (1 .. 8)
+    __device__ __forceinline__ void offer(uint32_t F, unsigned long long pr, uint32_t hc, uint32_t i) {
+        bool found = false;
+#pragma unroll
+        for (uint32_t e = 0; e < 8; ++e)
+            if (e < nb && h[e] == hc) {
+                found = true;
+                if (pr < p[e]) {
+                    p[e] = pr;
+                    idx[e] = i;
+                }
             }
+        if (found) return;
+        uint32_t at = nb;   // the entry it takes (8: none)
+        if (nb < F) {
+            nb++;
+        } else {
+            lost = true;
+            unsigned long long mx = 0ull;
+#pragma unroll
+            for (uint32_t e = 0; e < 8; ++e)
+                if (e < nb && p[e] > mx) {
+                    mx = p[e];
+                    at = e;
+                }
+            if (pr >= mx) at = 8;
         }
 #pragma unroll
-        for (uint32_t k = 0; k < 4; ++k) {
-            const uint32_t x = warp_append(&a.ctl->n_lists, first[k]);
-            if (first[k]) a.lists[1][x] = c[k];
+        for (uint32_t e = 0; e < 8; ++e)
+            if (e == at) {
+                h[e] = hc;
+                p[e] = pr;
+                idx[e] = i;
+            }
+    }
+    __device__ __forceinline__ bool has(uint32_t hc) const {
+        bool in = false;
+#pragma unroll
+        for (uint32_t e = 0; e < 8; ++e) in |= e < nb && h[e] == hc;
+        return in;
+    }
+};
+
+// First empty slot of a cell (N_e if full) from its words.
+__device__ __forceinline__ uint32_t first_empty(const uint4& w0, const uint4& w1, uint32_t ne) {
+    const uint32_t h[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+    uint32_t used = ne;
+#pragma unroll
+    for (int e = 7; e >= 0; --e)
+        if ((uint32_t)e < ne && h[e] == 0u) used = (uint32_t)e;
+    return used;
+}
+
+// Writes a cell's new entries: the kept keys in ascending priority into the slots from the first
+// empty one (`used`) on; w0, w1: the cell's words as they were.  value(i): r, g, b of candidate i.
+template <class VAL>
+__device__ __forceinline__ void write_cell(const BatchArgs& a, uint32_t cell, uint4 w0, uint4 w1, uint32_t used,
+                                           const CellBest& k, VAL value) {
+    const uint32_t ne = a.n_entries;
+    uint32_t word[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+    uint32_t by_rank[8];
+#pragma unroll
+    for (uint32_t r = 0; r < 8; ++r) by_rank[r] = 0u;
+#pragma unroll
+    for (uint32_t e = 0; e < 8; ++e) {
+        if (e >= k.nb) continue;
+        uint32_t rank = 0;
+#pragma unroll
+        for (uint32_t f = 0; f < 8; ++f) rank += (f < k.nb && k.p[f] < k.p[e]) ? 1u : 0u;
+#pragma unroll
+        for (uint32_t r = 0; r < 8; ++r) {
+            if (r == rank) by_rank[r] = k.idx[e];
+            if (r == used + rank) word[r] = k.h[e];
+        }
+    }
+    // whole 16-byte words, so that no sector is fetched to be merged: what lies behind the hash2
+    // words in them (N_e not a multiple of 4) is this thread's cell too and goes back as it was,
+    // before the values are written
+    uint4* hw = reinterpret_cast<uint4*>(cell_h2(a, cell));
+    if (used < 4) hw[0] = make_uint4(word[0], word[1], word[2], word[3]);
+    if (ne > 4 && used + k.nb > 4) hw[1] = make_uint4(word[4], word[5], word[6], word[7]);
+    if (used == 0 && (ne & 3u) == 0) {
+        // an empty cell's values, four entries in three 16-byte stores, up to the end of the last
+        // 32-byte sector (an absent entry's zeros fall on an empty slot, whose value is zero)
+        float4* vp = reinterpret_cast<float4*>(cell_val(a, cell, 0));
+#pragma unroll
+        for (uint32_t g = 0; g < 2; ++g) {
+            if (4 * g >= k.nb) break;
+            float4 v[4];
+#pragma unroll
+            for (uint32_t r = 0; r < 4; ++r)
+                v[r] = 4 * g + r < k.nb ? value(by_rank[4 * g + r]) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const uint32_t left = k.nb - 4 * g;   // entries from here on
+            vp[3 * g] = make_float4(v[0].x, v[0].y, v[0].z, v[1].x);
+            // with N_e = 8 the sectors are words 0-1, 2-3 and 4-5 of the six
+            if (left > 1 || (ne == 8 && g == 0)) vp[3 * g + 1] = make_float4(v[1].y, v[1].z, v[2].x, v[2].y);
+            if (left > 2 || (ne == 8 && g == 1 && left > 1)) vp[3 * g + 2] = make_float4(v[2].z, v[3].x, v[3].y, v[3].z);
+            if (ne == 8 && g == 0 && (left == 3 || left == 4)) vp[3] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    } else {
+#pragma unroll
+        for (uint32_t r = 0; r < 8; ++r) {
+            if (r >= k.nb) break;
+            const float4 v = value(by_rank[r]);
+            float* val = cell_val(a, cell, used + r);
+            val[0] = v.x;
+            val[1] = v.y;
+            val[2] = v.z;
         }
     }
 }
 
-__global__ void __launch_bounds__(256, 4) k_chain_resolve(BatchArgs a) {
+
+__global__ void __launch_bounds__(256, 3) k_chain_resolve(BatchArgs a) {
     const uint32_t n_in = min(a.ctl->n_cand, a.probe_cap);
     const uint32_t n_cells = min(a.ctl->n_lists, n_in);
-    const uint32_t ne = a.n_entries;
     const uint4* cb = reinterpret_cast<const uint4*>(a.cands);   // two 16-byte halves per candidate
     // every candidate counts as dropped full until its cell's resolution says otherwise
     // (modular arithmetic: the sum of the counter's updates is the non-negative count)
@@ -2670,118 +2814,56 @@ __global__ void __launch_bounds__(256, 4) k_chain_resolve(BatchArgs a) {
         const uint32_t head = atomicExch(&a.chain_head[cell], CHAIN_END);   // takes the list, leaves it empty
         uint4 w0, w1;
         load_cell_words(a, cell, &w0, &w1);
-        uint32_t used = ne;
-        {
-            const uint32_t h[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-            for (int e = 7; e >= 0; --e)
-                if ((uint32_t)e < ne && h[e] == 0u) used = (uint32_t)e;   // the first empty slot
-        }
-        const uint32_t F = ne - used;
+        const uint32_t used = first_empty(w0, w1, a.n_entries), F = a.n_entries - used;
         if (F == 0) continue;   // a full cell: every candidate is dropped, as counted
-        // walk 1: the buffer (hash2 and the smallest priority seen for it, unordered)
-        uint32_t hb[8];
-        unsigned long long pb[8];
-#pragma unroll
-        for (uint32_t e = 0; e < 8; ++e) {
-            hb[e] = 0u;
-            pb[e] = 0ull;
+        if (head >= n_in) {     // not a list of this batch's candidates
+            bad = true;
+            break;
         }
-        uint32_t nb = 0, steps = 0;
-        uint4 v = make_uint4(0, 0, 0, 0);   // r, g, b, target of the last candidate walked
-        for (uint32_t j = head; j != CHAIN_END;) {
-            if (j >= n_in || ++steps > n_in) {   // not a list of this batch's candidates
-                bad = true;
-                break;
-            }
-            // prio, successor (in place of the cell), hash2; the candidates are read-only here,
-            // so the loads go through L1, where the second walk finds them
-            const uint4 q = __ldg(cb + 2 * (size_t)j);
-            v = __ldg(cb + 2 * (size_t)j + 1);
+        CellBest k;
+        k.clear();
+        unsigned long long WI = 0;   // weight of the inserted keys' candidates
+        uint32_t steps = 0, j = head;
+        // prio, successor (in place of the cell), hash2; the candidates are read-only here, so the
+        // loads go through L1, where the values are found again
+        uint4 q = __ldg(cb + 2 * (size_t)j);
+        uint32_t tg = __ldg(&cb[2 * (size_t)j + 1].w);
+        for (;;) {
+            // the next record is on its way while this one is handled
+            uint4 qn = make_uint4(0, 0, 0, 0);
+            uint32_t tn = 0;
             const uint32_t nj = q.z;
-            const unsigned long long pr = ((unsigned long long)q.y << 32) | q.x;
-            const uint32_t hc = q.w;
-            bool found = false;
-#pragma unroll
-            for (uint32_t e = 0; e < 8; ++e)
-                if (e < nb && hb[e] == hc) {
-                    found = true;
-                    if (pr < pb[e]) pb[e] = pr;
+            const bool more = nj != CHAIN_END;
+            if (more) {
+                if (nj >= n_in || ++steps > n_in) {
+                    bad = true;
+                    break;
                 }
-            if (!found) {
-                uint32_t at = nb;   // the buffer entry it takes (8: none)
-                if (nb < F) {
-                    nb++;
-                } else {
-                    // a new key with the buffer full: it pushes out the entry of largest
-                    // priority if its own is smaller
-                    unsigned long long mx = 0ull;
-#pragma unroll
-                    for (uint32_t e = 0; e < 8; ++e)
-                        if (e < nb && pb[e] > mx) {
-                            mx = pb[e];
-                            at = e;
-                        }
-                    if (pr >= mx) at = 8;
-                }
-#pragma unroll
-                for (uint32_t e = 0; e < 8; ++e)
-                    if (e == at) {
-                        hb[e] = hc;
-                        pb[e] = pr;
-                    }
+                qn = __ldg(cb + 2 * (size_t)nj);
+                tn = __ldg(&cb[2 * (size_t)nj + 1].w);
             }
+            k.offer(F, ((unsigned long long)q.y << 32) | q.x, q.w, j);
+            WI += 1u + (tg >> 16);
+            if (!more) break;
             j = nj;
+            q = qn;
+            tg = tn;
         }
         if (bad) break;
-        uint32_t* cw = cell_h2(a, cell);
-        if (steps == 1) {
-            // one candidate: it takes the first empty slot; its shadows find it
-            const uint32_t w = 1u + (v.w >> 16);
-            cw[used] = hb[0];
-            float* val = cell_val(a, cell, used);
-            val[0] = __uint_as_float(v.x);
-            val[1] = __uint_as_float(v.y);
-            val[2] = __uint_as_float(v.z);
-            n_ins += 1;
-            n_dup += w - 1u;
-            n_full -= w;
-            continue;
-        }
-        // walk 2: the weight of the inserted keys' candidates; each key's candidate of
-        // smallest priority writes the key and its value into the slot of its rank
-        unsigned long long WI = 0;
-        for (uint32_t j = head, k = 0; j != CHAIN_END && k < steps; ++k) {   // the list checked above
-            const uint4 q = __ldg(cb + 2 * (size_t)j);
-            const uint4 x = __ldg(cb + 2 * (size_t)j + 1);
-            const uint32_t nj = q.z;
-            const unsigned long long pr = ((unsigned long long)q.y << 32) | q.x;
-            const uint32_t hc = q.w;
-            bool in = false;
-            unsigned long long best = 0ull;
-#pragma unroll
-            for (uint32_t e = 0; e < 8; ++e)
-                if (e < nb && hb[e] == hc) {
-                    in = true;
-                    best = pb[e];
-                }
-            if (in) {
-                WI += 1u + (x.w >> 16);
-                if (pr == best) {
-                    uint32_t slot = used;
-#pragma unroll
-                    for (uint32_t f = 0; f < 8; ++f) slot += (f < nb && pb[f] < best) ? 1u : 0u;
-                    cw[slot] = hc;
-                    float* val = cell_val(a, cell, slot);
-                    val[0] = __uint_as_float(x.x);
-                    val[1] = __uint_as_float(x.y);
-                    val[2] = __uint_as_float(x.z);
-                }
+        if (k.lost) {   // the list checked above once more
+            WI = 0;
+            for (uint32_t i = head; i != CHAIN_END;) {
+                const uint4 x = __ldg(cb + 2 * (size_t)i);
+                if (k.has(x.w)) WI += 1u + (__ldg(&cb[2 * (size_t)i + 1].w) >> 16);
+                i = x.z;
             }
-            j = nj;
         }
-        n_ins += nb;
-        n_dup += WI - nb;
+        write_cell(a, cell, w0, w1, used, k, [&](uint32_t i) {
+            const uint4 v = __ldg(cb + 2 * (size_t)i + 1);
+            return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), 0.f);
+        });
+        n_ins += k.nb;
+        n_dup += WI - k.nb;
         n_full -= WI;
     }
     if (bad) atomicOr(&a.ctl->err, ERR_INSERT);
