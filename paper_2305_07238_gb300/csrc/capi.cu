@@ -1444,13 +1444,17 @@ pmc_status pmc_autotune(pmc_cache* c, const pmc_points* sample, uint32_t reps, p
         return b;
     };
     for (size_t k = 0; k < cand.size() && e == cudaSuccess && st == PMC_OK; ++k) time_cand(k);
-    // the insert is independent of the evaluator's schedule: the fastest schedule again
-    // with the binned insert, where the per-cell lists would apply
+    // the insert is independent of the evaluator's schedule: of the schedules under which the
+    // per-cell lists apply, the fastest again with the binned insert.  (Of all schedules would
+    // leave it untried where the claim rounds happen to be ahead by a microsecond.)
     if (e == cudaSuccess && st == PMC_OK && cand.size() < PMC_TUNE_MAX) {
-        const pmc_schedule b = cand[fastest()];
-        pmc_schedule x = b;
-        x.flags |= PMC_INSERT_BINNED;
-        if ((st = pmc_set_schedule(c, &b)) == PMC_OK && insert_lists(c)) {
+        size_t b = cand.size();
+        for (size_t k = 0; k < cand.size() && st == PMC_OK; ++k)
+            if ((st = pmc_set_schedule(c, &cand[k])) == PMC_OK && insert_lists(c) &&
+                (b == cand.size() || best_ms[k] < best_ms[b])) b = k;
+        if (st == PMC_OK && b < cand.size()) {
+            pmc_schedule x = cand[b];
+            x.flags |= PMC_INSERT_BINNED;
             cand.push_back(x);
             time_cand(cand.size() - 1);
         }
