@@ -48,6 +48,8 @@ struct pmc_cache {
     uint32_t* d_miss_cnt = nullptr;       // roots + MAX_LEVELS
     uint32_t* d_root_items = nullptr;     // roots + 1, then MAX_LEVELS + 1 level item starts
     uint32_t* d_root_order = nullptr;     // roots by ascending level, then MAX_LEVELS + 1 starts
+    uint32_t* d_mat_order = nullptr;      // materials by descending cost: whole programs, outer programs
+    double uneven[2] = {1.0, 1.0};        // cost of the longest program over the mean: whole, outer
     bool table_empty = true;              // nothing inserted since creation or reset
     bool last_all_miss = false;           // the last batch ran on an empty table
     bool last_unsorted = false;           // the last batch kept no probe records
@@ -120,4 +122,21 @@ inline void set_bins(const pmc_cache* c, pmc::BatchArgs* a) {
     a->bin_cnt = c->d_bins;
     a->bin_base = c->d_bins + a->n_bins;
     a->bin_list = c->d_bins + 2 * (size_t)a->n_bins + 1;
+}
+
+// The order of the materials' work items in the batch in *a, by the programs its points run, and
+// whether its evaluators take one point per lane.  Two points share an instruction's fetch and
+// decode, but an item takes twice as long, and a batch cannot end before its longest one: with few
+// items, or with programs of very uneven length, one point per lane spreads the work over
+// more warps.  The line: 60 items per SM x (longest / mean program - 1/2).  Evaluation of a first
+// pass, two points against one, us:
+//   64 networks of 20-200 nodes (longest / mean 2.3): 230 k points 170 / 160, 518 k 278 / 227, 1.04 M 384 / 421
+//   512 of 5-400 (4.4): 518 k 556 / 286, 1.04 M 561 / 391, 2.07 M 658 / 759
+//   1024 of 5-2000 (6): 518 k 2634 / 1626, 1.04 M 3182 / 2666, 2.07 M 4650 / 4976
+//   one network of 8 nodes: 115 k 25 / 29, 230 k 33 / 41
+inline void set_order(const pmc_cache* c, pmc::BatchArgs* a) {
+    const bool outer = a->use_cache && a->split && !a->keys_inline && !a->unsorted && !a->probe_inline && !a->alg1;
+    a->mat_order = c->d_mat_order + (outer ? c->n_mats : 0);
+    const double items = (double)a->n / 32.0 + c->n_mats;
+    if (!a->block_items && items < 60.0 * c->num_sms * (c->uneven[outer] - 0.5)) a->one_point = 1;
 }

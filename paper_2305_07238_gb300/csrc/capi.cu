@@ -203,6 +203,7 @@ void pmc_destroy_cache(pmc_cache* c) {
         dfree(&c->d_miss_cnt);
         dfree(&c->d_root_items);
         dfree(&c->d_root_order);
+        dfree(&c->d_mat_order);
         dfree(&c->d_bins);
         dfree(&c->d_surr_theta);
         dfree(&c->d_surr_img);
@@ -368,6 +369,7 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
         (s = dalloc(&c->d_miss_cnt, c->root_info.size() + MAX_LEVELS)) != PMC_OK ||
         (s = dalloc(&c->d_root_items, c->root_info.size() + 1 + MAX_LEVELS + 1)) != PMC_OK ||
         (s = dalloc(&c->d_root_order, c->root_info.size() + MAX_LEVELS + 1)) != PMC_OK ||
+        (s = dalloc(&c->d_mat_order, 2 * (size_t)n_mats)) != PMC_OK ||
         (s = dalloc(&c->d_bins, 3 * (size_t)(c->use_cache ? insert_bins_max(desc->n_cells) : 0) + 1)) != PMC_OK ||
         (s = dalloc(&c->d_surr_slot, n_mats)) != PMC_OK ||
         (s = dalloc(&c->d_surr_ord, n_mats)) != PMC_OK ||
@@ -383,12 +385,41 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
         e = cudaMemcpy(c->d_rinfo, c->root_info.data(), c->root_info.size() * sizeof(RootInfo), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !c->roots.empty())
         e = cudaMemcpy(c->d_roots, c->roots_dev.data(), c->roots_dev.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
+    // instructions a program takes, roughly: about 30 around each node, and 1.6 per FP32 operation
+    auto cost = [](uint64_t nodes, uint64_t flops) { return 30 * nodes + flops * 8 / 5; };
     {
-        // cacheable nodes by ascending nesting level (stable), then where each level starts
+        // materials by descending cost of the whole program, then of the outer program
+        std::vector<uint32_t> order(2 * (size_t)n_mats);
+        for (uint32_t m = 0; m < n_mats; ++m) order[m] = order[n_mats + m] = m;
+        const MatInfo* mi = c->mat_info.data();
+        std::stable_sort(order.begin(), order.begin() + n_mats, [&](uint32_t x, uint32_t y) {
+            return cost(mi[x].full_nodes, mi[x].full_flops) > cost(mi[y].full_nodes, mi[y].full_flops);
+        });
+        std::stable_sort(order.begin() + n_mats, order.end(), [&](uint32_t x, uint32_t y) {
+            return cost(mi[x].outer_nodes, mi[x].outer_flops) > cost(mi[y].outer_nodes, mi[y].outer_flops);
+        });
+        double sum[2] = {0.0, 0.0}, top[2] = {0.0, 0.0};
+        for (uint32_t m = 0; m < n_mats; ++m) {
+            const double k[2] = {(double)cost(mi[m].full_nodes, mi[m].full_flops),
+                                 (double)cost(mi[m].outer_nodes, mi[m].outer_flops)};
+            for (int o = 0; o < 2; ++o) {
+                sum[o] += k[o];
+                top[o] = std::max(top[o], k[o]);
+            }
+        }
+        for (int o = 0; o < 2; ++o) c->uneven[o] = sum[o] > 0.0 ? top[o] * n_mats / sum[o] : 1.0;
+        if (e == cudaSuccess)
+            e = cudaMemcpy(c->d_mat_order, order.data(), order.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
+    }
+    {
+        // cacheable nodes by ascending nesting level, each level by descending cost, then where
+        // each level starts
         std::vector<uint32_t> order(c->root_info.size());
         for (uint32_t g = 0; g < order.size(); ++g) order[g] = g;
+        const pmc::RootInfo* ri = c->root_info.data();
         std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
-            return c->root_info[x].level < c->root_info[y].level;
+            return ri[x].level != ri[y].level ? ri[x].level < ri[y].level
+                                              : cost(ri[x].nodes, ri[x].flops) > cost(ri[y].nodes, ri[y].flops);
         });
         const size_t n_roots = order.size();
         std::vector<uint32_t> starts(MAX_LEVELS + 1);
@@ -509,6 +540,7 @@ pmc_status enqueue_batch(pmc_cache* c, const pmc_points* pts, float* out_rgb, ui
     a.lookup_rb = c->lookup_rb;
     a.block_items = c->block_items;
     a.one_point = c->one_point;
+    set_order(c, &a);
     if (replacing(c)) {
         a.slot_cls = c->d_cls;
         a.vis = pts->vis;

@@ -56,9 +56,15 @@ __device__ __forceinline__ uint32_t warp_append(uint32_t* counter, bool pred) {
     return base + __popc(m & ((1u << lane_id()) - 1u));
 }
 
-__device__ __forceinline__ uint32_t find_material(const uint32_t* item_base, uint32_t n_mats,
+// The rank r with item_base[r] <= item < item_base[r + 1].  Work items of the materials' programs are
+// laid out in descending cost of the program (mat_order[r] is the material of rank r), so
+// that the longest are claimed first and the last ones to finish are short: an item is one warp
+// running one program from end to end, up to 1 ms for one of 2000 nodes.  (In material order, the
+// evaluation of a 16-pass frame of 64 networks took 6,251 instead of 5,617 us, of two passes of
+// 1024 networks of 5-2000 nodes 7,816 instead of 6,497 us, of two uncached passes 1,242 instead of 1,113 us.)
+__device__ __forceinline__ uint32_t find_rank(const uint32_t* item_base, uint32_t n_mats,
                                                   uint32_t item) {
-    // largest m with item_base[m] <= item (item_base is non-decreasing, item_base[0] = 0)
+    // largest r with item_base[r] <= item (item_base is non-decreasing, item_base[0] = 0)
     uint32_t lo = 0, hi = n_mats;  // invariant: item_base[lo] <= item < item_base[hi]
     while (hi - lo > 1) {
         uint32_t mid = (lo + hi) >> 1;
@@ -218,7 +224,7 @@ __device__ __forceinline__ void scan_materials(const BatchArgs& a) {
         uint32_t k = (a.use_cache || surr) ? a.mats[m].n_roots : 0u;
         c0 += c;
         c1 += c * k;
-        c2 += (c + 31u) >> 5;
+        c2 += (__ldcg(&a.counts[a.mat_order[m]]) + 31u) >> 5;   // items are laid out by rank
         c3 += (surr && a.surr_slot[m] >= 0) ? (c + 127u) >> 7 : 0u;
     }
     uint32_t tot0, tot1, tot2, tot3;
@@ -237,7 +243,7 @@ __device__ __forceinline__ void scan_materials(const BatchArgs& a) {
         if (surr) a.surr_item_base[m] = b3;
         b0 += c;
         b1 += c * k;
-        b2 += (c + 31u) >> 5;
+        b2 += (__ldcg(&a.counts[a.mat_order[m]]) + 31u) >> 5;
         b3 += (surr && a.surr_slot[m] >= 0) ? (c + 127u) >> 7 : 0u;
     }
     if (t == T - 1) {
@@ -431,9 +437,9 @@ __global__ void __launch_bounds__(256, 4) k_lookup(BatchArgs a) {
     const uint32_t ne = a.n_entries;
     unsigned long long n_look = 0, n_hit = 0, n_slots = 0;
     for (uint32_t item = blockIdx.x * (blockDim.x >> 5) + warp; item < n_items; item += warps_total) {
-        const uint32_t m = find_material(a.item_base, a.n_mats, item);
+        const uint32_t rank = find_rank(a.item_base, a.n_mats, item), m = __ldg(&a.mat_order[rank]);
         const uint32_t cnt = __ldg(&a.counts[m]);
-        const uint32_t j = (item - __ldg(&a.item_base[m])) * 32u + lane;
+        const uint32_t j = (item - __ldg(&a.item_base[rank])) * 32u + lane;
         const bool valid = j < cnt;
         const uint32_t s = __ldg(&a.seg_start[m]) + j;
         uint32_t iu = 0, iv = 0, lev = a.level;
@@ -649,9 +655,9 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval(BatchArgs a, uint32_t*
         if (lane == 0) item = atomicAdd(item_ctr, 1u);
         item = __shfl_sync(FULL_MASK, item, 0);
         if (item >= n_items) break;
-        const uint32_t m = find_material(a.item_base, a.n_mats, item);
+        const uint32_t rank = find_rank(a.item_base, a.n_mats, item), m = __ldg(&a.mat_order[rank]);
         const uint32_t cnt = __ldg(&a.counts[m]);
-        const uint32_t j = (item - __ldg(&a.item_base[m])) * 32u + lane;
+        const uint32_t j = (item - __ldg(&a.item_base[rank])) * 32u + lane;
         const bool valid = j < cnt;
         const uint32_t jj = valid ? j : cnt - 1u;   // an item holds at least one point
         const uint32_t s = __ldg(&a.seg_start[m]) + jj;
@@ -772,12 +778,13 @@ __device__ __forceinline__ void prefetch_point(const BatchArgs& a, uint32_t s) {
 // EVAL_PLAIN, EVAL_FILL), one point per lane (Vb: the lane's base in a [row][lane]
 // file).
 template <int MODE>
-__device__ __forceinline__ void eval_item1(const BatchArgs& a, uint32_t item, uint32_t m, char* Vb, const float2* grad,
+__device__ __forceinline__ void eval_item1(const BatchArgs& a, uint32_t item, uint32_t rank, char* Vb, const float2* grad,
                                            unsigned long long* n_nodes, unsigned long long* n_flops, FillStats* fs) {
     constexpr bool outer = MODE == EVAL_OUTER;
     const uint32_t lane = lane_id();
+    const uint32_t m = __ldg(&a.mat_order[rank]);
     const uint32_t cnt = __ldg(&a.counts[m]);
-    const uint32_t j = (item - __ldg(&a.item_base[m])) * 32u + lane;
+    const uint32_t j = (item - __ldg(&a.item_base[rank])) * 32u + lane;
     const bool valid = j < cnt;
     const uint32_t jj = valid ? j : cnt - 1u;   // an idle lane shadows the segment's last point
     const uint32_t s = __ldg(&a.seg_start[m]) + jj;
@@ -838,12 +845,13 @@ __device__ __forceinline__ void eval_item1(const BatchArgs& a, uint32_t item, ui
 // Two consecutive 32-point items of one material, two points per lane (A from the first
 // item, B from the second; Vb: the lane's base in a [row][lane][2] file).
 template <int MODE>
-__device__ __forceinline__ void eval_item2(const BatchArgs& a, uint32_t item, uint32_t m, char* Vb, const float2* grad,
+__device__ __forceinline__ void eval_item2(const BatchArgs& a, uint32_t item, uint32_t rank, char* Vb, const float2* grad,
                                            unsigned long long* n_nodes, unsigned long long* n_flops, FillStats* fs) {
     constexpr bool outer = MODE == EVAL_OUTER;
     const uint32_t lane = lane_id();
+    const uint32_t m = __ldg(&a.mat_order[rank]);
     const uint32_t cnt = __ldg(&a.counts[m]);
-    const uint32_t j = (item - __ldg(&a.item_base[m])) * 32u + lane;
+    const uint32_t j = (item - __ldg(&a.item_base[rank])) * 32u + lane;
     const bool vA = j < cnt, vB = j + 32u < cnt;
     const uint32_t jA = vA ? j : cnt - 1u, jB = vB ? j + 32u : cnt - 1u;
     const uint32_t s0 = __ldg(&a.seg_start[m]);
@@ -944,7 +952,7 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval1(BatchArgs a, uint32_t
         if (lane == 0) item = atomicAdd(item_ctr, 1u);
         item = __shfl_sync(FULL_MASK, item, 0);
         if (item >= n_items) break;
-        eval_item1<MODE>(a, item, find_material(a.item_base, a.n_mats, item), Vb, s_grad, &n_nodes, &n_flops, &fs);
+        eval_item1<MODE>(a, item, find_rank(a.item_base, a.n_mats, item), Vb, s_grad, &n_nodes, &n_flops, &fs);
     }
     warp_add_u64(&a.stats[ST_NODES], n_nodes);
     warp_add_u64(&a.stats[ST_FLOPS], n_flops);
@@ -997,13 +1005,13 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32, MODE == EVAL_FILL ? 6 : 7) k_
             if (BLOCK) continue;   // this warp's pair is past the end; the block's tile is not
             break;
         }
-        const uint32_t m = find_material(a.item_base, a.n_mats, it);
-        if (it + 1u < __ldg(&a.item_base[m + 1])) {
-            eval_item2<MODE>(a, it, m, Vb2, s_grad, &n_nodes, &n_flops, &fs);
+        const uint32_t rank = find_rank(a.item_base, a.n_mats, it);
+        if (it + 1u < __ldg(&a.item_base[rank + 1])) {
+            eval_item2<MODE>(a, it, rank, Vb2, s_grad, &n_nodes, &n_flops, &fs);
         } else {
-            eval_item1<MODE>(a, it, m, Vb1, s_grad, &n_nodes, &n_flops, &fs);
+            eval_item1<MODE>(a, it, rank, Vb1, s_grad, &n_nodes, &n_flops, &fs);
             if (it + 1u < n_items)
-                eval_item1<MODE>(a, it + 1u, find_material(a.item_base, a.n_mats, it + 1u), Vb1, s_grad, &n_nodes,
+                eval_item1<MODE>(a, it + 1u, find_rank(a.item_base, a.n_mats, it + 1u), Vb1, s_grad, &n_nodes,
                                  &n_flops, &fs);
         }
     }
@@ -1171,9 +1179,10 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_fused(BatchArgs a, uin
         bool ok = false;
         PointIn pt{0, 0, 0, 0, 0, 0, 0, 0};
         if (GROUPED) {
-            m = find_material(a.item_base, a.n_mats, chunk);
+            const uint32_t rank = find_rank(a.item_base, a.n_mats, chunk);
+            m = __ldg(&a.mat_order[rank]);
             cnt = __ldg(&a.counts[m]);
-            jj = (chunk - __ldg(&a.item_base[m])) * 32u + lane;
+            jj = (chunk - __ldg(&a.item_base[rank])) * 32u + lane;
             ok = jj < cnt;
             if (ok) {
                 const uint32_t s = __ldg(&a.seg_start[m]) + jj;
@@ -1460,7 +1469,7 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_roots(BatchArgs a, uin
         if (lane == 0) item = first + atomicAdd(item_ctr, 1u);
         item = __shfl_sync(FULL_MASK, item, 0);
         if (item >= end) break;
-        roots_item1(a, item, find_material(a.root_item_base, a.n_roots_total, item), Vb, s_grad, &st);
+        roots_item1(a, item, find_rank(a.root_item_base, a.n_roots_total, item), Vb, s_grad, &st);
     }
     roots_stats(a, st);
 }
@@ -1486,13 +1495,13 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32, 6) k_eval_roots2(BatchArgs a,
         pr = __shfl_sync(FULL_MASK, pr, 0);
         const uint32_t it = first + 2u * pr;
         if (it >= end) break;
-        const uint32_t q = find_material(a.root_item_base, a.n_roots_total, it);
+        const uint32_t q = find_rank(a.root_item_base, a.n_roots_total, it);
         if (it + 1u < end && it + 1u < a.root_item_base[q + 1]) {
             roots_item2(a, it, q, Vb2, s_grad, &st);
         } else {
             roots_item1(a, it, q, Vb1, s_grad, &st);
             if (it + 1u < end)
-                roots_item1(a, it + 1u, find_material(a.root_item_base, a.n_roots_total, it + 1u), Vb1, s_grad,
+                roots_item1(a, it + 1u, find_rank(a.root_item_base, a.n_roots_total, it + 1u), Vb1, s_grad,
                                  &st);
         }
     }

@@ -171,6 +171,7 @@ extern "C" pmc_status pmc_eval_batch_noalloc(pmc_cache* c, const pmc_points* pts
     a.lookup_rb = c->lookup_rb;
     a.block_items = c->block_items;
     a.one_point = c->one_point;
+    set_order(c, &a);
     if (c->use_cache && (c->desc.flags & PMC_REPLACE_VISIBILITY)) {
         a.slot_cls = c->d_cls;
         a.vis = pts->vis;

@@ -208,8 +208,10 @@ struct BatchArgs {
     uint32_t max_rows_roots;   // ... standalone cacheable-node program
     uint32_t max_rows_outer;   // ... outer program
     // sort / segments
-    uint32_t* counts; uint32_t* seg_start; uint32_t* probe_base; uint32_t* item_base;
+    uint32_t* counts; uint32_t* seg_start; uint32_t* probe_base;
+    uint32_t* item_base;       // first work item of each rank (n_mats + 1)
     uint32_t* cursor;
+    const uint32_t* mat_order; // materials by descending cost of the program this pass runs per point
     float* su; float* sv; float* spx; float* spy; float* spz;
     float* snx; float* sny; float* snz; uint32_t* sidx;
     uint32_t* slev;            // grouped per-point mip levels (with ray-cone gradients)
@@ -232,7 +234,8 @@ struct BatchArgs {
     int split;
     const RootInfo* rinfo; uint32_t n_roots_total; uint32_t max_level;
     uint32_t* miss_cnt;        // n_roots_total counters, then MAX_LEVELS item counters
-    // cacheable nodes in ascending nesting level (a permutation of the global root index),
+    // cacheable nodes in ascending nesting level, each level by descending cost (a permutation of
+    // the global root index),
     // and where each level starts in it (MAX_LEVELS + 1 entries): the batched evaluation of
     // one level visits only that level's work items
     const uint32_t* root_order; const uint32_t* level_start;
