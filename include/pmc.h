@@ -189,10 +189,10 @@ typedef struct {
                                      64 points, so the warps of a block share the material's
                                      instruction and parameter lines (same results)          */
 #define PMC_ONE_POINT 0x800u    /* schedule only: one point per lane in the per-point and
-                                     batched-miss evaluators throughout; without it two, and
-                                     one in the per-point evaluator of a batch too small to
-                                     spread pairs over the GPU (same results)                */
-#define PMC_INSERT_BINNED 0x1000u /* schedule only: group the candidates by bins of 256 cells
+                                     batched-miss evaluators of every batch; without it two,
+                                     and one in a batch too small, or with networks too
+                                     uneven, to spread pairs over the GPU (same results)     */
+#define PMC_INSERT_BINNED 0x1000u /* schedule only: group the candidates by bins of cells
                                      (count, scan, scatter, then a warp or a block per bin)
                                      where the default would chain each cell's candidates in
                                      a list resolved by its first arrival (keep-first tables

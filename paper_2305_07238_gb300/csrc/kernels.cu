@@ -2975,6 +2975,14 @@ int insert_grid(int num_sms) {
     return per_sm * num_sms;
 }
 
+// Blocks of a grid that takes `work` blocks' worth at most, up to `per_sm` per SM: a small batch
+// does not pay for launching blocks that find nothing to do.  (Full grids against these, us over four
+// passes: 4096 points, evaluation 58 / 39 and batched misses 52 / 40; 56,743 points,
+// evaluation 354 / 303.)
+static unsigned grid_for(uint64_t work, int num_sms, int per_sm) {
+    return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(work, (uint64_t)num_sms * per_sm));
+}
+
 // Insert phase: the candidates of the batch into the table (Alg. 1 semantics).
 static cudaError_t launch_insert(const BatchArgs& a, cudaStream_t s, int num_sms, uint64_t* nl) {
     cudaError_t e = cudaSuccess;
@@ -2994,8 +3002,8 @@ static cudaError_t launch_insert(const BatchArgs& a, cudaStream_t s, int num_sms
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_chain_resolve, 256, 0) != cudaSuccess || v <= 0) v = 1;
             per_sm = v;
         }
-        k_chain_link<<<num_sms * 8, 256, 0, s>>>(a);
-        k_chain_resolve<<<num_sms * per_sm, 256, 0, s>>>(a);
+        k_chain_link<<<grid_for(a.probe_cap / 2048u + 1u, num_sms, 8), 256, 0, s>>>(a);
+        k_chain_resolve<<<grid_for(a.probe_cap / 256u + 1u, num_sms, per_sm), 256, 0, s>>>(a);
         *nl += 2;
     } else if (a.n > 0 && a.use_cache) {
         if ((e = cudaMemsetAsync(a.bin_cnt, 0, (size_t)a.n_bins * sizeof(uint32_t), s)) != cudaSuccess) return e;
@@ -3058,6 +3066,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
         nl++;
     }
     uint32_t* item_ctr = a.counts + a.n_mats;
+    const uint64_t items = ((uint64_t)a.n + 31u) / 32u + a.n_mats;   // work items of 32 points, at most
     if (a.alg1 && a.use_cache) {
         // the paper's concurrent update: lookups and inserts inside the evaluator, no
         // lookup kernel, no insert phase; grouped by material unless unsorted
@@ -3083,13 +3092,13 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
                     (e = cudaFuncSetAttribute(k_eval_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem)) != cudaSuccess)
                     return e;
-                k_eval_fused<false><<<num_sms * 16, EVAL_WARPS * 32, smem, s>>>(a, nullptr);
+                k_eval_fused<false><<<grid_for(items / EVAL_WARPS + 1u, num_sms, 16), EVAL_WARPS * 32, smem, s>>>(a, nullptr);
             } else {
                 if (smem > 48 * 1024 &&
                     (e = cudaFuncSetAttribute(k_eval_fused<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem)) != cudaSuccess)
                     return e;
-                k_eval_fused<true><<<num_sms * 16, EVAL_WARPS * 32, smem, s>>>(a, item_ctr);
+                k_eval_fused<true><<<grid_for(items / EVAL_WARPS + 1u, num_sms, 16), EVAL_WARPS * 32, smem, s>>>(a, item_ctr);
             }
             nl++;
         }
@@ -3110,7 +3119,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
                 (e = cudaFuncSetAttribute(k_eval_fused<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
                     cudaSuccess)
                 return e;
-            k_eval_fused<false><<<num_sms * 16, EVAL_WARPS * 32, smem, s>>>(a, nullptr);
+            k_eval_fused<false><<<grid_for(items / EVAL_WARPS + 1u, num_sms, 16), EVAL_WARPS * 32, smem, s>>>(a, nullptr);
             nl++;
         }
         if ((e = mark(4)) != cudaSuccess) return e;
@@ -3131,7 +3140,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
     const bool fused = a.probe_inline && a.use_cache;
     if (a.n > 0 && a.use_cache && !a.keys_inline && !fused && !a.all_surr) {
         const uint32_t ne = a.n_entries, rb = a.lookup_rb;
-        const unsigned lb = (unsigned)num_sms * 8u;
+        const unsigned lb = grid_for(items / 8u + 1u, num_sms, 8);
         if (a.pos_level >= 0)
             launch_lookup<true>(a, ne, rb, lb, s);
         else
@@ -3150,7 +3159,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
                 cudaSuccess)
             return e;
         if ((e = mark(3)) != cudaSuccess) return e;
-        k_eval_fused<true><<<num_sms * 16, EVAL_WARPS * 32, smem, s>>>(a, item_ctr);
+        k_eval_fused<true><<<grid_for(items / EVAL_WARPS + 1u, num_sms, 16), EVAL_WARPS * 32, smem, s>>>(a, item_ctr);
         nl++;
     } else if (a.n > 0) {
         const bool outer = a.use_cache && a.split && !a.keys_inline;
@@ -3186,14 +3195,16 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
                 k_scan_roots<<<1, 1024, 0, s>>>(a);
                 nl++;
             }
+            const uint64_t root_items = (uint64_t)a.probe_cap / 32u + a.n_roots_total;
             // the level counters live after the per-root miss counters
             for (uint32_t lv = 0; lv <= a.max_level; ++lv) {
-                kroots<<<num_sms * 16, EVAL_WARPS * 32, smem_kroots, s>>>(a, lv, a.miss_cnt + a.n_roots_total + lv);
+                kroots<<<grid_for(root_items / EVAL_WARPS + 1u, num_sms, 16), EVAL_WARPS * 32, smem_kroots, s>>>(
+                    a, lv, a.miss_cnt + a.n_roots_total + lv);
                 nl++;
             }
         }
         if ((e = mark(3)) != cudaSuccess) return e;
-        keval<<<num_sms * 16, EVAL_WARPS * 32, smem_eval, s>>>(a, item_ctr);
+        keval<<<grid_for(items / EVAL_WARPS + 1u, num_sms, 16), EVAL_WARPS * 32, smem_eval, s>>>(a, item_ctr);
         nl++;
     } else if ((e = mark(3)) != cudaSuccess) {
         return e;
