@@ -124,6 +124,9 @@ inline void set_bins(const pmc_cache* c, pmc::BatchArgs* a) {
     a->bin_list = c->d_bins + 2 * (size_t)a->n_bins + 1;
 }
 
+// Instructions a program takes, roughly: about 30 around each node, and 1.6 per FP32 operation.
+inline uint64_t program_cost(uint64_t nodes, uint64_t flops) { return 30 * nodes + flops * 8 / 5; }
+
 // The order of the materials' work items in the batch in *a, by the programs its points run, and
 // whether its evaluators take one point per lane.  Two points share an instruction's fetch and
 // decode, but an item takes twice as long, and a batch cannot end before its longest one: with few

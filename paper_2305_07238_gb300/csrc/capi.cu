@@ -385,23 +385,21 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
         e = cudaMemcpy(c->d_rinfo, c->root_info.data(), c->root_info.size() * sizeof(RootInfo), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !c->roots.empty())
         e = cudaMemcpy(c->d_roots, c->roots_dev.data(), c->roots_dev.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
-    // instructions a program takes, roughly: about 30 around each node, and 1.6 per FP32 operation
-    auto cost = [](uint64_t nodes, uint64_t flops) { return 30 * nodes + flops * 8 / 5; };
     {
         // materials by descending cost of the whole program, then of the outer program
         std::vector<uint32_t> order(2 * (size_t)n_mats);
         for (uint32_t m = 0; m < n_mats; ++m) order[m] = order[n_mats + m] = m;
         const MatInfo* mi = c->mat_info.data();
         std::stable_sort(order.begin(), order.begin() + n_mats, [&](uint32_t x, uint32_t y) {
-            return cost(mi[x].full_nodes, mi[x].full_flops) > cost(mi[y].full_nodes, mi[y].full_flops);
+            return program_cost(mi[x].full_nodes, mi[x].full_flops) > program_cost(mi[y].full_nodes, mi[y].full_flops);
         });
         std::stable_sort(order.begin() + n_mats, order.end(), [&](uint32_t x, uint32_t y) {
-            return cost(mi[x].outer_nodes, mi[x].outer_flops) > cost(mi[y].outer_nodes, mi[y].outer_flops);
+            return program_cost(mi[x].outer_nodes, mi[x].outer_flops) > program_cost(mi[y].outer_nodes, mi[y].outer_flops);
         });
         double sum[2] = {0.0, 0.0}, top[2] = {0.0, 0.0};
         for (uint32_t m = 0; m < n_mats; ++m) {
-            const double k[2] = {(double)cost(mi[m].full_nodes, mi[m].full_flops),
-                                 (double)cost(mi[m].outer_nodes, mi[m].outer_flops)};
+            const double k[2] = {(double)program_cost(mi[m].full_nodes, mi[m].full_flops),
+                                 (double)program_cost(mi[m].outer_nodes, mi[m].outer_flops)};
             for (int o = 0; o < 2; ++o) {
                 sum[o] += k[o];
                 top[o] = std::max(top[o], k[o]);
@@ -419,7 +417,7 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
         const pmc::RootInfo* ri = c->root_info.data();
         std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) {
             return ri[x].level != ri[y].level ? ri[x].level < ri[y].level
-                                              : cost(ri[x].nodes, ri[x].flops) > cost(ri[y].nodes, ri[y].flops);
+                                              : program_cost(ri[x].nodes, ri[x].flops) > program_cost(ri[y].nodes, ri[y].flops);
         });
         const size_t n_roots = order.size();
         std::vector<uint32_t> starts(MAX_LEVELS + 1);
@@ -1045,50 +1043,100 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     const uint32_t s0 = c->n_surr_slots;
     pmc_status st = grow_surrogate_slots(c, s0 + L);
     if (st != PMC_OK) return st;
-    // initial parameters
-    std::vector<float> th((size_t)L * MLP_PARAMS);
-    for (uint32_t i = 0; i < L; ++i) init_theta(d->seed * 0x100000001B3ull + train[i] + 1, th.data() + (size_t)i * MLP_PARAMS);
-    float* theta = c->d_surr_theta + (size_t)s0 * MLP_PARAMS;
-    cudaError_t e = cudaMemcpyAsync(theta, th.data(), th.size() * sizeof(float), cudaMemcpyHostToDevice, s);
-    // temporaries: Adam moments, pairs, losses
-    float *m1 = nullptr, *m2 = nullptr, *data = nullptr, *loss = nullptr;
-    uint32_t* groots = nullptr;
-    const uint32_t nv = d->n_valid;
-    if ((st = dalloc(&m1, th.size())) != PMC_OK || (st = dalloc(&m2, th.size())) != PMC_OK ||
+    // The first epoch reads its pairs in a known order, so training starts when the first of up to
+    // PARTS parts of them (at least 32 steps each) is drawn and runs beside the drawing of the next, and of
+    // the validation pairs: a network trains on one SM, the evaluator needs them all.  The initial
+    // weights are drawn here meanwhile.  (64 networks of 500-2000 nodes, 65,536 pairs, one epoch: 22.6 ms
+    // per call one after the other, 18.3 ms so.)
+    constexpr uint32_t PARTS = 8;
+    const uint32_t steps_per_epoch = d->n_train / 128u, nv = d->n_valid;
+    uint32_t n_parts = 1;
+    while (n_parts < PARTS && steps_per_epoch / (2 * n_parts) >= 32u) n_parts *= 2;
+    // temporaries: initial weights, Adam moments, pairs, losses
+    const size_t n_theta = (size_t)L * MLP_PARAMS;
+    std::vector<float> th(n_theta);
+    float *m1 = nullptr, *m2 = nullptr, *data = nullptr, *vdata = nullptr, *loss = nullptr;
+    uint32_t* groots = nullptr;            // cacheable nodes, networks by cost, work counters
+    cudaStream_t ts = s;                   // training's stream
+    cudaEvent_t ev[PARTS + 1] = {};
+    auto release = [&]() {
+        if (ts != s) {
+            cudaStreamSynchronize(ts);
+            cudaStreamDestroy(ts);
+        }
+        for (cudaEvent_t x : ev)
+            if (x) cudaEventDestroy(x);
+        dfree(&m1); dfree(&m2); dfree(&data); dfree(&vdata); dfree(&loss); dfree(&groots);
+    };
+    if ((st = dalloc(&m1, n_theta)) != PMC_OK || (st = dalloc(&m2, n_theta)) != PMC_OK ||
         (st = dalloc(&data, (size_t)L * std::max(d->n_train, nv) * 5)) != PMC_OK || (st = dalloc(&loss, L)) != PMC_OK ||
-        (st = dalloc(&groots, L)) != PMC_OK) {
-        dfree(&m1); dfree(&m2); dfree(&data); dfree(&loss); dfree(&groots);
+        (st = dalloc(&groots, 2 * (size_t)L + PARTS + 1)) != PMC_OK) {
+        release();
         return st;
     }
-    std::vector<uint32_t> gr(L);
-    for (uint32_t i = 0; i < L; ++i) gr[i] = c->mat_info[train[i]].root_base + (uint32_t)c->surr_cand[train[i]];
-    if (e == cudaSuccess) e = cudaMemcpyAsync(groots, gr.data(), L * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m1, 0, th.size() * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m2, 0, th.size() * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, L * sizeof(float), s);
+    // the validation pairs get room of their own if there is some, or wait for the training
+    if (n_parts > 1 && dalloc(&vdata, (size_t)L * nv * 5) != PMC_OK) vdata = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (n_parts > 1) {
+        int lo = 0, hi = 0;
+        e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
+        if (e == cudaSuccess && (e = cudaStreamCreateWithPriority(&ts, cudaStreamNonBlocking, hi)) != cudaSuccess) ts = s;
+        for (uint32_t p = 0; e == cudaSuccess && p <= n_parts; ++p) e = cudaEventCreateWithFlags(&ev[p], cudaEventDisableTiming);
+    }
+    std::vector<uint32_t> gr(2 * (size_t)L + PARTS + 1, 0u);
+    for (uint32_t i = 0; i < L; ++i) {
+        gr[i] = c->mat_info[train[i]].root_base + (uint32_t)c->surr_cand[train[i]];
+        gr[L + i] = i;
+    }
+    std::stable_sort(gr.begin() + L, gr.begin() + 2 * L, [&](uint32_t x, uint32_t y) {
+        const RootInfo &rx = c->root_info[gr[x]], &ry = c->root_info[gr[y]];
+        return program_cost(rx.nodes, rx.flops) > program_cost(ry.nodes, ry.flops);
+    });
+    if (e == cudaSuccess) e = cudaMemcpyAsync(groots, gr.data(), gr.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
+    auto draw = [&](uint32_t part, uint32_t k0, uint32_t count, bool valid) {
+        RootSamples r{k0, count, valid ? 1u : TRAIN_SHUFFLE, valid ? ~0u : d->n_train - 1u, valid ? nv : d->n_train,
+                      valid ? d->seed ^ 0x5DEECE66Dull : d->seed, valid && vdata ? vdata : data, groots + 2 * (size_t)L + part};
+        return launch_root_samples(c->d_prog, c->d_params, c->d_rinfo, groots, L, r,
+                                   c->max_rows_roots ? c->max_rows_roots : 1, c->num_sms, s);
+    };
     // training pairs from the exact evaluator
-    if (e == cudaSuccess)
-        e = launch_root_samples(c->d_prog, c->d_params, c->d_rinfo, groots, L, d->n_train, d->seed, data,
-                                c->max_rows_roots ? c->max_rows_roots : 1, c->num_sms, s);
-    const uint32_t steps_per_epoch = d->n_train / 128u;
-    const uint32_t total = steps_per_epoch * d->epochs;
+    const uint32_t part_rows = d->n_train / n_parts;
+    for (uint32_t p = 0; e == cudaSuccess && p < n_parts; ++p) {
+        e = draw(p, p * part_rows, part_rows, false);
+        if (e == cudaSuccess && ts != s) e = cudaEventRecord(ev[p], s);
+    }
+    if (e == cudaSuccess && vdata) e = draw(PARTS, 0, nv, true);
+    for (uint32_t i = 0; i < L; ++i) init_theta(d->seed * 0x100000001B3ull + train[i] + 1, th.data() + (size_t)i * MLP_PARAMS);
+    float* theta = c->d_surr_theta + (size_t)s0 * MLP_PARAMS;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(theta, th.data(), n_theta * sizeof(float), cudaMemcpyHostToDevice, ts);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m1, 0, n_theta * sizeof(float), ts);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m2, 0, n_theta * sizeof(float), ts);
+    if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, L * sizeof(float), ts);
+    const uint32_t total = steps_per_epoch * d->epochs, part_steps = steps_per_epoch / n_parts;
     const float lr = d->lr > 0.0f ? d->lr : 1e-2f;
     for (uint32_t done = 0; e == cudaSuccess && done < total;) {
-        const uint32_t chunk = std::min<uint32_t>(total - done, 256u);
+        uint32_t chunk = std::min<uint32_t>(total - done, 256u);
+        if (ts != s && done < steps_per_epoch) {
+            const uint32_t in_part = done % part_steps;
+            if (in_part == 0 && (e = cudaStreamWaitEvent(ts, ev[done / part_steps], 0)) != cudaSuccess) break;
+            chunk = std::min(chunk, part_steps - in_part);
+        }
         e = launch_mlp_train(theta, m1, m2, nullptr, data, loss, &c->d_ctl->err, L, d->n_train, chunk,
                              (uint64_t)done * 128u, done,
-                             total, lr, 2.0f / (3.0f * 128.0f), 0, 1, s);
+                             total, lr, 2.0f / (3.0f * 128.0f), 0, 1, ts);
         done += chunk;
     }
+    if (e == cudaSuccess && ts != s) {
+        e = cudaEventRecord(ev[n_parts], ts);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev[n_parts], 0);
+    }
     // validation against held-out exact values, all networks in one launch
-    if (e == cudaSuccess)
-        e = launch_root_samples(c->d_prog, c->d_params, c->d_rinfo, groots, L, nv, d->seed ^ 0x5DEECE66Dull, data,
-                                c->max_rows_roots ? c->max_rows_roots : 1, c->num_sms, s);
+    if (e == cudaSuccess && !vdata) e = draw(PARTS, 0, nv, true);
     const uint32_t parts = mlp_validate_parts(L, nv, c->num_sms);
     double* d_sum = nullptr;
     std::vector<double> sums((size_t)L * parts);
     if (e == cudaSuccess && dalloc(&d_sum, sums.size()) != PMC_OK) e = cudaErrorMemoryAllocation;
-    if (e == cudaSuccess) e = launch_mlp_validate(theta, data, L, nv, d_sum, &c->d_ctl->err, c->num_sms, s);
+    if (e == cudaSuccess) e = launch_mlp_validate(theta, vdata ? vdata : data, L, nv, d_sum, &c->d_ctl->err, c->num_sms, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(sums.data(), d_sum, sums.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1106,7 +1154,7 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
                 if (list[k] == m) rmse[k] = err;
     }
     dfree(&d_sum);
-    dfree(&m1); dfree(&m2); dfree(&data); dfree(&loss); dfree(&groots);
+    release();
     if (e != cudaSuccess) return cuda_fail(c, e);
     c->n_surr_slots = s0 + L;
     e = upload_surrogate_maps(c);

@@ -834,7 +834,7 @@ __device__ __forceinline__ const float* tr_row(const TcTrainArgs& A, const float
         row = (uint32_t)k;
     } else {
         const uint32_t epoch = (uint32_t)(k >> (31 - __clz(A.n_data)));
-        row = (uint32_t)(k * 2654435761ull + (uint64_t)epoch * 0x9E3779B9ull) & (A.n_data - 1);
+        row = (uint32_t)(k * TRAIN_SHUFFLE + (uint64_t)epoch * 0x9E3779B9ull) & (A.n_data - 1);
     }
     return data + (size_t)row * 5;
 }

@@ -334,9 +334,19 @@ cudaError_t launch_mlp_forward_tc(const float* theta, const float* u, const floa
 uint32_t mlp_validate_parts(uint32_t n_nets, uint32_t n, int num_sms);
 cudaError_t launch_mlp_validate(const float* theta, const float* data, uint32_t n_nets, uint32_t n, double* sum,
                                 uint32_t* err, int num_sms, cudaStream_t s);
+// The rows of the training pairs to draw: (k * mult) & mask for k in [k0, k0 + count), of n_rows per network.
+struct RootSamples {
+    uint32_t k0, count, mult, mask, n_rows;
+    uint64_t seed;
+    float* data;               // per network: n_rows rows of (u, v, r, g, b)
+    uint32_t* ctr;             // a zeroed work counter of this launch's own
+};
+// groots: per network its cacheable node, then the networks in descending cost of its program.
 cudaError_t launch_root_samples(const uint4* prog, const float* params, const RootInfo* rinfo, const uint32_t* groots,
-                                uint32_t n_train_mats, uint32_t n_rows, uint64_t seed, float* data, uint32_t max_rows,
-                                int num_sms, cudaStream_t s);
+                                uint32_t n_train_mats, const RootSamples& r, uint32_t max_rows, int num_sms,
+                                cudaStream_t s);
+// Odd multiplier of the order in which training reads its pairs.
+constexpr uint32_t TRAIN_SHUFFLE = 2654435761u;
 cudaError_t launch_surrogate(const BatchArgs& a, int num_sms, cudaStream_t s);
 // Writes the operand images of slots 0 .. n_slots - 1 from their FP32 parameters.
 cudaError_t launch_surrogate_images(const float* theta, uint32_t n_slots, unsigned char* img, cudaStream_t s);
