@@ -544,12 +544,6 @@ constexpr uint32_t EVAL_WARPS = 4;
 
 size_t eval_smem_bytes(uint32_t rows) { return (size_t)EVAL_WARPS * rows * ROW_BYTES; }
 
-// Largest slot file (bytes per block) with which two points per lane run: four blocks of that size
-// fit an SM's shared memory.  Plain evaluation of 2 M points, two points against one per lane:
-// 42 KB 336 vs 388 us, 54 KB 458 vs 502, 66 KB 651 vs 654, 90 KB 998 vs 992: from there on the
-// warps that no longer fit cost what the shared decode saves.
-constexpr size_t EVAL2_MAX_SMEM = 56 * 1024;
-
 // Offers the lanes' freshly evaluated cacheable-node values to the table (Sec. 3).
 // `full`: the cell cannot take the value in this batch, so it is counted as dropped
 // without becoming a candidate.  Keep-first: the cell was full at lookup (nothing is

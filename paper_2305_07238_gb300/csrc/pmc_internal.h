@@ -318,6 +318,11 @@ cudaError_t launch_keys(const uint32_t* mat, const uint32_t* node, const float* 
                         uint64_t* key, uint64_t* cell, uint32_t* h2, cudaStream_t s);
 // Shared memory of an evaluator block with one point per lane; with two it is twice that.
 size_t eval_smem_bytes(uint32_t rows);
+// Largest slot file (bytes per block) with which two points per lane run: four blocks of that size
+// fit an SM's shared memory.  Plain evaluation of 2 M points, two points against one per lane:
+// 42 KB 336 vs 388 us, 54 KB 458 vs 502, 66 KB 651 vs 654, 90 KB 998 vs 992: from there on the
+// warps that no longer fit cost what the shared decode saves.
+constexpr size_t EVAL2_MAX_SMEM = 56 * 1024;
 
 // Training of the learned surrogates on the tcgen05 tensor cores (mlp_tc.cu): `steps`
 // minibatches of 128 rows per (split, material); mode 0 takes Adam steps, mode 1 adds the

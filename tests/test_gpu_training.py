@@ -84,12 +84,24 @@ def _net(layers, seed):
     return b.build()
 
 
+def _wide(n):
+    """A network that holds n values at a time."""
+    b = W.Builder()
+    uv = b.add(W.OP_UV)
+    v = [b.add(W.OP_FBM, [uv], ip=[1, k], fp=[1.0 + 0.05 * k, 2.0, 0.5]) for k in range(n)]
+    r = v[0]
+    for x in v[1:] + v[::-1]:
+        r = b.add(W.OP_MIX, [r, x], fp=[0.3])
+    return b.build()
+
+
+@pytest.mark.parametrize("wide", [2, 100])   # two points per lane, one
 @pytest.mark.parametrize("n_train,n_valid,epochs", [(128, 1, 1), (4096, 1000, 2), (8192, 1000, 2), (32768, 4099, 1)])
-def test_training_beside_the_drawing_of_its_pairs(n_train, n_valid, epochs):
+def test_training_beside_the_drawing_of_its_pairs(n_train, n_valid, epochs, wide):
     """The call draws its pairs in parts (none below 64 steps an epoch, two, eight) while it
     trains; the result has the bits of training on the whole set of pairs."""
     import torch
-    nets = [_net(2, 5), _net(9, 6), _net(4, 7)]
+    nets = [_net(2, 5), _net(9, 6), _wide(wide), _net(4, 7)]
     c = P.Cache(nets, 64, 8)
     seed = 21
     rmse = c.train_surrogates(n_train=n_train, n_valid=n_valid, epochs=epochs, lr=1e-2, seed=seed)
