@@ -339,7 +339,7 @@ def ours(args, rank, world, local_rank, dist):
     # the first pass of a frame runs on an empty table: no lookup launch
     per_launch_ms["lookup"] = ms["lookup"] / max(1, timing["batches"] - args.steps)
     fp32_peak = n_sms(torch, dev) * FP32_LANES_PER_SM * 2 * sm_mhz_max * 1e6 / 1e12   # TFLOP/s
-    # FP32 work of the per-point programs (k_eval) and of the batched misses (k_eval_roots)
+    # FP32 work of the per-point programs (k_eval2) and of the batched misses (k_eval_roots)
     flops_missed = frame_stats["flops_missed"]
     flops_eval = frame_stats["flops"] - flops_missed
     eval_tflops = flops_eval * args.steps / (ms["eval"] / 1e3) / 1e12 if ms["eval"] else 0.0
@@ -387,7 +387,7 @@ def ours(args, rank, world, local_rank, dist):
     # the evaluators of the tuned schedule: two points per lane unless it is PMC_ONE_POINT
     one_point = bool(tune["schedule"]["flags"] & P.PMC_ONE_POINT)
     binned = bool(tune["schedule"]["flags"] & P.PMC_INSERT_BINNED)
-    names = {"eval": "k_eval" if one_point else "k_eval2", "eval_roots": "k_eval_roots" if one_point else "k_eval_roots2",
+    names = {"eval": "k_eval1" if one_point else "k_eval2", "eval_roots": "k_eval_roots" if one_point else "k_eval_roots2",
              "lookup": "k_lookup",
              "insert": "k_bin_count .. k_bin_insert (binned)" if binned else "k_chain_link + k_chain_resolve"}
     for k in kernels:

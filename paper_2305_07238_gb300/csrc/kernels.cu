@@ -4,18 +4,26 @@
 //   k_hist     material histogram of the batch (+ range check of material indices); its last
 //              block lays out the per-material segments, probe offsets and warp work items
 //   k_scatter  groups the points by material into structure-of-arrays copies
+//   k_group    these three for a small batch, in one launch of one cluster
 //   k_lookup   probes of every (point, cacheable node) against the table as it was
-//              when the pass started (Sec. 3.2, Fig. 3); several probes in flight per lane
-//   k_eval_roots
-//              the missed cacheable nodes, listed per node by k_lookup, evaluated 32 at a
+//              when the pass started (Sec. 3.2, Fig. 3); several probes in flight per lane; its
+//              last block lays out the work items of the missed nodes
+//   k_eval_roots, k_eval_roots2
+//              the missed cacheable nodes, listed per node by k_lookup, evaluated 32 or 64 at a
 //              time with each node's standalone program; values go back into the probe
 //              records and become insert candidates (Sec. 3)
-//   k_eval     warp-uniform interpreter of the material programs (Sec. 2); every cached
-//              or computed block is skipped by the whole warp
+//   k_eval1, k_eval2, k_eval
+//              warp-uniform interpreter of the material programs (Sec. 2), one or two points
+//              per lane; k_eval also skips blocks that every lane has a value for
+//   k_chain_link, k_chain_resolve
+//              the insert through per-cell lists of candidates
+//   k_bin_*    the insert through candidates grouped by ranges of cells
 //   k_insert   rounds of the insert in one cooperative launch: every live candidate
 //              targets the first slot of its cell holding its hash2 (duplicate) or 0
 //              (free, Alg. 1); the smallest (point index, node ID) per cell wins by
 //              atomicMin and writes its slot
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstddef>
 #include <cstdio>
@@ -129,8 +137,7 @@ __device__ __forceinline__ U block_incl_scan(U v, U* tmp, U* total) {
 // block of k_hist and k_lookup): the
 // control block's per-batch part, the material and miss counts with the work-item counters
 // behind them, and the round counters of the claim-round insert.  Counts the batch.
-__global__ void __launch_bounds__(256) k_begin(BatchArgs a) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, T = gridDim.x * blockDim.x;
+__device__ __forceinline__ void clear_batch(const BatchArgs& a, uint32_t t, uint32_t T) {
     uint32_t* ctl = reinterpret_cast<uint32_t*>(a.ctl);
     for (uint32_t i = t; i < offsetof(Control, epoch) / 4; i += T) ctl[i] = 0u;
     if (a.insert_rounds)
@@ -139,6 +146,10 @@ __global__ void __launch_bounds__(256) k_begin(BatchArgs a) {
     if (a.split)
         for (uint32_t i = t; i < a.n_roots_total + MAX_LEVELS; i += T) a.miss_cnt[i] = 0u;
     if (t == 0) a.stats[ST_BATCHES] += 1ull;
+}
+
+__global__ void __launch_bounds__(256) k_begin(BatchArgs a) {
+    clear_batch(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // True in every thread of the block that arrives last of the grid's blocks (after its threads'
@@ -273,6 +284,40 @@ __device__ __forceinline__ void zero_output(const BatchArgs& a, uint32_t i) {
     if (a.out_hits) a.out_hits[i] = 0;
 }
 
+// Places point i (of a range that ends at hi) behind the points of its material placed so far
+// (pos_of: the next position per material, in shared or global memory).  Called by whole warps.
+__device__ __forceinline__ void scatter_point(const BatchArgs& a, uint32_t i, uint32_t hi, uint32_t* pos_of) {
+    const bool act = i < hi;
+    const uint32_t m = act ? a.mat[i] : 0u;
+    const bool ok = act && m < a.n_mats;
+    // the point's fields are loaded before its position is known, so that the loads
+    // overlap the match and the reservation
+    PointIn p{0, 0, 0, 0, 0, 0, 0, 0};
+    uint32_t lev = 0;
+    if (ok) {
+        p.u = a.u[i]; p.v = a.v[i];
+        p.px = a.px[i]; p.py = a.py[i]; p.pz = a.pz[i];
+        p.nx = a.nx[i]; p.ny = a.ny[i]; p.nz = a.nz[i];
+        if (a.g1u) lev = d_level(a.g1u[i], a.g1v[i], a.g2u[i], a.g2v[i], a.level_offset);
+    }
+    const unsigned vmask = __ballot_sync(FULL_MASK, ok);
+    if (ok) {
+        const unsigned peers = __match_any_sync(vmask, m);
+        const int leader = __ffs(peers) - 1;
+        uint32_t base = 0;
+        if ((int)lane_id() == leader) base = atomicAdd(&pos_of[m], (uint32_t)__popc(peers));
+        base = __shfl_sync(peers, base, leader);
+        const uint32_t pos = base + __popc(peers & ((1u << lane_id()) - 1u));
+        a.su[pos] = p.u; a.sv[pos] = p.v;
+        a.spx[pos] = p.px; a.spy[pos] = p.py; a.spz[pos] = p.pz;
+        a.snx[pos] = p.nx; a.sny[pos] = p.ny; a.snz[pos] = p.nz;
+        a.sidx[pos] = i;
+        if (a.g1u) a.slev[pos] = lev;
+    } else if (act) {
+        zero_output(a, i);
+    }
+}
+
 // Groups the block's contiguous range of points by material.  With few materials the
 // block counts its points per material in shared memory, reserves one range per
 // material with a single global atomic, then hands out positions from shared counters.
@@ -311,38 +356,76 @@ __global__ void __launch_bounds__(256) k_scatter(BatchArgs a) {
             if (s_cnt[m]) s_cnt[m] = atomicAdd(&a.cursor[m], s_cnt[m]);
         __syncthreads();
     }
-    for (uint32_t i = lo + threadIdx.x; i < hi32 && lo < hi; i += blockDim.x) {
+    for (uint32_t i = lo + threadIdx.x; i < hi32 && lo < hi; i += blockDim.x)
+        scatter_point(a, i, hi, local ? s_cnt : a.cursor);
+}
+
+// A small batch's grouping in one launch of one cluster: clear, count, lay out, place, with the
+// counts of the cluster's blocks exchanged through distributed shared memory.  Such a batch is
+// bound by launches and their chains of dependent reads, not by the bytes it moves.  The line: three
+// launches over the whole GPU against this one over eight SMs, us,
+//   64 materials: 1,024 points 18.1 / 12.3, 4,096 19.6 / 14.4, 16,384 19.2 / 24.6, 65,536 23.3 / 58.7
+//   1,024 materials: 22.7 / 14.5, 25.4 / 18.0, 26.7 / 29.6, 31.2 / 70.6
+constexpr uint32_t GROUP_CLUSTER = 8, GROUP_CLUSTER_T = 1024;
+constexpr uint32_t GROUP_CLUSTER_MATS = 2048;    // two per thread
+constexpr uint32_t GROUP_CLUSTER_MAX = 8192;     // points
+__global__ void __cluster_dims__(GROUP_CLUSTER, 1, 1) __launch_bounds__(GROUP_CLUSTER_T) k_group(BatchArgs a) {
+    __shared__ uint32_t s_cnt[GROUP_CLUSTER_MATS];   // this block's points per material
+    __shared__ uint32_t s_pos[GROUP_CLUSTER_MATS];   // its next position in each material's segment
+    __shared__ uint32_t s_tmp[33];
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const uint32_t t = threadIdx.x, rank = blockIdx.x;   // the grid is one cluster
+    for (uint32_t m = t; m < a.n_mats; m += GROUP_CLUSTER_T) s_cnt[m] = 0u;
+    if (rank == 0) clear_batch(a, t, GROUP_CLUSTER_T);
+    __syncthreads();
+    uint32_t lo, hi;
+    block_range(a.n, &lo, &hi);
+    const uint32_t hi32 = (hi + 31u) & ~31u;
+    uint32_t bad = 0;
+    for (uint32_t i = lo + t; i < hi32 && lo < hi; i += GROUP_CLUSTER_T) {
         const bool act = i < hi;
         const uint32_t m = act ? a.mat[i] : 0u;
         const bool ok = act && m < a.n_mats;
-        // the point's fields are loaded before its position is known, so that the loads
-        // overlap the match and the reservation
-        PointIn p{0, 0, 0, 0, 0, 0, 0, 0};
-        uint32_t lev = 0;
-        if (ok) {
-            p.u = a.u[i]; p.v = a.v[i];
-            p.px = a.px[i]; p.py = a.py[i]; p.pz = a.pz[i];
-            p.nx = a.nx[i]; p.ny = a.ny[i]; p.nz = a.nz[i];
-            if (a.g1u) lev = d_level(a.g1u[i], a.g1v[i], a.g2u[i], a.g2v[i], a.level_offset);
-        }
+        if (act && !ok) ++bad;
         const unsigned vmask = __ballot_sync(FULL_MASK, ok);
         if (ok) {
             const unsigned peers = __match_any_sync(vmask, m);
-            const int leader = __ffs(peers) - 1;
-            uint32_t base = 0;
-            if ((int)lane_id() == leader)
-                base = atomicAdd(local ? &s_cnt[m] : &a.cursor[m], (uint32_t)__popc(peers));
-            base = __shfl_sync(peers, base, leader);
-            const uint32_t pos = base + __popc(peers & ((1u << lane_id()) - 1u));
-            a.su[pos] = p.u; a.sv[pos] = p.v;
-            a.spx[pos] = p.px; a.spy[pos] = p.py; a.spz[pos] = p.pz;
-            a.snx[pos] = p.nx; a.sny[pos] = p.ny; a.snz[pos] = p.nz;
-            a.sidx[pos] = i;
-            if (a.g1u) a.slev[pos] = lev;
-        } else if (act) {
-            zero_output(a, i);
+            if ((int)lane_id() == __ffs(peers) - 1) atomicAdd(&s_cnt[m], (uint32_t)__popc(peers));
         }
     }
+    if (bad) {
+        atomicAdd(&a.stats[ST_BAD], (unsigned long long)bad);
+        atomicOr(&a.ctl->err, ERR_BAD_MAT);
+    }
+    cluster.sync();   // every block's counts
+    // each thread: two consecutive materials' totals, and what lower blocks hold of them
+    constexpr uint32_t PER = GROUP_CLUSTER_MATS / GROUP_CLUSTER_T;
+    uint32_t tot[PER] = {}, before[PER] = {}, sum = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < PER; ++k) {
+        const uint32_t m = t * PER + k;
+        if (m < a.n_mats) {
+#pragma unroll
+            for (uint32_t r = 0; r < GROUP_CLUSTER; ++r) {
+                const uint32_t c = cluster.map_shared_rank(s_cnt, r)[m];
+                tot[k] += c;
+                before[k] += r < rank ? c : 0u;
+            }
+            if (rank == 0) a.counts[m] = tot[k];
+        }
+        sum += tot[k];
+    }
+    uint32_t all;
+    uint32_t start = block_incl_scan(sum, s_tmp, &all) - sum;
+#pragma unroll
+    for (uint32_t k = 0; k < PER; ++k) {
+        if (t * PER + k < a.n_mats) s_pos[t * PER + k] = start + before[k];
+        start += tot[k];
+    }
+    __syncthreads();
+    if (rank == 0) scan_materials(a);   // reads the counts this block wrote
+    for (uint32_t i = lo + t; i < hi32 && lo < hi; i += GROUP_CLUSTER_T) scatter_point(a, i, hi, s_pos);
+    cluster.sync();   // no block leaves while another may read its counts
 }
 
 // =======================================================================================
@@ -3046,32 +3129,38 @@ static unsigned group_blocks(uint32_t n, int num_sms) {
     return std::max(1u, std::min((n + 255u) / 256u, (unsigned)num_sms * GROUP_BLOCKS_PER_SM));
 }
 
+// Clears the batch's counters and groups its points by material.
+static void launch_group(const BatchArgs& a, cudaStream_t s, int num_sms, uint64_t* nl) {
+    if (!a.unsorted && a.n > 0 && a.n <= GROUP_CLUSTER_MAX && a.n_mats <= GROUP_CLUSTER_MATS) {
+        k_group<<<GROUP_CLUSTER, GROUP_CLUSTER_T, 0, s>>>(a);
+        *nl += 1;
+        return;
+    }
+    // counts has n_mats + 1 entries, the last one the evaluation's work-item counter
+    const uint32_t words = a.n_mats + (a.split ? a.n_roots_total : 0u);
+    k_begin<<<std::min<uint32_t>(1u + words / 1024u, 64u), 256, 0, s>>>(a);
+    *nl += 1;
+    if (a.unsorted) return;
+    k_hist<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
+    *nl += 1;
+    if (a.n == 0) return;
+    k_scatter<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
+    *nl += 1;
+}
+
 cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEvent_t* ev,
                          uint64_t* launches) {
     cudaError_t e;
     uint64_t nl = 0;
     auto mark = [&](int k) { return ev ? cudaEventRecord(ev[k], s) : cudaSuccess; };
     if ((e = mark(0)) != cudaSuccess) return e;
-    // per-batch counters (epoch, errors and the barrier persist); counts has n_mats + 1 entries,
-    // the last one the evaluation's work-item counter
-    {
-        const uint32_t words = a.n_mats + (a.split ? a.n_roots_total : 0u);
-        k_begin<<<std::min<uint32_t>(1u + words / 1024u, 64u), 256, 0, s>>>(a);
-        nl++;
-    }
+    // per-batch counters (epoch, errors and the barrier persist)
+    launch_group(a, s, num_sms, &nl);
     uint32_t* item_ctr = a.counts + a.n_mats;
     const uint64_t items = ((uint64_t)a.n + 31u) / 32u + a.n_mats;   // work items of 32 points, at most
     if (a.alg1 && a.use_cache) {
         // the paper's concurrent update: lookups and inserts inside the evaluator, no
         // lookup kernel, no insert phase; grouped by material unless unsorted
-        if (!a.unsorted) {
-            k_hist<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
-            nl++;
-        }
-        if (!a.unsorted && a.n > 0) {
-            k_scatter<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
-            nl++;
-        }
         if ((e = mark(1)) != cudaSuccess) return e;
         if (!a.unsorted && a.n > 0 && a.surr_slot) {
             if ((e = launch_surrogate(a, num_sms, s)) != cudaSuccess) return e;
@@ -3122,12 +3211,6 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
         if ((e = mark(6)) != cudaSuccess) return e;
         if (launches) *launches += nl;
         return cudaGetLastError();
-    }
-    k_hist<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
-    nl++;
-    if (a.n > 0) {
-        k_scatter<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
-        nl++;
     }
     if ((e = mark(1)) != cudaSuccess) return e;
     // grouped schedule with the probes in the evaluator: no lookup kernel, no records
