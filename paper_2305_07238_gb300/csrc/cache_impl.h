@@ -49,7 +49,7 @@ struct pmc_cache {
     uint32_t* d_root_items = nullptr;     // roots + 1, then MAX_LEVELS + 1 level item starts
     uint32_t* d_root_order = nullptr;     // roots by ascending level, then MAX_LEVELS + 1 starts
     uint32_t* d_mat_order = nullptr;      // materials by descending cost: whole programs, outer programs
-    double uneven[2] = {1.0, 1.0};        // cost of the longest program over the mean: whole, outer
+    double uneven[3] = {1.0, 1.0, 1.0};   // cost of the longest program over the mean: whole, outer, cacheable nodes
     bool table_empty = true;              // nothing inserted since creation or reset
     bool last_all_miss = false;           // the last batch ran on an empty table
     bool last_unsorted = false;           // the last batch kept no probe records
@@ -142,4 +142,6 @@ inline void set_order(const pmc_cache* c, pmc::BatchArgs* a) {
     a->mat_order = c->d_mat_order + (outer ? c->n_mats : 0);
     const double items = (double)a->n / 32.0 + c->n_mats;
     if (!a->block_items && items < 60.0 * c->num_sms * (c->uneven[outer] - 0.5)) a->one_point = 1;
+    // the batched misses likewise, by the items of a level, which the device counts
+    a->root_pairs_min = (uint32_t)std::min(4e9, 60.0 * c->num_sms * (c->uneven[2] - 0.5));
 }

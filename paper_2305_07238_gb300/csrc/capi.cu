@@ -420,6 +420,13 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
                                               : program_cost(ri[x].nodes, ri[x].flops) > program_cost(ri[y].nodes, ri[y].flops);
         });
         const size_t n_roots = order.size();
+        double sum = 0.0, top = 0.0;
+        for (const RootInfo& r : c->root_info) {
+            const double k = (double)program_cost(r.nodes, r.flops);
+            sum += k;
+            top = std::max(top, k);
+        }
+        c->uneven[2] = sum > 0.0 ? top * (double)c->root_info.size() / sum : 1.0;
         std::vector<uint32_t> starts(MAX_LEVELS + 1);
         for (uint32_t l = 0; l <= MAX_LEVELS; ++l) {
             uint32_t start = 0;

@@ -1565,19 +1565,21 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32, 6) k_eval_roots2(BatchArgs a,
     char* Vb1 = Vw + lane * 4u;
     const uint32_t* level_items = a.root_item_base + a.n_roots_total + 1;
     const uint32_t first = level_items[level], end = level_items[level + 1];
+    // few items: one by one, or the launch lasts as long as its longest pair
+    const uint32_t step = end - first >= a.root_pairs_min ? 2u : 1u;
     RootStats st;
     for (;;) {
         uint32_t pr = 0;
         if (lane == 0) pr = atomicAdd(item_ctr, 1u);
         pr = __shfl_sync(FULL_MASK, pr, 0);
-        const uint32_t it = first + 2u * pr;
+        const uint32_t it = first + step * pr;
         if (it >= end) break;
         const uint32_t q = find_rank(a.root_item_base, a.n_roots_total, it);
-        if (it + 1u < end && it + 1u < a.root_item_base[q + 1]) {
+        if (step == 2u && it + 1u < end && it + 1u < a.root_item_base[q + 1]) {
             roots_item2(a, it, q, Vb2, s_grad, &st);
         } else {
             roots_item1(a, it, q, Vb1, s_grad, &st);
-            if (it + 1u < end)
+            if (step == 2u && it + 1u < end)
                 roots_item1(a, it + 1u, find_rank(a.root_item_base, a.n_roots_total, it + 1u), Vb1, s_grad,
                                  &st);
         }
@@ -3258,9 +3260,9 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
             (e = cudaFuncSetAttribute(keval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_eval)) !=
                 cudaSuccess)
             return e;
-        // the batched misses: two misses per lane under the same conditions as the per-point
-        // evaluator (the item counter then counts pairs)
-        const bool two_roots = !a.one_point && 2 * smem_roots <= EVAL2_MAX_SMEM;
+        // the batched misses: two misses per lane up to a smaller slot file, and in the kernel only
+        // where a level has enough items (the item counter then counts pairs)
+        const bool two_roots = !a.one_point && 2 * smem_roots <= ROOTS2_MAX_SMEM;
         auto kroots = two_roots ? k_eval_roots2 : k_eval_roots;
         const size_t smem_kroots = two_roots ? 2 * smem_roots : smem_roots;
         if (smem_kroots > 48 * 1024 &&

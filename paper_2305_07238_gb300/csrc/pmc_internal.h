@@ -268,6 +268,7 @@ struct BatchArgs {
     uint32_t lookup_rb;        // k_lookup: probes in flight per lane (1, 2 or 4)
     int block_items;           // 1: the per-point evaluator claims block-wide tiles of items
     int one_point;             // 1: one point per lane in the per-point evaluator (else two)
+    uint32_t root_pairs_min;   // batched misses: work items of a level from which two misses run per lane
     int alg1;                  // the paper's concurrent update: 8-byte slots {hash2, RGB9E5},
                                // looked up and inserted inside the evaluator (one 64-bit CAS)
     // replacement by visibility class (Sec. 5): per point its class (caller-owned, optional,
@@ -323,6 +324,11 @@ size_t eval_smem_bytes(uint32_t rows);
 // 42 KB 336 vs 388 us, 54 KB 458 vs 502, 66 KB 651 vs 654, 90 KB 998 vs 992: from there on the
 // warps that no longer fit cost what the shared decode saves.
 constexpr size_t EVAL2_MAX_SMEM = 56 * 1024;
+// The same for the batched misses, which are fewer: a warp's pair of misses of a long program takes
+// as long as the whole launch.  16 passes over 256 networks of 500-2000 nodes (44 KB), batched misses:
+// two per lane always 26.5 ms, two from 60 items per SM x (longest / mean program - 1/2) on 17.5 ms,
+// one 16.4 ms; 64 such networks (39 KB), 640 x 360, eight passes: 4.8 / 4.8 / 4.9 ms.
+constexpr size_t ROOTS2_MAX_SMEM = 40 * 1024;
 
 // Training of the learned surrogates on the tcgen05 tensor cores (mlp_tc.cu): `steps`
 // minibatches of 128 rows per (split, material); mode 0 takes Adam steps, mode 1 adds the

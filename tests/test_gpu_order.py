@@ -61,3 +61,37 @@ def test_large_batches_match_one_point(kind, n, cells):
     for (r0, h0), (r1, h1) in zip(a, b):
         assert np.array_equal(r0, r1) and np.array_equal(h0, h1)
     assert sa == sb
+
+
+@pytest.mark.parametrize("n", [60_000, 150_001, 400_003])
+@pytest.mark.parametrize("kind", ["equal", "wide"])
+def test_batched_misses_match_one_point(kind, n):
+    """Second and third passes whose misses fill fewer or more items than the line for two misses
+    per lane, and a program whose values fill more than its row file's limit."""
+    if kind == "wide":
+        b = W.Builder()
+        uv = b.add(W.OP_UV)
+        v = [b.add(W.OP_FBM, [uv], ip=[1, k], fp=[1.0 + 0.05 * k, 2.0, 0.5]) for k in range(60)]
+        r = v[0]
+        for x in v[1:] + v[::-1]:
+            r = b.add(W.OP_MIX, [r, x], fp=[0.3])
+        b.add(W.OP_MUL, [r, b.add(W.OP_FACING, [b.add(W.OP_NORMAL)], fp=[0.2, 0.5, 0.4])])
+        mats = [b.build()]
+    else:
+        mats = W.random_materials(2, 10, 10, 0.3, seed=5)
+    passes = [W.points_uniform(n, seed=s, n_mats=len(mats)) for s in (1, 2, 3)]
+    res = []
+    import torch
+    for flags in (0, P.PMC_ONE_POINT):
+        c = P.Cache(mats, 1 << 16, 8)
+        c.set_schedule(flags)
+        out = []
+        for p in passes:
+            rgb, hits = torch.empty((3, n), device="cuda"), torch.empty(n, dtype=torch.int16, device="cuda")
+            c.eval_batch(P.points_to_device(p), rgb, hits)
+            c.sync()
+            out += [rgb.cpu().numpy(), hits.cpu().numpy()]
+        assert out[3].any() and c.stats()["misses"] > n
+        res.append(out + [c.stats()["inserted"], c.stats()["nodes_evaluated"]] + list(c.table()))
+    for x, y in zip(*res):
+        assert np.array_equal(x, y)
