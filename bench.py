@@ -42,8 +42,9 @@ SAMPLE_ROWS = (0, 40)            # CPU-oracle sample: 40 full-width rows, all 16
 REF_ROWS = (0, 16)               # reference arm: 16 full-width rows per step, all 16 passes
 # The cost threshold of the headline frame (FP32 operations per cacheable sub-graph): the
 # break-even value the rule below gives on this frame with the per-cell-list insert
-# (about 490, rounded to a multiple of 50). It is fixed, so that the reference arm and
-# every leg run the same configuration; the line reports the live estimate beside it.
+# (about 490 when it was fixed, rounded to a multiple of 50). It stays fixed, so that the
+# reference arm and every leg run the same configuration; the line reports the live
+# estimate beside it.
 MIN_ROOT_COST = 500
 REF_MIN_ROOT_COST = MIN_ROOT_COST   # reference arm: the same threshold
 # DRAM bytes (read + written) per launch of each kernel, the mean of the two launches one
