@@ -138,10 +138,7 @@ __device__ __forceinline__ U block_incl_scan(U v, U* tmp, U* total) {
 // control block's per-batch part, the material and miss counts with the work-item counters
 // behind them, and the round counters of the claim-round insert.  Counts the batch.
 __device__ __forceinline__ void clear_batch(const BatchArgs& a, uint32_t t, uint32_t T) {
-    uint32_t* ctl = reinterpret_cast<uint32_t*>(a.ctl);
-    for (uint32_t i = t; i < offsetof(Control, epoch) / 4; i += T) ctl[i] = 0u;
-    if (a.insert_rounds)
-        for (uint32_t i = t; i < 2 * (MAX_ENTRIES + 2); i += T) a.ctl->mid_count[i] = 0u;   // and out_count behind it
+    clear_control(a.ctl, a.insert_rounds, t, T);
     for (uint32_t i = t; i <= a.n_mats; i += T) a.counts[i] = 0u;
     if (a.split)
         for (uint32_t i = t; i < a.n_roots_total + MAX_LEVELS; i += T) a.miss_cnt[i] = 0u;

@@ -2,6 +2,7 @@
 // C-ABI layer.  Not installed; the public interface is include/pmc.h.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 #include <vector>
@@ -174,6 +175,18 @@ struct Control {
     uint32_t mid_count[MAX_ENTRIES + 2];
     uint32_t out_count[MAX_ENTRIES + 2];
 };
+
+// Thread t of T's share of clearing the control block for a batch: everything before the epoch,
+// and the two arrays of round counters where the claim-round insert will count in them.
+__host__ __device__ inline void clear_control(Control* c, int insert_rounds, uint32_t t, uint32_t T) {
+    uint32_t* w = reinterpret_cast<uint32_t*>(c);
+    for (uint32_t i = t; i < offsetof(Control, epoch) / 4; i += T) w[i] = 0u;
+    if (!insert_rounds) return;
+    for (uint32_t i = t; i < MAX_ENTRIES + 2; i += T) {
+        c->mid_count[i] = 0u;
+        c->out_count[i] = 0u;
+    }
+}
 
 constexpr uint32_t ERR_BAD_MAT = 1;
 constexpr uint32_t ERR_INSERT = 2;
