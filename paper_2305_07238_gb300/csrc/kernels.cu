@@ -3,6 +3,8 @@
 //   k_begin    clears the batch's counters
 //   k_hist     material histogram of the batch (+ range check of material indices); its last
 //              block lays out the per-material segments, probe offsets and warp work items
+//   k_scan_materials
+//              this layout where there are many materials
 //   k_scatter  groups the points by material into structure-of-arrays copies
 //   k_group    these three for a small batch, in one launch of one cluster
 //   k_lookup   probes of every (point, cacheable node) against the table as it was
@@ -162,9 +164,16 @@ __device__ __forceinline__ bool last_block(uint32_t* ticket) {
     return true;
 }
 
+template <uint32_t U, bool SEGMENTS, bool ITEMS>
 __device__ __forceinline__ void scan_materials(const BatchArgs& a);
 
-__global__ void __launch_bounds__(256) k_hist(BatchArgs a) {
+// Up to this many materials the last block of k_hist lays them out (four per thread); above, a launch
+// of its own does, with four times the threads in each of two blocks, one for the segments and one for
+// the work items.  Clearing and grouping 65,536 points, us, last block / own launch: 1,024 materials
+// 30 / 34, 2,048 38 / 36, 4,096 54 / 44, 16,384 143 / 72, 60,000 365 / 228.
+constexpr uint32_t SCAN_IN_HIST = 1024;
+
+__global__ void __launch_bounds__(256, 6) k_hist(BatchArgs a) {
     __shared__ uint32_t s_cnt[GROUP_SMEM_MATS];
     const bool local = a.n_mats <= GROUP_SMEM_MATS;
     if (local) {
@@ -213,10 +222,17 @@ __global__ void __launch_bounds__(256) k_hist(BatchArgs a) {
         atomicOr(&a.ctl->err, ERR_BAD_MAT);
     }
     // the block that finishes last lays out the materials' segments
-    if (last_block(&a.ctl->hist_done)) scan_materials(a);
+    if (a.n_mats <= SCAN_IN_HIST && last_block(&a.ctl->hist_done)) scan_materials<4, true, true>(a);
 }
 
-// One block: exclusive scans of counts, counts * roots and ceil(counts / 32).
+__global__ void __launch_bounds__(1024) k_scan_materials(BatchArgs a) {
+    if (blockIdx.x == 0) scan_materials<8, true, false>(a);
+    else scan_materials<8, false, true>(a);
+}
+
+// One block: exclusive scans of counts and counts * roots (SEGMENTS), and of ceil(counts / 32) by rank
+// (ITEMS).  A thread's reads of U materials go out together: one block has few warps to hide them behind.
+template <uint32_t U, bool SEGMENTS, bool ITEMS>
 __device__ __forceinline__ void scan_materials(const BatchArgs& a) {
     __shared__ uint32_t s_tmp[33];
     const uint32_t T = blockDim.x, t = threadIdx.x;
@@ -225,51 +241,83 @@ __device__ __forceinline__ void scan_materials(const BatchArgs& a) {
     // probes are laid out for every cacheable node (surrogate ones get their record from
     // the surrogate instead of a lookup)
     const bool surr = a.surr_slot != nullptr;
-    uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
-#pragma unroll 4
-    for (uint32_t m = lo; m < hi; ++m) {
-        uint32_t c = __ldcg(&a.counts[m]);
-        uint32_t k = (a.use_cache || surr) ? a.mats[m].n_roots : 0u;
-        c0 += c;
-        c1 += c * k;
-        c2 += (__ldcg(&a.counts[a.mat_order[m]]) + 31u) >> 5;   // items are laid out by rank
-        c3 += (surr && a.surr_slot[m] >= 0) ? (c + 127u) >> 7 : 0u;
+    uint32_t c[U], k[U], x[U], r[U];   // points, probes, surrogate items; work items of the material of this rank
+    auto load = [&](uint32_t m0) {
+#pragma unroll
+        for (uint32_t j = 0; j < U; ++j) {
+            const uint32_t m = m0 + j;
+            const bool in = m < hi;
+            if (SEGMENTS) {
+                c[j] = in ? __ldcg(&a.counts[m]) : 0u;
+                k[j] = in && (a.use_cache || surr) ? c[j] * __ldg(&a.mats[m].n_roots) : 0u;
+                x[j] = in && surr && __ldg(&a.surr_slot[m]) >= 0 ? (c[j] + 127u) >> 7 : 0u;
+            }
+            if (ITEMS) r[j] = in ? (__ldcg(&a.counts[__ldg(&a.mat_order[m])]) + 31u) >> 5 : 0u;
+        }
+    };
+    uint32_t s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+    for (uint32_t m = lo; m < hi; m += U) {
+        load(m);
+#pragma unroll
+        for (uint32_t j = 0; j < U; ++j) {
+            if (SEGMENTS) {
+                s0 += c[j];
+                s1 += k[j];
+                s2 += x[j];
+            }
+            if (ITEMS) s3 += r[j];
+        }
     }
-    uint32_t tot0, tot1, tot2, tot3;
-    uint32_t b0 = block_incl_scan(c0, s_tmp, &tot0) - c0;
-    uint32_t b1 = block_incl_scan(c1, s_tmp, &tot1) - c1;
-    uint32_t b2 = block_incl_scan(c2, s_tmp, &tot2) - c2;
-    uint32_t b3 = block_incl_scan(c3, s_tmp, &tot3) - c3;
-#pragma unroll 4
-    for (uint32_t m = lo; m < hi; ++m) {
-        uint32_t c = __ldcg(&a.counts[m]);
-        uint32_t k = (a.use_cache || surr) ? a.mats[m].n_roots : 0u;
-        a.seg_start[m] = b0;
-        a.cursor[m] = b0;
-        a.probe_base[m] = b1;
-        a.item_base[m] = b2;
-        if (surr) a.surr_item_base[m] = b3;
-        b0 += c;
-        b1 += c * k;
-        b2 += (__ldcg(&a.counts[a.mat_order[m]]) + 31u) >> 5;
-        b3 += (surr && a.surr_slot[m] >= 0) ? (c + 127u) >> 7 : 0u;
+    uint32_t tot0 = 0, tot1 = 0, tot2 = 0, tot3 = 0, b0 = 0, b1 = 0, b2 = 0, b3 = 0;
+    if (SEGMENTS) {
+        b0 = block_incl_scan(s0, s_tmp, &tot0) - s0;
+        b1 = block_incl_scan(s1, s_tmp, &tot1) - s1;
+        b2 = block_incl_scan(s2, s_tmp, &tot2) - s2;
+    }
+    if (ITEMS) b3 = block_incl_scan(s3, s_tmp, &tot3) - s3;
+    for (uint32_t m0 = lo; m0 < hi; m0 += U) {
+        load(m0);
+#pragma unroll
+        for (uint32_t j = 0; j < U; ++j) {
+            const uint32_t m = m0 + j;
+            if (m >= hi) break;
+            if (SEGMENTS) {
+                a.seg_start[m] = b0;
+                a.cursor[m] = b0;
+                a.probe_base[m] = b1;
+                if (surr) a.surr_item_base[m] = b2;
+                b0 += c[j];
+                b1 += k[j];
+                b2 += x[j];
+            }
+            if (ITEMS) {
+                a.item_base[m] = b3;
+                b3 += r[j];
+            }
+        }
     }
     if (t == T - 1) {
-        a.seg_start[a.n_mats] = tot0;
-        a.probe_base[a.n_mats] = tot1;
-        a.item_base[a.n_mats] = tot2;
-        if (surr) a.surr_item_base[a.n_mats] = tot3;
-        a.ctl->n_surr_items = surr ? tot3 : 0u;
-        a.ctl->n_items = tot2;
-        a.ctl->total_probes = tot1;
-        if (tot1 > a.probe_cap) {
-            // more probe records than the scratch holds: the batch does no work and the
-            // next synchronising call reports it
-            a.ctl->n_items = 0;
-            a.ctl->n_surr_items = 0;
-            atomicOr(&a.ctl->err, ERR_CAPACITY);
+        if (SEGMENTS) {
+            a.seg_start[a.n_mats] = tot0;
+            a.probe_base[a.n_mats] = tot1;
+            if (surr) a.surr_item_base[a.n_mats] = tot2;
+            a.ctl->n_surr_items = tot2;
+            a.ctl->total_probes = tot1;
+            atomicAdd(&a.stats[ST_POINTS], (unsigned long long)a.n);
         }
-        atomicAdd(&a.stats[ST_POINTS], (unsigned long long)a.n);
+        if (ITEMS) {
+            a.item_base[a.n_mats] = tot3;
+            a.ctl->n_items = tot3;
+        }
+    }
+    // the block that holds both totals last
+    if (!(SEGMENTS && ITEMS) && !last_block(&a.ctl->hist_done)) return;
+    if (t == T - 1 && (SEGMENTS && ITEMS ? tot1 : __ldcg(&a.ctl->total_probes)) > a.probe_cap) {
+        // more probe records than the scratch holds: the batch does no work and the
+        // next synchronising call reports it
+        a.ctl->n_items = 0;
+        a.ctl->n_surr_items = 0;
+        atomicOr(&a.ctl->err, ERR_CAPACITY);
     }
 }
 
@@ -420,7 +468,7 @@ __global__ void __cluster_dims__(GROUP_CLUSTER, 1, 1) __launch_bounds__(GROUP_CL
         start += tot[k];
     }
     __syncthreads();
-    if (rank == 0) scan_materials(a);   // reads the counts this block wrote
+    if (rank == 0) scan_materials<GROUP_CLUSTER_MATS / GROUP_CLUSTER_T, true, true>(a);   // reads the counts this block wrote
     for (uint32_t i = lo + t; i < hi32 && lo < hi; i += GROUP_CLUSTER_T) scatter_point(a, i, hi, s_pos);
     cluster.sync();   // no block leaves while another may read its counts
 }
@@ -3142,6 +3190,10 @@ static void launch_group(const BatchArgs& a, cudaStream_t s, int num_sms, uint64
     if (a.unsorted) return;
     k_hist<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
     *nl += 1;
+    if (a.n_mats > SCAN_IN_HIST) {
+        k_scan_materials<<<2, 1024, 0, s>>>(a);
+        *nl += 1;
+    }
     if (a.n == 0) return;
     k_scatter<<<group_blocks(a.n, num_sms), 256, 0, s>>>(a);
     *nl += 1;
