@@ -113,10 +113,11 @@ inline bool insert_lists(const pmc_cache* c) {
            !(c->desc.flags & (PMC_INSERT_ROUNDS | PMC_ALG1 | PMC_REPLACE_VISIBILITY)) && !c->insert_binned;
 }
 
-// The bins of the cell-grouped insert for the batch in *a (n and probe_cap set).
+// The bins of the cell-grouped insert for the batch in *a (n and probe_cap set), its points spread evenly
+// over the materials.
 inline void set_bins(const pmc_cache* c, pmc::BatchArgs* a) {
     const uint64_t cells = c->use_cache ? c->desc.n_cells : 0;
-    const uint64_t probes = std::min<uint64_t>((uint64_t)a->n * c->max_roots, a->probe_cap);
+    const uint64_t probes = std::min<uint64_t>((uint64_t)a->n * c->root_info.size() / std::max(c->n_mats, 1u), a->probe_cap);
     a->bin_shift = pmc::insert_bin_shift(cells, probes);
     a->n_bins = pmc::insert_bins(cells, a->bin_shift);
     a->bin_cnt = c->d_bins;

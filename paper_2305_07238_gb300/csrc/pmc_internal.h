@@ -294,19 +294,28 @@ constexpr uint32_t INSERT_BIN_SHIFT = 8;
 constexpr uint32_t INSERT_BIN_CELLS = 1u << INSERT_BIN_SHIFT;   // most cells per bin
 constexpr uint32_t INSERT_SMALL_BINS = 8192;                    // most bins of fewer cells
 
-// Bins of the cell-grouped insert for a batch that can offer up to `probes` candidates.  A bin
-// is resolved fastest by a block that stages all of its candidates at once (up to 2048); larger
-// ones are re-read for every range of cells that fits.  So bins shrink below 256 cells while
-// a bin could get more than 1024 on average and their number stays within what one block
-// scans quickly and the partition counts in shared memory.  (403 k points x 6.3 cacheable nodes
-// on 65,536 cells: 256 bins of 256 cells take 412 us per pass, 4096 bins of 16 cells 131 us.)
-inline uint32_t insert_bin_shift(uint64_t n_cells, uint64_t probes) {
-    uint32_t s = INSERT_BIN_SHIFT;
-    while (s > 0 && (n_cells >> (s - 1)) < INSERT_SMALL_BINS && probes >> 10 > (n_cells >> s)) --s;
-    return s;
-}
 inline uint32_t insert_bins(uint64_t n_cells, uint32_t shift) {
     return (uint32_t)((n_cells + (1ull << shift) - 1) >> shift);
+}
+// log2 of the cells per bin of the cell-grouped insert for a batch expected to offer up to `probes`
+// candidates (on an empty table; later passes offer fewer).  A bin is resolved fastest by a block
+// that stages all of its candidates at once (up to 2048); larger ones are re-read for every range of
+// cells that fits.  So bins shrink below 256 cells while one could get more than 1536 on average and
+// their number stays within what one block scans quickly and the partition counts in shared
+// memory; not further, since every bin costs its block or warp a chain of dependent steps.  Insert
+// phase of a pass with three visibility classes, us, by cells per bin (points x cacheable nodes, cells):
+//   403 k x 7.3, 65,536      256: 429   64: 235   32: 112*  16: 132
+//   403 k x 2.7, 65,536      256: 142  128: 121   64: 84*   32: 88   16: 107
+//   207 k x 2.7, 131,072     256: 84*  128: 99    64: 98
+//   99 k x 2.7, 50,021       256: 71*  128: 77    64: 82    32: 65
+//   1.05 M x 1.7, 524,288    256: 162* 128: 187   64: 180
+//   35 k x 7.3, 1,024        256: 3831   8: 177    4: 69*    2: 66    1: 96
+// (*: chosen here.  With a limit of 1024 and the network of most cacheable nodes in the place of
+// the mean, these were 132, 107, 99, 65, 187 and 96.)
+inline uint32_t insert_bin_shift(uint64_t n_cells, uint64_t probes) {
+    uint32_t s = INSERT_BIN_SHIFT;
+    while (s > 0 && (n_cells >> (s - 1)) < INSERT_SMALL_BINS && probes > 1536ull * insert_bins(n_cells, s)) --s;
+    return s;
 }
 // Bins to reserve room for, whatever the batch.
 inline uint32_t insert_bins_max(uint64_t n_cells) {
