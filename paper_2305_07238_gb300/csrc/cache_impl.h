@@ -50,6 +50,7 @@ struct pmc_cache {
     uint32_t* d_root_order = nullptr;     // roots by ascending level, then MAX_LEVELS + 1 starts
     uint32_t* d_mat_order = nullptr;      // materials by descending cost: whole programs, outer programs
     double uneven[3] = {1.0, 1.0, 1.0};   // cost of the longest program over the mean: whole, outer, cacheable nodes
+    double mean_cost[2] = {0.0, 0.0};     // mean cost of a program: whole, outer
     bool table_empty = true;              // nothing inserted since creation or reset
     bool last_all_miss = false;           // the last batch ran on an empty table
     bool last_unsorted = false;           // the last batch kept no probe records
@@ -129,20 +130,36 @@ inline void set_bins(const pmc_cache* c, pmc::BatchArgs* a) {
 inline uint64_t program_cost(uint64_t nodes, uint64_t flops) { return 30 * nodes + flops * 8 / 5; }
 
 // The order of the materials' work items in the batch in *a, by the programs its points run, and
-// whether its evaluators take one point per lane.  Two points share an instruction's fetch and
+// whether its per-point evaluator takes one point per lane.  Two points share an instruction's fetch and
 // decode, but an item takes twice as long, and a batch cannot end before its longest one: with few
 // items, or with programs of very uneven length, one point per lane spreads the work over
-// more warps.  The line: 60 items per SM x (longest / mean program - 1/2).  Evaluation of a first
-// pass, two points against one, us:
-//   64 networks of 20-200 nodes (longest / mean 2.3): 230 k points 170 / 160, 518 k 278 / 227, 1.04 M 384 / 421
+// more warps.  The line: 60 items per SM x (longest / mean program - 0.4), and less in proportion for
+// programs so short that what is done once per item (claiming it, its points, a first pass's
+// offers) outweighs them: below a mean of 1,500 instructions for whole programs, 4,000 with offers, 1,000
+// for outer programs.  Evaluation of a pass, two points against one, us (longest / mean, mean):
+//   first pass:
+//   one network of 8 nodes (1, 473): 30 k points 17.6 / 16.1, 65 k 20.0 / 22.0, 115 k 25 / 32, 230 k 33 / 40
+//   one of 12 (1, 1596): 30 k 20.8 / 19.1, 65 k 24.2 / 24.6, 115 k 29 / 31
+//   one of 60 (1, 8363): 115 k 97 / 76, 147 k 98 / 85, 184 k 100 / 118
+//   16 of 9-21 (1.65, 1388): 65 k 40 / 30, 115 k 42 / 33, 184 k 44.2 / 43.4, 230 k 45 / 49
+//   64 of 20-200 (2.5): 230 k 170 / 160, 518 k 278 / 227, 1.04 M 384 / 421
 //   512 of 5-400 (4.4): 518 k 556 / 286, 1.04 M 561 / 391, 2.07 M 658 / 759
 //   1024 of 5-2000 (6): 518 k 2634 / 1626, 1.04 M 3182 / 2666, 2.07 M 4650 / 4976
-//   one network of 8 nodes: 115 k 25 / 29, 230 k 33 / 41
+//   without the cache:
+//   one of 8 (1, 473): 16 k 10.2 / 10.1, 115 k 13.4 / 15.3, 147 k 14.6 / 17.4
+//   one of 12 (1, 1596): 115 k 22 / 19, 147 k 23.6 / 22.2, 184 k 23.9 / 24.7
+//   one of 60 (1, 8363): 147 k 77 / 58, 184 k 78 / 70, 230 k 78 / 81
+//   outer programs:
+//   one of 24 (1, 567): 65 k 12.3 / 12.3, 115 k 14.3 / 16.4
+//   one of 60 (1, 2307): 131 k 33 / 25, 184 k 33 / 33
+//   64 of 20-200 (2.9, 2296): 131 k 72 / 43, 400 k 76 / 57
 inline void set_order(const pmc_cache* c, pmc::BatchArgs* a) {
     const bool outer = a->use_cache && a->split && !a->keys_inline && !a->unsorted && !a->probe_inline && !a->alg1;
     a->mat_order = c->d_mat_order + (outer ? c->n_mats : 0);
     const double items = (double)a->n / 32.0 + c->n_mats;
-    if (!a->block_items && items < 60.0 * c->num_sms * (c->uneven[outer] - 0.5)) a->one_point = 1;
-    // the batched misses likewise, by the items of a level, which the device counts
+    const double shortest = outer ? 1000.0 : a->use_cache ? 4000.0 : 1500.0;
+    const double line = 60.0 * c->num_sms * (c->uneven[outer] - 0.4) * std::min(1.0, c->mean_cost[outer] / shortest);
+    if (!a->block_items && items < line) a->one_point = 1;
+    // the batched misses by a line of their own, against the items of a level, which the device counts
     a->root_pairs_min = (uint32_t)std::min(4e9, 60.0 * c->num_sms * (c->uneven[2] - 0.5));
 }

@@ -405,7 +405,10 @@ pmc_status pmc_create_cache(const pmc_cache_desc* desc, const pmc_material* mats
                 top[o] = std::max(top[o], k[o]);
             }
         }
-        for (int o = 0; o < 2; ++o) c->uneven[o] = sum[o] > 0.0 ? top[o] * n_mats / sum[o] : 1.0;
+        for (int o = 0; o < 2; ++o) {
+            c->uneven[o] = sum[o] > 0.0 ? top[o] * n_mats / sum[o] : 1.0;
+            c->mean_cost[o] = sum[o] / n_mats;
+        }
         if (e == cudaSuccess)
             e = cudaMemcpy(c->d_mat_order, order.data(), order.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
     }
@@ -544,7 +547,7 @@ pmc_status enqueue_batch(pmc_cache* c, const pmc_points* pts, float* out_rgb, ui
     a.probe_inline = c->probe_inline;
     a.lookup_rb = c->lookup_rb;
     a.block_items = c->block_items;
-    a.one_point = c->one_point;
+    a.one_point = a.roots_one_point = c->one_point;
     set_order(c, &a);
     if (replacing(c)) {
         a.slot_cls = c->d_cls;

@@ -3314,7 +3314,7 @@ cudaError_t launch_batch(const BatchArgs& a, cudaStream_t s, int num_sms, cudaEv
             return e;
         // the batched misses: two misses per lane up to a smaller slot file, and in the kernel only
         // where a level has enough items (the item counter then counts pairs)
-        const bool two_roots = !a.one_point && 2 * smem_roots <= ROOTS2_MAX_SMEM;
+        const bool two_roots = !a.roots_one_point && 2 * smem_roots <= ROOTS2_MAX_SMEM;
         auto kroots = two_roots ? k_eval_roots2 : k_eval_roots;
         const size_t smem_kroots = two_roots ? 2 * smem_roots : smem_roots;
         if (smem_kroots > 48 * 1024 &&

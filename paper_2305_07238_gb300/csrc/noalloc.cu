@@ -170,7 +170,7 @@ extern "C" pmc_status pmc_eval_batch_noalloc(pmc_cache* c, const pmc_points* pts
     a.probe_inline = c->probe_inline;
     a.lookup_rb = c->lookup_rb;
     a.block_items = c->block_items;
-    a.one_point = c->one_point;
+    a.one_point = a.roots_one_point = c->one_point;
     set_order(c, &a);
     if (c->use_cache && (c->desc.flags & PMC_REPLACE_VISIBILITY)) {
         a.slot_cls = c->d_cls;

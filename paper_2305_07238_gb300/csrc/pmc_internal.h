@@ -281,6 +281,7 @@ struct BatchArgs {
     uint32_t lookup_rb;        // k_lookup: probes in flight per lane (1, 2 or 4)
     int block_items;           // 1: the per-point evaluator claims block-wide tiles of items
     int one_point;             // 1: one point per lane in the per-point evaluator (else two)
+    int roots_one_point;       // 1: one miss per lane in the batched evaluation of misses (else by root_pairs_min)
     uint32_t root_pairs_min;   // batched misses: work items of a level from which two misses run per lane
     int alg1;                  // the paper's concurrent update: 8-byte slots {hash2, RGB9E5},
                                // looked up and inserted inside the evaluator (one 64-bit CAS)
