@@ -1050,8 +1050,15 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     DeviceGuard g(c->desc.device);
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t L = (uint32_t)train.size();
-    const uint32_t s0 = c->n_surr_slots;
-    pmc_status st = grow_surrogate_slots(c, s0 + L);
+    // slots: a material keeps the one it has, so that training again takes no more memory
+    std::vector<int32_t> slot = c->surr_slot;
+    uint32_t n_slots = c->n_surr_slots;
+    bool again = false;
+    for (uint32_t m : train) {
+        again |= c->surr_slot[m] >= 0;
+        if (slot[m] < 0) slot[m] = (int32_t)n_slots++;
+    }
+    pmc_status st = grow_surrogate_slots(c, n_slots);
     if (st != PMC_OK) return st;
     // The first epoch reads its pairs in a known order, so training starts when the first of up to
     // PARTS parts of them (at least 32 steps each) is drawn and runs beside the drawing of the next, and of
@@ -1062,10 +1069,11 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     const uint32_t steps_per_epoch = d->n_train / 128u, nv = d->n_valid;
     uint32_t n_parts = 1;
     while (n_parts < PARTS && steps_per_epoch / (2 * n_parts) >= 32u) n_parts *= 2;
-    // temporaries: initial weights, Adam moments, pairs, losses
+    // temporaries: initial weights, the weights in training (passes under way on other streams
+    // may read the slots meanwhile), Adam moments, pairs, losses
     const size_t n_theta = (size_t)L * MLP_PARAMS;
     std::vector<float> th(n_theta);
-    float *m1 = nullptr, *m2 = nullptr, *data = nullptr, *vdata = nullptr, *loss = nullptr;
+    float *theta = nullptr, *m1 = nullptr, *m2 = nullptr, *data = nullptr, *vdata = nullptr, *loss = nullptr;
     uint32_t* groots = nullptr;            // cacheable nodes, networks by cost, work counters
     cudaStream_t ts = s;                   // training's stream
     cudaEvent_t ev[PARTS + 1] = {};
@@ -1076,9 +1084,9 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
         }
         for (cudaEvent_t x : ev)
             if (x) cudaEventDestroy(x);
-        dfree(&m1); dfree(&m2); dfree(&data); dfree(&vdata); dfree(&loss); dfree(&groots);
+        dfree(&theta); dfree(&m1); dfree(&m2); dfree(&data); dfree(&vdata); dfree(&loss); dfree(&groots);
     };
-    if ((st = dalloc(&m1, n_theta)) != PMC_OK || (st = dalloc(&m2, n_theta)) != PMC_OK ||
+    if ((st = dalloc(&theta, n_theta)) != PMC_OK || (st = dalloc(&m1, n_theta)) != PMC_OK || (st = dalloc(&m2, n_theta)) != PMC_OK ||
         (st = dalloc(&data, (size_t)L * std::max(d->n_train, nv) * 5)) != PMC_OK || (st = dalloc(&loss, L)) != PMC_OK ||
         (st = dalloc(&groots, 2 * (size_t)L + PARTS + 1)) != PMC_OK) {
         release();
@@ -1117,7 +1125,6 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     }
     if (e == cudaSuccess && vdata) e = draw(PARTS, 0, nv, true);
     for (uint32_t i = 0; i < L; ++i) init_theta(d->seed * 0x100000001B3ull + train[i] + 1, th.data() + (size_t)i * MLP_PARAMS);
-    float* theta = c->d_surr_theta + (size_t)s0 * MLP_PARAMS;
     if (e == cudaSuccess) e = cudaMemcpyAsync(theta, th.data(), n_theta * sizeof(float), cudaMemcpyHostToDevice, ts);
     if (e == cudaSuccess) e = cudaMemsetAsync(m1, 0, n_theta * sizeof(float), ts);
     if (e == cudaSuccess) e = cudaMemsetAsync(m2, 0, n_theta * sizeof(float), ts);
@@ -1150,12 +1157,20 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(sums.data(), d_sum, sums.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    // the trained weights into their slots, consecutive ones in one copy; slots in use only once
+    // no pass on any stream reads them
+    if (e == cudaSuccess && again) e = cudaDeviceSynchronize();
+    for (uint32_t i = 0, k; e == cudaSuccess && i < L; i = k) {
+        for (k = i + 1; k < L && slot[train[k]] == slot[train[k - 1]] + 1;) ++k;
+        e = cudaMemcpyAsync(c->d_surr_theta + (size_t)slot[train[i]] * MLP_PARAMS, theta + (size_t)i * MLP_PARAMS,
+                            (size_t)(k - i) * MLP_PARAMS * sizeof(float), cudaMemcpyDeviceToDevice, 0);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     for (uint32_t i = 0; e == cudaSuccess && i < L; ++i) {
         double se = 0.0;
         for (uint32_t p = 0; p < parts; ++p) se += sums[(size_t)i * parts + p];
         const float err = (float)std::sqrt(se / (3.0 * nv));
         const uint32_t m = train[i];
-        c->surr_slot[m] = (int32_t)(s0 + i);
         // enabled at a margin under the accuracy bar of 2e-3, so that held-out points stay
         // within the bar (the validation set is a sample)
         c->surr_on[m] = err <= (d->rmse_max > 0.0f ? d->rmse_max : 1.6e-3f);
@@ -1166,7 +1181,8 @@ pmc_status pmc_train_surrogates(pmc_cache* c, const pmc_train_desc* d, float* rm
     dfree(&d_sum);
     release();
     if (e != cudaSuccess) return cuda_fail(c, e);
-    c->n_surr_slots = s0 + L;
+    c->surr_slot = slot;
+    c->n_surr_slots = n_slots;
     e = upload_surrogate_maps(c);
     if (e != cudaSuccess) return cuda_fail(c, e);
     return PMC_OK;
