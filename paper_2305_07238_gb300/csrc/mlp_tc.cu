@@ -60,6 +60,9 @@ struct Sm {                                     // byte offsets into dynamic sha
 static_assert(Sm::bias + 132 * 4 - Sm::w1 == SURR_IMG_BYTES, "operand image = weights and biases of Sm");
 static_assert(Sm::w1 % 16 == 0, "bulk copies land on 16-byte boundaries");
 static_assert(Sm::end <= TC_SMEM, "inference shared memory");
+// A block may ask for this much without the attribute of a kernel being set first, which a short call of
+// the stand-alone network would pay for each time (host time of a call 2.76 us with it, 2.43 without).
+static_assert(TC_SMEM + 1024 <= 48 * 1024, "inference shared memory without opting in");
 static_assert(TC_CTAS_PER_SM * (TC_SMEM + 1024) <= 228 * 1024 && (TC_CTAS_PER_SM + 1) * (TC_SMEM + 1024) > 228 * 1024,
               "exactly TC_CTAS_PER_SM inference CTAs fit an SM's shared memory");
 static_assert(TC_CTAS_PER_SM * (TC_COLS + TC_ACOLS) <= 512, "inference CTAs per SM by tensor memory");
@@ -1057,16 +1060,12 @@ uint32_t mlp_validate_parts(uint32_t n_nets, uint32_t n, int num_sms) {
 
 cudaError_t launch_mlp_validate(const float* theta, const float* data, uint32_t n_nets, uint32_t n, double* sum,
                                 uint32_t* err, int num_sms, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_validate_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
-    if (e != cudaSuccess) return e;
     k_mlp_validate_tc<<<dim3(mlp_validate_parts(n_nets, n, num_sms), n_nets), TC_ROWS, TC_SMEM, s>>>(theta, data, n, sum,
                                                                                                  err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_surrogate(const BatchArgs& a, int num_sms, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_surrogate_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
-    if (e != cudaSuccess) return e;
     k_surrogate_tc<<<num_sms * TC_CTAS_PER_SM, TC_ROWS, TC_SMEM, s>>>(a);
     return cudaGetLastError();
 }
@@ -1083,8 +1082,6 @@ cudaError_t launch_mlp_forward_tc(const float* theta, const float* u, const floa
     const uint32_t full = (uint32_t)num_sms * TC_CTAS_PER_SM;
     uint32_t blocks = tiles < full ? tiles : full;
     if (blocks == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
-    if (e != cudaSuccess) return e;
     k_mlp_forward_tc<<<blocks, TC_ROWS, TC_SMEM, s>>>(theta, u, v, n, out, clamp, err);
     return cudaGetLastError();
 }
