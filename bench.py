@@ -50,7 +50,7 @@ REF_MIN_ROOT_COST = MIN_ROOT_COST   # reference arm: the same threshold
 # DRAM bytes (read + written) per launch of each kernel, the mean of the two launches one
 # ncu capture of that kernel takes from a four-pass frame of this workload at the bench's
 # cost threshold; None while the kernel has changed since its capture
-NCU_TRAFFIC = {"eval": 159.2e6, "eval_roots": 98.9e6, "lookup": 372.3e6}
+NCU_TRAFFIC = {"eval": 159.3e6, "eval_roots": 99.6e6, "lookup": 372.5e6}
 
 FP32_LANES_PER_SM = 128          # Blackwell SM: 4 partitions x 32 FP32 lanes
 

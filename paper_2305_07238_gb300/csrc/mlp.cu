@@ -36,7 +36,8 @@ __device__ __forceinline__ void store_pair(float* d, const PointIn& pt, float x,
 // Training pairs of the exact evaluator: the generator's points and the values of the cacheable
 // node's standalone program at them.  Rows (k * mult) mod mask + 1 for k in [k0, k0 + count): a training
 // epoch reads its rows in that order, so a part of the pairs is enough for the steps that come
-// first.  Bound by instruction issue, as every evaluation: TWO points per lane share an instruction's
+// first.  Bound by instruction issue (68 % of the slots over a launch of 4,096 items, whose end runs with
+// few warps): TWO points per lane share an instruction's
 // fetch and decode, and the next instruction is fetched while one runs.  A warp claims 32 or 64 rows
 // of one network at a time, the networks of the longest programs (descending cost) first.
 // (64 networks of 500-2000 nodes, 73,728 pairs each: one point per lane, in the networks' order 17.2 ms,
